@@ -126,6 +126,11 @@ def _lattice(wl):
     return np.eye(3) * float(wl["a"])
 
 
+def _lattice_and_inverse(wl, dev):
+    L = _lattice(wl)
+    return torch.tensor(L, device=dev), torch.tensor(np.linalg.inv(L), device=dev)
+
+
 def _wavevector(wl):
     """(1/4, 1/4, 1/4) in the reciprocal lattice."""
     return 2.0 * math.pi * np.linalg.solve(_lattice(wl), np.full(3, 0.25))
@@ -177,8 +182,7 @@ def _states(wl, n_dof, nocc, seed, dev, k=None):
 def _potential(wl, x, seed):
     """The local potential -Z erf(r / sigma) / r of the nearest image of every
     atom, with a smooth modulation drawn from the seed."""
-    L = torch.tensor(_lattice(wl), device=x.device)
-    inv = torch.linalg.inv(L)
+    L, inv = _lattice_and_inverse(wl, x.device)
     V = torch.zeros(len(x), dtype=F64, device=x.device)
     for s, tau in wl["atoms"]:
         sp = wl["species"][s]
@@ -413,8 +417,8 @@ def _images(wl, reach, dev):
 def _orbital(wl, orb, rc, d):
     """Psi and grad Psi of one orbital at displacements d (..., 3) from its atom."""
     n, l, m, zeta = orb
-    L = torch.tensor(_lattice(wl), device=d.device)
-    d = d - torch.round(d @ torch.linalg.inv(L)) @ L
+    L, inv = _lattice_and_inverse(wl, d.device)
+    d = d - torch.round(d @ inv) @ L
     norm = (2.0 * zeta) ** (n + 0.5) / math.sqrt(math.factorial(2 * n))
     out = [torch.zeros_like(d[..., 0]) for _ in range(4)]
     for R in _images(wl, rc, d.device):
@@ -500,7 +504,7 @@ class _Exact:
         self.dofs = torch.tensor(dofs, device=self.dev).long()
         self.doff = torch.cumsum(self.n_e, 0) - self.n_e
         wl, nel = self.wl, int(self.wl["nel"])
-        self.L, self.nel = torch.tensor(_lattice(wl), device=self.dev), nel
+        (self.L, self.inv), self.nel = _lattice_and_inverse(wl, self.dev), nel
         self.ser = wl.get("fe") == "serendipity32"
         # enrichment DOFs: by atom, orbital, vertex within r_e of the atom
         g = torch.arange(nel ** 3, device=self.dev)
@@ -509,7 +513,7 @@ class _Exact:
         for ia, (sp, tau) in enumerate(wl["atoms"]):
             sp = wl["species"][sp]
             d = (frac @ self.L) - torch.tensor(tau, dtype=F64, device=self.dev)
-            d = d - torch.round(d @ torch.linalg.inv(self.L)) @ self.L
+            d = d - torch.round(d @ self.inv) @ self.L
             r = torch.linalg.norm(d[:, None, :] + _images(wl, 2 * sp["r_e"], self.dev), dim=2)
             v = torch.nonzero(r.min(dim=1).values <= sp["r_e"] + 1e-12)[:, 0]
             for o in sp["orbitals"]:
@@ -540,7 +544,7 @@ class _Exact:
         qi = self.off[el][:, None] + torch.arange(Q, device=self.dev)
         col = self.dofs[self.doff[el][:, None] + torch.arange(n, device=self.dev)]
         x, ec = self.x[qi], torch.stack([el % nel, (el // nel) % nel, el // nel ** 2], 1)
-        Jinv = torch.linalg.inv(self.L) * 2.0 * nel     # d xi / d x
+        Jinv = self.inv * 2.0 * nel     # d xi / d x
         xi = (x - (ec.double() / nel @ self.L)[:, None, :]) @ Jinv - 1.0
         B, G = _fe_columns(xi, self.ser)
         loc = torch.arange(64, device=self.dev)
@@ -637,7 +641,7 @@ class _Exact:
             l, rp = q["l"], q["rp"]
             nrm = math.sqrt(2.0 / (math.gamma(l + 1.5) * rp ** (2 * l + 3)))
             d0 = self.x - torch.tensor(q["tau"], dtype=F64, device=self.dev)
-            lat = torch.round(d0 @ torch.linalg.inv(self.L)) @ self.L
+            lat = torch.round(d0 @ self.inv) @ self.L
             for R in _images(wl, 9.6 * rp, self.dev):
                 d = d0 - lat + R
                 v = nrm * torch.exp(-(d * d).sum(1) / (2.0 * rp * rp)) * _solid(l, q["m"], d)[0]
