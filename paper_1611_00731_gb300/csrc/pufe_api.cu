@@ -81,10 +81,7 @@ pufe_status pufe_assemble_HS(pufe_ctx *ctx, const double *V, int prec, int what,
   if (!g.ok) return fail(PUFE_ECUDA, "cudaSetDevice failed");
   cudaStream_t st = (cudaStream_t)stream;
   if (prec == PUFE_TF32X3) return launch_assemble_tc(ctx, V, what, H, S, st);
-  const size_t bytes = (size_t)ctx->nnz * sizeof(double);
-  if (what & PUFE_WANT_H) PUFE_CUDA_TRY(cudaMemsetAsync(H, 0, bytes, st));
-  if (what & PUFE_WANT_S) PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
-  return launch_assemble_fp64(ctx, V, what, H, S, st);
+  return launch_assemble_fp64(ctx, nullptr, V, what, H, nullptr, S, nullptr, st);
 }
 
 pufe_status pufe_assemble_HS_static(pufe_ctx *ctx, const double *V, int what, double *H,
@@ -142,16 +139,8 @@ pufe_status pufe_assemble_HS_bloch(pufe_ctx *ctx, const double *k, const double 
   if (prec == PUFE_TF32X3)
     return launch_assemble_mixed_bloch(ctx, phase_table(ctx, k), V, what, H_re, H_im, S_re, S_im,
                                        st);
-  const size_t bytes = (size_t)ctx->nnz * sizeof(double);
-  if (what & PUFE_WANT_H) {
-    PUFE_CUDA_TRY(cudaMemsetAsync(H_re, 0, bytes, st));
-    PUFE_CUDA_TRY(cudaMemsetAsync(H_im, 0, bytes, st));
-  }
-  if (what & PUFE_WANT_S) {
-    PUFE_CUDA_TRY(cudaMemsetAsync(S_re, 0, bytes, st));
-    PUFE_CUDA_TRY(cudaMemsetAsync(S_im, 0, bytes, st));
-  }
-  return launch_assemble_fp64_bloch(ctx, phase_table(ctx, k), V, what, H_re, H_im, S_re, S_im, st);
+  const PhaseTab ph = phase_table(ctx, k);
+  return launch_assemble_fp64(ctx, &ph, V, what, H_re, H_im, S_re, S_im, st);
 }
 
 pufe_status pufe_density_bloch(pufe_ctx *ctx, const double *k, const double *C_re,

@@ -716,18 +716,38 @@ static unsigned fp64_items(const pufe_ctx *ctx) {
   return ctx->d.wsplit ? (unsigned)ctx->n_wsplit : (unsigned)ctx->nelem;
 }
 
-pufe_status launch_assemble_fp64(pufe_ctx *ctx, const double *V, int what, double *H, double *S,
-                                 cudaStream_t st) {
+// FP64 assembly into caller arrays: H (and Hi, Si at a wavevector, ph != nullptr)
+// zeroed here, S too -- or, on the sum-factorized path at the Gamma point, set
+// to the constant FE-FE overlap that path does not add
+pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
+                                 double *H, double *Hi, double *S, double *Si, cudaStream_t st) {
   auto &D = ctx->d;
   const int npad = (ctx->max_basis + 3) & ~3;
   const size_t sm = (size_t)5 * QC * npad * sizeof(double) + QC * sizeof(Tab1D);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "element basis too large for the FP64 kernel");
-  auto kern = ctx->general ? k_assemble_fp64<false, true> : k_assemble_fp64<false, false>;
+  const size_t bytes = (size_t)ctx->nnz * sizeof(double);
+  if (what & PUFE_WANT_H) {
+    PUFE_CUDA_TRY(cudaMemsetAsync(H, 0, bytes, st));
+    if (ph) PUFE_CUDA_TRY(cudaMemsetAsync(Hi, 0, bytes, st));
+  }
+  if (what & PUFE_WANT_S) {
+    if (ph) {
+      PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
+      PUFE_CUDA_TRY(cudaMemsetAsync(Si, 0, bytes, st));
+    } else if (ctx->n_aitems > 0) {
+      PUFE_CUDA_TRY(cudaMemcpyAsync(S, D.S0, bytes, cudaMemcpyDeviceToDevice, st));
+    } else {
+      PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
+    }
+  }
+  if (ctx->n_aitems > 0) return launch_assemble_sf64(ctx, ph, V, what, H, Hi, S, Si, st);
+  auto kern = ph ? (ctx->general ? k_assemble_fp64<true, true> : k_assemble_fp64<true, false>)
+                 : (ctx->general ? k_assemble_fp64<false, true> : k_assemble_fp64<false, false>);
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   kern<<<fp64_items(ctx), ASM_NT, sm, st>>>(
       D.order, D.qoff, D.w, D.xi, D.doff, D.ecol, D.toff, D.psi, D.soff, D.smap, V,
-      2.0 / ctx->h[0], 2.0 / ctx->h[1], 2.0 / ctx->h[2], npad, what, H, S, D.err, nullptr,
-      PhaseTab{}, nullptr, nullptr, D.wsplit, jit_of(ctx), ctx->nfe_e);
+      2.0 / ctx->h[0], 2.0 / ctx->h[1], 2.0 / ctx->h[2], npad, what, H, S, D.err, D.eshift,
+      ph ? *ph : PhaseTab{}, Hi, Si, D.wsplit, jit_of(ctx), ctx->nfe_e);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
@@ -781,23 +801,6 @@ PhaseTab phase_table(const pufe_ctx *ctx, const double k[3]) {
     t.im[c] = sin(th);
   }
   return t;
-}
-
-pufe_status launch_assemble_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *V,
-                                       int what, double *H, double *Hi, double *S, double *Si,
-                                       cudaStream_t st) {
-  auto &D = ctx->d;
-  const int npad = (ctx->max_basis + 3) & ~3;
-  const size_t sm = (size_t)5 * QC * npad * sizeof(double) + QC * sizeof(Tab1D);
-  if (sm > 227 * 1024) return fail(PUFE_EINVAL, "element basis too large for the FP64 kernel");
-  auto kern = ctx->general ? k_assemble_fp64<true, true> : k_assemble_fp64<true, false>;
-  PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<fp64_items(ctx), ASM_NT, sm, st>>>(
-      D.order, D.qoff, D.w, D.xi, D.doff, D.ecol, D.toff, D.psi, D.soff, D.smap, V,
-      2.0 / ctx->h[0], 2.0 / ctx->h[1], 2.0 / ctx->h[2], npad, what, H, S, D.err, D.eshift, ph,
-      Hi, Si, D.wsplit, jit_of(ctx), ctx->nfe_e);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
 }
 
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,

@@ -101,6 +101,8 @@ struct DeviceArrays {
   // FP64 assembly/adjoint work list, 3 per item (element, first point, end
   // point), largest first; null when every item is a whole element
   int32_t *wsplit = nullptr;
+  // sum-factorized FP64 assembly: (element, kind, begin, end) items
+  int32_t *aitems = nullptr;
   // mixed-path work list of the n_e > 128 elements, 3 per item (index into
   // `order`, first chunk, end chunk; chunks of 8 padded points), largest first
   int32_t *titems = nullptr;
@@ -147,6 +149,8 @@ struct pufe_ctx {
   int n_big = 0;              // elements with n_e > 128 (listed first in `order`)
   int64_t big_pad_end = 0;    // end of the last n_e > 128 element's padded points (0: none)
   int64_t n_wsplit = 0;       // items of the FP64 point-range work list (0: none)
+  int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
+  int asm64_work = 0;         // doubles of its shared work area
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
   int n_gitems32 = 0, n_gitems64 = 0;   // items of the Gram-form lists
@@ -402,8 +406,6 @@ __host__ __device__ inline void enrichment_eval(const Orbital &o, const double p
 
 // launchers implemented in the .cu files
 pufe_status launch_tabulate(pufe_ctx *ctx, cudaStream_t s);
-pufe_status launch_assemble_fp64(pufe_ctx *ctx, const double *V, int what, double *H, double *S,
-                                 cudaStream_t s);
 pufe_status launch_density_fp64(pufe_ctx *ctx, const double *C, int64_t ldc, const double *f,
                                 int nocc, double *rho, cudaStream_t s);
 pufe_status launch_adjoint_fp64(pufe_ctx *ctx, const double *Hbar, double *Vbar, cudaStream_t s);
@@ -439,9 +441,13 @@ __host__ __device__ inline double cot_entry(double hr, double hi, int ci, int cj
   const double pim = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
   return hr * pr + hi * pim;
 }
-pufe_status launch_assemble_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *V,
-                                       int what, double *H, double *Hi, double *S, double *Si,
-                                       cudaStream_t s);
+// FP64 assembly (outputs initialised here); ph != nullptr: at a wavevector
+pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
+                                 double *H, double *Hi, double *S, double *Si, cudaStream_t s);
+// its sum-factorized form, and the work list of that form
+pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
+                                 double *H, double *Hi, double *S, double *Si, cudaStream_t s);
+void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, int &work);
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,
                                       const double *Ci, int64_t ldc, const double *f, int nocc,
                                       double *rho, cudaStream_t s);

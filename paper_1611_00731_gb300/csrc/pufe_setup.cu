@@ -1551,6 +1551,22 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   }
   ctx->n_tblk = tblk[nelem];
 
+  // work list of the sum-factorized FP64 assembly
+  ctx->n_e = n_e;
+  ctx->q_e = q_e;
+  std::vector<int32_t> aitems;
+  {
+    int nsm = 152;
+    if (ctx->on_device) {
+      int v = 0;
+      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
+          v > 0)
+        nsm = v;
+    }
+    sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
+  }
+  ctx->n_aitems = (int)(aitems.size() / 4);
+
   pufe_status st;
   auto &D = ctx->d;
   if (ctx->on_device) {
@@ -1580,6 +1596,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   if ((st = upload(&D.smap, smap)) != PUFE_OK) return st;
   if ((st = upload(&D.order, order)) != PUFE_OK) return st;
   if (!wsplit.empty() && (st = upload(&D.wsplit, wsplit)) != PUFE_OK) return st;
+  if (!aitems.empty() && (st = upload(&D.aitems, aitems)) != PUFE_OK) return st;
   if (!titems.empty() && (st = upload(&D.titems, titems)) != PUFE_OK) return st;
   if (!sitems.empty() && (st = upload(&D.sitems, sitems)) != PUFE_OK) return st;
   if (!gitems32.empty() && (st = upload(&D.gitems32, gitems32)) != PUFE_OK) return st;
@@ -1616,8 +1633,6 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   ctx->col = std::move(colv);
   ctx->doff = std::move(doff);
   ctx->dofs = std::move(dofs);
-  ctx->n_e = std::move(n_e);
-  ctx->q_e = std::move(q_e);
   ctx->order = std::move(order);
   ctx->x = std::move(X);
   ctx->w = std::move(Wt);
@@ -1630,7 +1645,7 @@ static void free_device(pufe_ctx *ctx) {
   void *ptrs[] = {D.qoff, D.x, D.w, D.xi, D.doff, D.dofs, D.ecol, D.eshift, D.aoff, D.alist,
                   D.toff, D.psi, D.psi32, D.qpoff, D.qdat, D.ptab, D.vpad, D.toff32, D.eorig,
                   D.Tfe, D.Sfe, D.S0, D.partoff, D.part_p, D.part_q,
-                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit,
+                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems,
                   D.titems, D.sitems, D.gitems32, D.gitems64, D.citems, D.pitems, D.tblk, D.eeform, D.err};
   for (void *p : ptrs)
     if (p) cudaFree(p);
