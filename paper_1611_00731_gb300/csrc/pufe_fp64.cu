@@ -1,7 +1,6 @@
 // FP64 CUDA-core kernels of the PUFE hot path:
 //   K0  enrichment tabulation (Sec. 5.1, eqs. Psitilde/Psi)
 //   K1+K2+K3  element basis tile, contraction and scatter (Sec. 4, eq. disceig3d)
-//   K4  density at quadrature points (Sec. 3, eq. rhoe)
 //   K5  adjoint of V -> H (derivative of sum Hbar_ij H_ij with respect to V_q)
 //
 // The element basis (the FE columns -- 64 tricubic or 32 cubic serendipity
@@ -17,7 +16,6 @@ namespace {
 
 constexpr int QC = 8;         // quadrature points per chunk
 constexpr int ASM_NT = 256;   // threads of the assembly kernel
-constexpr int DEN_NT = 128;   // threads of the density kernel
 constexpr int ADJ_NT = 256;   // threads of the adjoint kernel
 
 __device__ __forceinline__ void set_err(unsigned *err, unsigned bit) { atomicOr(err, bit); }
@@ -313,116 +311,6 @@ __global__ void __launch_bounds__(ASM_NT) k_assemble_fp64(
           }
         }
     }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// K4 (FP64): one CTA per element, one thread per quadrature point.  The
-// element's coefficient block C_e (n x nocc, gathered through the element DOF
-// list) sits in shared memory; each thread evaluates its basis row on the fly.
-// ---------------------------------------------------------------------------
-template <int KC, bool SER>
-__device__ __forceinline__ double density_point(const double xi[3], int q, int Q, int nenr,
-                                                const int32_t *ec, const double *pe,
-                                                const double *Cs, const double *fs, int nocc,
-                                                int k0) {
-  double acc[KC];
-#pragma unroll
-  for (int k = 0; k < KC; ++k) acc[k] = 0.0;
-  constexpr int NF = SER ? 32 : 64;
-  if (SER) {   // the 32 serendipity columns
-    for (int c = 0; c < 32; ++c) {
-      double b, g3[3];
-      serendipity32(c, xi, b, g3);
-      const double *cr = Cs + c * nocc + k0;
-#pragma unroll
-      for (int k = 0; k < KC; ++k) acc[k] = fma(b, cr[k], acc[k]);
-    }
-  } else {
-    double L[3][4], dL[3][4];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) lagrange3(xi[d], L[d], dL[d]);
-#pragma unroll
-    for (int c3 = 0; c3 < 4; ++c3)
-#pragma unroll
-      for (int c2 = 0; c2 < 4; ++c2) {
-        const double lyz = L[1][c2] * L[2][c3];
-#pragma unroll
-        for (int c1 = 0; c1 < 4; ++c1) {
-          const double b = L[0][c1] * lyz;
-          const double *cr = Cs + (c1 + 4 * c2 + 16 * c3) * nocc + k0;
-#pragma unroll
-          for (int k = 0; k < KC; ++k) acc[k] = fma(b, cr[k], acc[k]);
-        }
-      }
-  }
-  for (int j = 0; j < nenr; ++j) {
-    const int code = ec[j];
-    const int slot = code >> 3, lv = code & 7;
-    double phi = 1.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) phi *= ((lv >> d) & 1) ? 0.5 * (1.0 + xi[d]) : 0.5 * (1.0 - xi[d]);
-    const double b = phi * pe[(int64_t)slot * 4 * Q + q];
-    const double *cr = Cs + (NF + j) * nocc + k0;
-#pragma unroll
-    for (int k = 0; k < KC; ++k) acc[k] = fma(b, cr[k], acc[k]);
-  }
-  double r = 0.0;
-#pragma unroll
-  for (int k = 0; k < KC; ++k) r = fma(fs[k0 + k] * acc[k], acc[k], r);
-  return r;
-}
-
-// BLOCH: complex coefficients C + i Ci; each element block is gathered with
-// the column phases applied, and n = sum_k f_k (Re psi_k^2 + Im psi_k^2).
-template <bool BLOCH, bool SER>
-__global__ void __launch_bounds__(DEN_NT) k_density_fp64(
-    const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
-    const double *__restrict__ xi_all, const int64_t *__restrict__ doff,
-    const int32_t *__restrict__ dofs, const int32_t *__restrict__ ecol,
-    const int64_t *__restrict__ toff, const double *__restrict__ psi,
-    const double *__restrict__ C, int64_t ldc, const double *__restrict__ f, int nocc,
-    int noccp, double *__restrict__ rho, const uint8_t *__restrict__ eshift, PhaseTab ph,
-    const double *__restrict__ Ci) {
-  extern __shared__ __align__(16) double smem[];
-  const int e = order[blockIdx.x];
-  const int64_t q0 = qoff[e];
-  const int Q = (int)(qoff[e + 1] - q0);
-  const int n = (int)(doff[e + 1] - doff[e]);
-  constexpr int NF = SER ? 32 : 64;   // FE columns
-  const int nenr = n - NF;
-  const int32_t *ec = ecol + (doff[e] - (int64_t)NF * e);
-  const int32_t *dl = dofs + doff[e];
-  const double *pe = psi + 4 * toff[e];
-  double *Cs = smem;             // n x noccp
-  double *fs = Cs + n * noccp;   // noccp
-  double *Cz = fs + noccp;       // n x noccp, imaginary parts (BLOCH)
-  for (int k = threadIdx.x; k < n * noccp; k += DEN_NT) {
-    const int j = k / noccp, kk = k - j * noccp;
-    if (BLOCH) {
-      double cr = 0.0, ci = 0.0;
-      if (kk < nocc) {
-        const double ar = C[(int64_t)dl[j] * ldc + kk], ai = Ci[(int64_t)dl[j] * ldc + kk];
-        const int c = eshift[doff[e] + j];
-        cr = ph.re[c] * ar - ph.im[c] * ai;
-        ci = ph.re[c] * ai + ph.im[c] * ar;
-      }
-      Cs[k] = cr;
-      Cz[k] = ci;
-    } else {
-      Cs[k] = (kk < nocc) ? C[(int64_t)dl[j] * ldc + kk] : 0.0;
-    }
-  }
-  for (int k = threadIdx.x; k < noccp; k += DEN_NT) fs[k] = (k < nocc) ? f[k] : 0.0;
-  __syncthreads();
-  for (int q = threadIdx.x; q < Q; q += DEN_NT) {
-    const double xq[3] = {xi_all[3 * (q0 + q)], xi_all[3 * (q0 + q) + 1], xi_all[3 * (q0 + q) + 2]};
-    double r = 0.0;
-    for (int k0 = 0; k0 < noccp; k0 += 8) {
-      r += density_point<8, SER>(xq, q, Q, nenr, ec, pe, Cs, fs, noccp, k0);
-      if (BLOCH) r += density_point<8, SER>(xq, q, Q, nenr, ec, pe, Cz, fs, noccp, k0);
-    }
-    rho[q0 + q] = r;
   }
 }
 
@@ -758,16 +646,11 @@ pufe_status launch_density_fp64(pufe_ctx *ctx, const double *C, int64_t ldc, con
   const int noccp = (nocc + 7) & ~7;
   const size_t sm = ((size_t)ctx->max_basis * noccp + noccp) * sizeof(double);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e * nocc too large for the density kernel");
-  auto kern = ctx->ser ? k_density_fp64<false, true> : k_density_fp64<false, false>;
-  PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<(unsigned)ctx->nelem, DEN_NT, sm, st>>>(
-      D.order, D.qoff, D.xi, D.doff, D.dofs, D.ecol, D.toff, D.psi, C, ldc, f, nocc, noccp, rho,
-      nullptr, PhaseTab{}, nullptr);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
+  return launch_density_sf64(ctx, nullptr, C, nullptr, ldc, f, nocc, rho, st);
 }
 
 pufe_status launch_adjoint_fp64(pufe_ctx *ctx, const double *Hbar, double *Vbar, cudaStream_t st) {
+  if (ctx->n_jitems > 0) return launch_adjoint_sf64(ctx, nullptr, Hbar, nullptr, Vbar, st);
   auto &D = ctx->d;
   const int n = ctx->max_basis;
   size_t sm = (size_t)QC * n * sizeof(double) + QC * sizeof(double) + QC * sizeof(Tab1D);
@@ -810,17 +693,12 @@ pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const d
   const int noccp = (nocc + 7) & ~7;
   const size_t sm = ((size_t)2 * ctx->max_basis * noccp + noccp) * sizeof(double);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e * nocc too large for the density kernel");
-  auto kern = ctx->ser ? k_density_fp64<true, true> : k_density_fp64<true, false>;
-  PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<(unsigned)ctx->nelem, DEN_NT, sm, st>>>(
-      D.order, D.qoff, D.xi, D.doff, D.dofs, D.ecol, D.toff, D.psi, Cr, ldc, f, nocc, noccp, rho,
-      D.eshift, ph, Ci);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
+  return launch_density_sf64(ctx, &ph, Cr, Ci, ldc, f, nocc, rho, st);
 }
 
 pufe_status launch_adjoint_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Hr,
                                       const double *Hi, double *Vbar, cudaStream_t st) {
+  if (ctx->n_jitems > 0) return launch_adjoint_sf64(ctx, &ph, Hr, Hi, Vbar, st);
   auto &D = ctx->d;
   const int n = ctx->max_basis;
   size_t sm = (size_t)QC * n * sizeof(double) + QC * sizeof(double) + QC * sizeof(Tab1D);

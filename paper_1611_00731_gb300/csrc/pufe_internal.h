@@ -101,8 +101,13 @@ struct DeviceArrays {
   // FP64 assembly/adjoint work list, 3 per item (element, first point, end
   // point), largest first; null when every item is a whole element
   int32_t *wsplit = nullptr;
-  // sum-factorized FP64 assembly: (element, kind, begin, end) items
+  // sum-factorized FP64 assembly: (element, kind, begin, end, (sub)cell range) items
   int32_t *aitems = nullptr;
+  // FP64 adjoint: (element, kind, begin, end, (sub)cell range) items; FP64 density: (element,
+  // (sub)cell, first plane, end plane) units; nodal values of the serendipity
+  // functions at the tricubic nodes (64 x 32, serendipity space only)
+  int32_t *jitems = nullptr, *dunits = nullptr;
+  double *Rser = nullptr;
   // mixed-path work list of the n_e > 128 elements, 3 per item (index into
   // `order`, first chunk, end chunk; chunks of 8 padded points), largest first
   int32_t *titems = nullptr;
@@ -151,6 +156,8 @@ struct pufe_ctx {
   int64_t n_wsplit = 0;       // items of the FP64 point-range work list (0: none)
   int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
   int asm64_work = 0;         // doubles of its shared work area
+  int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
+  int n_dunits = 0;           // units of the FP64 density (0: direct form)
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
   int n_gitems32 = 0, n_gitems64 = 0;   // items of the Gram-form lists
@@ -448,6 +455,14 @@ pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double
 pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
                                  double *H, double *Hi, double *S, double *Si, cudaStream_t s);
 void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, int &work);
+// FP64 adjoint and density by sum factorization, and their work lists
+pufe_status launch_adjoint_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *Hr,
+                                const double *Hi, double *Vbar, cudaStream_t s);
+pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *C,
+                                const double *Ci, int64_t ldc, const double *f, int nocc,
+                                double *rho, cudaStream_t s);
+void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
+                     std::vector<int32_t> &den);
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,
                                       const double *Ci, int64_t ldc, const double *f, int nocc,
                                       double *rho, cudaStream_t s);

@@ -1551,10 +1551,10 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   }
   ctx->n_tblk = tblk[nelem];
 
-  // work list of the sum-factorized FP64 assembly
+  // work lists of the sum-factorized FP64 assembly, adjoint and density
   ctx->n_e = n_e;
   ctx->q_e = q_e;
-  std::vector<int32_t> aitems;
+  std::vector<int32_t> aitems, jitems, dunits;
   {
     int nsm = 152;
     if (ctx->on_device) {
@@ -1564,8 +1564,11 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
         nsm = v;
     }
     sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
+    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits);
   }
-  ctx->n_aitems = (int)(aitems.size() / 4);
+  ctx->n_aitems = (int)(aitems.size() / 6);
+  ctx->n_jitems = (int)(jitems.size() / 6);
+  ctx->n_dunits = (int)(dunits.size() / 4);
 
   pufe_status st;
   auto &D = ctx->d;
@@ -1597,6 +1600,21 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   if ((st = upload(&D.order, order)) != PUFE_OK) return st;
   if (!wsplit.empty() && (st = upload(&D.wsplit, wsplit)) != PUFE_OK) return st;
   if (!aitems.empty() && (st = upload(&D.aitems, aitems)) != PUFE_OK) return st;
+  if (!jitems.empty() && (st = upload(&D.jitems, jitems)) != PUFE_OK) return st;
+  if (!dunits.empty() && (st = upload(&D.dunits, dunits)) != PUFE_OK) return st;
+  if (ser) {
+    std::vector<double> R(64 * 32);
+    for (int j = 0; j < 64; ++j) {
+      const double nd[4] = {-1.0, -1.0 / 3.0, 1.0 / 3.0, 1.0};
+      const double xi[3] = {nd[j & 3], nd[(j >> 2) & 3], nd[j >> 4]};
+      double g[3];
+      for (int c = 0; c < 32; ++c) {
+        serendipity32(c, xi, R[32 * j + c], g);
+        if (std::fabs(R[32 * j + c]) < 1e-15) R[32 * j + c] = 0.0;   // zeros up to rounding
+      }
+    }
+    if ((st = upload(&D.Rser, R)) != PUFE_OK) return st;
+  }
   if (!titems.empty() && (st = upload(&D.titems, titems)) != PUFE_OK) return st;
   if (!sitems.empty() && (st = upload(&D.sitems, sitems)) != PUFE_OK) return st;
   if (!gitems32.empty() && (st = upload(&D.gitems32, gitems32)) != PUFE_OK) return st;
@@ -1645,7 +1663,7 @@ static void free_device(pufe_ctx *ctx) {
   void *ptrs[] = {D.qoff, D.x, D.w, D.xi, D.doff, D.dofs, D.ecol, D.eshift, D.aoff, D.alist,
                   D.toff, D.psi, D.psi32, D.qpoff, D.qdat, D.ptab, D.vpad, D.toff32, D.eorig,
                   D.Tfe, D.Sfe, D.S0, D.partoff, D.part_p, D.part_q,
-                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems,
+                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems, D.jitems, D.dunits, D.Rser,
                   D.titems, D.sitems, D.gitems32, D.gitems64, D.citems, D.pitems, D.tblk, D.eeform, D.err};
   for (void *p : ptrs)
     if (p) cudaFree(p);

@@ -58,7 +58,7 @@ namespace {
 constexpr int A64_NT = 128;
 
 struct Asm64 {
-  const int4 *items;
+  const int32_t *items;   // six per item: element, kind, range, (sub)cell range
   const int64_t *qoff;
   const double *w, *xi;
   const int32_t *partoff, *part_p, *part_q;
@@ -116,17 +116,17 @@ __device__ __forceinline__ double axis_xi(const Asm64 &P, int64_t qs, int p, int
 
 // ---- FE x FE block -----------------------------------------------------------
 template <bool BLOCH>
-__device__ void fefe_item(const Asm64 &P, int e, double *sm) {
+__device__ void fefe_item(const Asm64 &P, int e, int cb, int ce, double *sm) {
   const int tid = threadIdx.x;
   double *M = sm;   // 1000 moments
   for (int o = tid; o < 1000; o += A64_NT) M[o] = 0.0;
   const bool h = (P.want & PUFE_WANT_H) != 0;
-  if (!h && P.V) {   // an S-only call still reports a V that is not finite
+  if (!h && P.V && cb == 0) {   // an S-only call still reports a V that is not finite
     bool bad = false;
     for (int64_t q = P.qoff[e] + tid; q < P.qoff[e + 1]; q += A64_NT) bad |= !isfinite(P.V[q]);
     if (bad) atomicOr(P.err, DEVERR_NONFINITE);
   }
-  for (int k = P.partoff[e]; h && k < P.partoff[e + 1]; ++k) {
+  for (int k = P.partoff[e] + cb; h && k < P.partoff[e] + ce; ++k) {
     const int p = P.part_p[k], p2 = p * p;
     double *F = M + 1000;           // [axis][10][p]
     double *G1 = F + 30 * p;        // [10][p^2]
@@ -190,13 +190,14 @@ __device__ void fefe_item(const Asm64 &P, int e, double *sm) {
   const int n = (int)(P.doff[e + 1] - P.doff[e]);
   const int32_t *m = P.smap + P.soff[e];
   const uint8_t *es = P.eshift + P.doff[e];
-  // at the Gamma point S starts as the summed constants, so only H is added
-  const bool s = BLOCH && (P.want & PUFE_WANT_S);
+  // the constants come with the element's first (sub)cell range; at the Gamma
+  // point S starts as their sum, so only H is added
+  const bool s = BLOCH && (P.want & PUFE_WANT_S) && cb == 0;
   for (int o = tid; o < 4096; o += A64_NT) {
     const int i = o >> 6, j = o & 63;
     const double v = M[pidx64(i & 3, j & 3) * 100 + pidx64((i >> 2) & 3, (j >> 2) & 3) * 10 +
                        pidx64(i >> 4, j >> 4)];
-    add_entry<BLOCH>(P, m[i * n + j], h ? P.Tfe[o] + v : 0.0, s ? P.Sfe[o] : 0.0, h, s,
+    add_entry<BLOCH>(P, m[i * n + j], h && cb == 0 ? P.Tfe[o] + v : v, s ? P.Sfe[o] : 0.0, h, s,
                      BLOCH ? es[i] : 0, BLOCH ? es[j] : 0);
   }
 }
@@ -234,7 +235,7 @@ constexpr int FXE_EXP = 1616;   // doubles of the expansion's intermediates
 constexpr int EXE_MOM = 162;    // moments of a slot pair
 
 template <bool BLOCH>
-__device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, double *sm) {
+__device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x, G = s1 - s0;
   const bool h = (P.want & PUFE_WANT_H) != 0, ws = (P.want & PUFE_WANT_S) != 0;
   const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - 64;
@@ -253,7 +254,7 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, double *sm) {
     if (c >= 0 && c < 8 * G) scol[c] = o;
   }
   const int nr1 = h ? 24 : 5, nr2 = h ? 115 : 25;   // rows of the z and y stages
-  for (int k = P.partoff[e]; k < P.partoff[e + 1]; ++k) {
+  for (int k = P.partoff[e] + cb; k < P.partoff[e] + ce; ++k) {
     const int p = P.part_p[k], p2 = p * p, GP2 = G * p2, GP = G * p, pq = P.part_q[k];
     const int64_t qs = q0 + pq;
     double *F = base;              // [axis][5][p]: L_0..L_3, omega
@@ -416,7 +417,7 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, double *sm) {
 // ---- enrichment x enrichment block of the slot pairs [k0, k1) ------------------
 // z rows: A u (3), E u (3), B_x u, C_x u, B_y u, C_y u (3 each), B_z l, C_z l (2 each)
 template <bool BLOCH>
-__device__ void exe_item(const Asm64 &P, int e, int k0, int k1, double *sm) {
+__device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x;
   const bool h = (P.want & PUFE_WANT_H) != 0, ws = (P.want & PUFE_WANT_S) != 0;
   const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - 64;
@@ -453,7 +454,7 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, double *sm) {
       pr[2 * o] = a;
       pr[2 * o + 1] = a + t;
     }
-    for (int k = P.partoff[e]; k < P.partoff[e + 1]; ++k) {
+    for (int k = P.partoff[e] + cb; k < P.partoff[e] + ce; ++k) {
       const int p = P.part_p[k], p2 = p * p, NP2 = nc * p2, NP = nc * p, pq = P.part_q[k];
       const int64_t qs = q0 + pq;
       double *T1 = F + 18 * p;      // [22][nc p^2]
@@ -698,15 +699,16 @@ __device__ void eed_item(const Asm64 &P, int e, int qa, int qb, double *sm) {
 template <bool BLOCH>
 __global__ void __launch_bounds__(A64_NT) k_assemble_sf64(Asm64 P) {
   extern __shared__ __align__(16) double sm64[];
-  const int4 it = P.items[blockIdx.x];   // element, kind, range
-  if (it.y == 0)
-    fefe_item<BLOCH>(P, it.x, sm64);
-  else if (it.y == 1)
-    fxe_item<BLOCH>(P, it.x, it.z, it.w, sm64);
-  else if (it.y == 2)
-    exe_item<BLOCH>(P, it.x, it.z, it.w, sm64);
+  const int32_t *it = P.items + 6ll * blockIdx.x;
+  const int e = it[0], kind = it[1], a = it[2], b = it[3], cb = it[4], ce = it[5];
+  if (kind == 0)
+    fefe_item<BLOCH>(P, e, cb, ce, sm64);
+  else if (kind == 1)
+    fxe_item<BLOCH>(P, e, a, b, cb, ce, sm64);
+  else if (kind == 2)
+    exe_item<BLOCH>(P, e, a, b, cb, ce, sm64);
   else
-    eed_item<BLOCH>(P, it.x, it.z, it.w, sm64);
+    eed_item<BLOCH>(P, e, a, b, sm64);
 }
 
 // shared doubles of one item
@@ -738,11 +740,13 @@ static double ee_pair_ops(const std::vector<int32_t> &cells) {
   return c;
 }
 
-// Work list of the sum-factorized FP64 assembly (host): int4 items (element,
-// kind 0 FE x FE / 1 slot range / 2 pair range / 3 point range of the direct
-// E x E products, begin, end), largest first.  Items are cut to the mean cost of
-// a CTA slot (four per SM) as far as slots, pairs and points allow; slot ranges
-// also to what the shared work area holds.  The E x E block takes the form of
+// Work list of the sum-factorized FP64 assembly (host): items (element, kind 0
+// FE x FE / 1 slot range / 2 pair range / 3 point range of the direct E x E
+// products, begin, end, (sub)cell range), largest first.  Items are cut to the
+// mean cost of a CTA slot (four per SM) as far as slots, pairs and points allow,
+// then by (sub)cells where the cells' work is several times what a range adds
+// (the expansion of its moments and the scatter); slot ranges also to what the
+// shared work area holds.  The E x E block takes the form of
 // fewer operations: slots of one vertex column each (64 + 30 functions, 30 slots,
 // 4,096 points: 12 M direct against 88 M) fall on the direct side, slots of eight
 // (64 + 40, 5 slots, 216 points: 1.06 M against 0.18 M) on the other.
@@ -752,7 +756,7 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
   if (ctx->general || ctx->ser || !ctx->fe_exact || ctx->max_part_p > 16) return;
   const int64_t ne = (int64_t)ctx->n_e.size();
   struct Item {
-    int32_t e, kind, a, b;
+    int32_t e, kind, a, b, cb, ce;
     double c;
   };
   double total = 0.0;
@@ -774,16 +778,25 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
   }
   const double target = std::max(1.0, total / (4.0 * nsm));
   std::vector<Item> L;
+  // one range over (sub)cell ranges of at least `least` operations
+  auto cells = [&](int64_t e, int kind, int a, int b, double c, double least) {
+    const int nc = (int)ctx->part_p_host[e].size();
+    const double m = std::min(std::min(std::ceil(c / target), c / least), (double)nc);
+    const int cuts = std::max(1, (int)m);
+    for (int j = 0; j < cuts; ++j)
+      L.push_back(Item{(int32_t)e, kind, a, b, (int)((int64_t)j * nc / cuts),
+                       (int)((int64_t)(j + 1) * nc / cuts), c / cuts});
+  };
   for (int64_t e = 0; e < ne; ++e) {
     const int A = ctx->n_slot[e], np = A * (A + 1) / 2, p = pm[e], nE = ctx->n_e[e] - 64;
-    L.push_back(Item{(int32_t)e, 0, 0, 0, cf[e]});
+    cells(e, 0, 0, 0, cf[e], 40000.0);
     work = std::max(work, fefe_doubles(p));
     if (A == 0) continue;
     int G = std::max(1, std::min(A, (int)std::min(1e6, target / cs[e])));
     while (G > 1 && fxe_doubles(G, p) > A64_WORK) --G;
     work = std::max(work, fxe_doubles(G, p));
     for (int a = 0; a < A; a += G)
-      L.push_back(Item{(int32_t)e, 1, a, std::min(A, a + G), cs[e] * std::min(G, A - a)});
+      cells(e, 1, a, std::min(A, a + G), cs[e] * std::min(G, A - a), 40000.0 * G);
     if (cd[e] < np * cp[e]) {
       const int Q = ctx->q_e[e];
       const int cuts = std::max(1, std::min(Q / 32, (int)std::min(1e6, std::ceil(cd[e] / target))));
@@ -791,7 +804,7 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
       work = std::max(work, std::min(A64_WORK, 5 * nE * ((Q + cuts - 1) / cuts) + 2 * A64_NT));
       for (int j = 0; j < cuts; ++j) {
         const int a = (int)((int64_t)j * Q / cuts), b = (int)((int64_t)(j + 1) * Q / cuts);
-        L.push_back(Item{(int32_t)e, 3, a, b, cd[e] * (b - a) / Q});
+        L.push_back(Item{(int32_t)e, 3, a, b, 0, 0, cd[e] * (b - a) / Q});
       }
       continue;
     }
@@ -800,7 +813,7 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
     const int cuts = (np + M - 1) / M;
     for (int j = 0; j < cuts; ++j) {
       const int a = (int)((int64_t)j * np / cuts), b = (int)((int64_t)(j + 1) * np / cuts);
-      L.push_back(Item{(int32_t)e, 2, a, b, cp[e] * (b - a)});
+      cells(e, 2, a, b, cp[e] * (b - a), 8000.0 * (b - a));
       for (int c = b - a; c > 1; --c)   // pairs that fit the work area together
         if (exe_doubles(A, c, p) <= A64_WORK) {
           work = std::max(work, exe_doubles(A, c, p));
@@ -809,7 +822,7 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
     }
   }
   std::stable_sort(L.begin(), L.end(), [](const Item &x, const Item &y) { return x.c > y.c; });
-  for (const Item &i : L) items.insert(items.end(), {i.e, i.kind, i.a, i.b});
+  for (const Item &i : L) items.insert(items.end(), {i.e, i.kind, i.a, i.b, i.cb, i.ce});
 }
 
 // H, S (and Hi, Si at a wavevector: ph != nullptr) must hold zeros, S at the
@@ -818,7 +831,7 @@ pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double
                                  double *H, double *Hi, double *S, double *Si, cudaStream_t st) {
   auto &D = ctx->d;
   Asm64 P{};
-  P.items = reinterpret_cast<const int4 *>(D.aitems);
+  P.items = D.aitems;
   P.qoff = D.qoff;
   P.w = D.w;
   P.xi = D.xi;

@@ -2,7 +2,8 @@
 FP64 oracle: the smallest and largest points per axis (4 and 16) that the
 factorized assembly takes and the 3 that it leaves to the direct kernel, one
 element (every node repeated by periodicity), slots of one vertex column (the
-direct enrichment blocks) and of eight (the pair form).  Tolerance 1e-12 of the
+direct enrichment blocks) and of eight (the pair form), one state, an odd count
+and the most that a call takes.  Tolerance 1e-12 of the
 largest entry, as in the other FP64 parity tests."""
 import math
 
@@ -24,7 +25,9 @@ CELLS = {
     "p9": lambda: W.small_two_atom(nel=2, quad_p=9),
     "p16_one_element": lambda: W.small_two_atom(nel=1, quad_p=16),
     "one_vertex_slots": lambda: W.small_two_atom(nel=3, quad_p=6, r_e=0.5),
-    "wide_support": lambda: W.small_two_atom(nel=3, quad_p=5, r_c=1.9, r_e=1.9),
+    # (an even order: an odd one puts a point on the nucleus, where the oracle's
+    # direction cosines are 0/0)
+    "wide_support": lambda: W.small_two_atom(nel=3, quad_p=6, r_c=1.9, r_e=1.9),
 }
 
 
@@ -78,3 +81,37 @@ def test_assembly_at_a_wavevector(cell):
     c = lambda v: _csr(ctx, v[0].cpu().numpy() + 1j * v[1].cpu().numpy())
     assert _off(c(H), Ho) < TOL
     assert _off(c(S), So) < TOL
+
+
+@pytest.mark.parametrize("nocc", [1, 17, 64])
+def test_density(cell, nocc):
+    wl, m, rules, ctx = cell
+    Cm = W.random_coefficients(ctx.n_dof, nocc, seed=nocc)
+    f = W.random_occupations(nocc, seed=nocc)
+    rho = torch.full((ctx.n_q,), 3.0, dtype=torch.float64, device="cuda:0")
+    ctx.pufe_density(_dev(Cm), _dev(f), rho)
+    ctx.pufe_sync_status()
+    assert _off(rho.cpu().numpy(), oasm.density(m, rules, Cm, f)) < TOL
+
+
+def test_adjoint(cell):
+    wl, m, rules, ctx = cell
+    h = W.random_symmetric_values(ctx.nnz, seed=3)   # (not symmetrised: a general cotangent)
+    v = torch.full((ctx.n_q,), 3.0, dtype=torch.float64, device="cuda:0")
+    ctx.pufe_assemble_HV_adjoint(_dev(h), v)
+    ctx.pufe_sync_status()
+    assert _off(v.cpu().numpy(), oasm.adjoint_V(m, rules, _csr(ctx, h))) < TOL
+
+
+def test_density_and_adjoint_at_a_wavevector(cell):
+    wl, m, rules, ctx = cell
+    k = 2.0 * math.pi / wl["a"] * np.array([0.3, -0.2, 0.1])
+    Cr, Ci = (W.random_coefficients(ctx.n_dof, 7, seed=s) for s in (1, 2))
+    f = W.random_occupations(7, seed=3)
+    hr, hi = (W.random_symmetric_values(ctx.nnz, seed=s) for s in (4, 5))
+    out = [torch.full((ctx.n_q,), 3.0, dtype=torch.float64, device="cuda:0") for _ in range(2)]
+    ctx.pufe_density_bloch(k, _dev(Cr), _dev(Ci), _dev(f), out[0])
+    ctx.pufe_assemble_HV_adjoint_bloch(k, _dev(hr), _dev(hi), out[1])
+    ctx.pufe_sync_status()
+    assert _off(out[0].cpu().numpy(), ob.density_k(m, rules, Cr + 1j * Ci, f, k)) < TOL
+    assert _off(out[1].cpu().numpy(), ob.adjoint_V_k(m, rules, _csr(ctx, hr + 1j * hi), k)) < TOL
