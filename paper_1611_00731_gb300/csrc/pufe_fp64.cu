@@ -23,34 +23,110 @@ __device__ __forceinline__ void set_err(unsigned *err, unsigned bit) { atomicOr(
 // ---------------------------------------------------------------------------
 // K0: Psi and grad Psi for every (enrichment slot, quadrature point) of an element.
 // Layout per element: psi[4*toff[e] + (slot*4 + comp)*Q + q].
+//
+// One CTA per work item, a run of slots of one element that share an atom and
+// TAB64_NT of its points; one thread per point.  FP64 operations bind it (two
+// multiply-adds per clock and SM), so what the orbitals of an atom share is
+// formed once per point: the displacement, its length, the cutoff and its slope;
+// the exponential and the radial function carry over while consecutive slots have
+// the same exponent and the same (n, l).  Only the images that can lie within r_c
+// are visited: those with |s_d + i| <= r_c b_d on every lattice direction (s_d the
+// displacement in lattice coordinates, 1/b_d the distance of the lattice planes),
+// one or two per axis instead of 27 in all.  On the 12^3 rocksalt cell that is
+// about 40 operations per value in place of 400, and the elements of 30 slots and
+// 4,096 points of the CsCl-like cell spread over 32 CTAs each instead of one.
+// Measured: 12^3 rocksalt 2.19 -> 0.21 ms, CsCl-like 16^3 30.3 -> 0.26 ms, two-atom
+// 4^3 377 -> 30 us.
 // ---------------------------------------------------------------------------
-// (general cells: `gen` with the lattice `lat`, Sec. 6.2)
-__global__ void k_tabulate(const int64_t *__restrict__ qoff, const double *__restrict__ x,
-                           const int32_t *__restrict__ aoff, const int32_t *__restrict__ alist,
-                           const int64_t *__restrict__ toff, const Orbital *__restrict__ orb,
-                           double a0, double a1, double a2, int i0, int i1, int i2,
-                           double *__restrict__ psi, int gen, LatticeDev lat) {
-  const int64_t e = blockIdx.x;
-  const int64_t q0 = qoff[e];
+constexpr int TAB64_NT = 128;
+
+// (general cells: `gen`, Sec. 6.2)
+__global__ void __launch_bounds__(TAB64_NT) k_tabulate(
+    const int4 *__restrict__ items, const int64_t *__restrict__ qoff,
+    const double *__restrict__ x, const int32_t *__restrict__ aoff,
+    const int32_t *__restrict__ alist, const int64_t *__restrict__ toff,
+    const Orbital *__restrict__ orb, LatticeDev lat, double b0, double b1, double b2, int gen,
+    double *__restrict__ psi) {
+  const int4 it = items[blockIdx.x];   // element, first slot, slots, first point
+  const int64_t e = it.x, q0 = qoff[e];
   const int Q = (int)(qoff[e + 1] - q0);
-  const int A = aoff[e + 1] - aoff[e];
-  const double av[3] = {a0, a1, a2};
-  const int img[3] = {i0, i1, i2};
-  double *out = psi + 4 * toff[e];
-  for (int idx = threadIdx.x; idx < Q * A; idx += blockDim.x) {
-    const int slot = idx / Q, q = idx - slot * Q;
-    const Orbital o = orb[alist[aoff[e] + slot]];
-    const double p[3] = {x[3 * (q0 + q)], x[3 * (q0 + q) + 1], x[3 * (q0 + q) + 2]};
-    double v, g[3];
-    if (gen)
-      enrichment_eval_lat(o, p, lat, v, g);
-    else
-      enrichment_eval(o, p, av, img, v, g);
-    double *dst = out + (int64_t)slot * 4 * Q + q;
-    dst[0] = v;
-    dst[Q] = g[0];
-    dst[2 * Q] = g[1];
-    dst[3 * Q] = g[2];
+  const int32_t *al = alist + aoff[e] + it.y;
+  double *out = psi + 4 * toff[e] + (int64_t)it.y * 4 * Q;
+  for (int q = it.w + threadIdx.x; q < min(it.w + TAB64_CHUNK, Q); q += TAB64_NT) {
+    const Orbital &o0 = orb[al[0]];   // the atom and the cutoff of the run
+    const double rc = o0.rc, irc = 1.0 / rc, bn[3] = {b0, b1, b2};
+    double d[3], s[3];
+    int lo[3], hi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d[k] = x[3 * (q0 + q) + k] - o0.tau[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      s[k] = gen ? lat.Lit[3 * k] * d[0] + lat.Lit[3 * k + 1] * d[1] + lat.Lit[3 * k + 2] * d[2]
+                 : d[k] * lat.Lit[4 * k];
+      const double reach = rc * bn[k] * (1.0 + 1e-9);
+      lo[k] = (int)ceil(-reach - s[k]);
+      hi[k] = (int)floor(reach - s[k]);
+    }
+    bool first = true;
+    for (int i = lo[0]; i <= hi[0]; ++i)
+      for (int j = lo[1]; j <= hi[1]; ++j)
+        for (int k = lo[2]; k <= hi[2]; ++k) {
+          double v[3];
+          if (gen) {
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+              v[m] = d[m] + (i * lat.L[m] + j * lat.L[3 + m] + k * lat.L[6 + m]);
+          } else {
+            v[0] = d[0] + i * lat.L[0];
+            v[1] = d[1] + j * lat.L[4];
+            v[2] = d[2] + k * lat.L[8];
+          }
+          const double r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+          if (r2 >= rc * rc) continue;
+          const double r = sqrt(r2), t = r * irc, t3 = t * t * t, om = 1.0 - t;
+          const double ir = r > 1e-14 ? 1.0 / r : 0.0;
+          const double hc = 1.0 + t3 * t * (-35.0 + t * (84.0 + t * (-70.0 + 20.0 * t)));
+          const double dh = -140.0 * irc * t3 * om * om * om;
+          double zeta = -1.0, ex = 0.0, f = 0.0, df = 0.0;
+          int pn = -1, pl = -1;
+          for (int c = 0; c < it.z; ++c) {
+            const Orbital &o = orb[al[c]];
+            if (o.zeta != zeta || o.n != pn || o.l != pl) {   // the radial function of (n, l, zeta)
+              if (o.zeta != zeta) ex = exp(-o.zeta * r);
+              zeta = o.zeta;
+              pn = o.n;
+              pl = o.l;
+              const int kk = pn - 1 - pl;
+              double rk = 1.0, rkm = 0.0;
+              for (int u = 0; u < kk; ++u) {
+                rkm = rk;
+                rk *= r;
+              }
+              const double ez = o.norm * ex, rh = rk * hc;
+              f = ez * rh;
+              df = ez * fma(rk, dh, fma((double)kk * rkm, hc, -zeta * rh)) * ir;
+            }
+            double gs[3];
+            const double S = solid_harmonic<double>(o.l, o.m, v[0], v[1], v[2], gs);
+            const double ds = df * S;
+            double *dst = out + (int64_t)c * 4 * Q + q;
+            double w0 = f * S, w1 = fma(ds, v[0], f * gs[0]), w2 = fma(ds, v[1], f * gs[1]),
+                   w3 = fma(ds, v[2], f * gs[2]);
+            if (!first) {   // a second image within r_c adds to the first's
+              w0 += dst[0];
+              w1 += dst[Q];
+              w2 += dst[2 * Q];
+              w3 += dst[3 * Q];
+            }
+            dst[0] = w0;
+            dst[Q] = w1;
+            dst[2 * Q] = w2;
+            dst[3 * Q] = w3;
+          }
+          first = false;
+        }
+    if (first)
+      for (int c = 0; c < 4 * it.z; ++c) out[(int64_t)c * Q + q] = 0.0;
   }
 }
 
@@ -588,12 +664,21 @@ static Mat3 jit_of(const pufe_ctx *ctx) {
 }
 
 pufe_status launch_tabulate(pufe_ctx *ctx, cudaStream_t st) {
-  if (ctx->psi_len == 0) return PUFE_OK;
+  if (ctx->n_kitems == 0) return PUFE_OK;
   auto &D = ctx->d;
-  k_tabulate<<<(unsigned)ctx->nelem, 128, 0, st>>>(D.qoff, D.x, D.aoff, D.alist, D.toff, D.orb,
-                                                   ctx->a[0], ctx->a[1], ctx->a[2],
-                                                   ctx->images[0], ctx->images[1], ctx->images[2],
-                                                   D.psi, ctx->general ? 1 : 0, lattice_of(ctx));
+  LatticeDev lat = lattice_of(ctx);
+  double bn[3];   // inverse distances of the lattice planes
+  for (int k = 0; k < 3; ++k) {
+    if (!ctx->general) {
+      lat.L[4 * k] = ctx->a[k];
+      lat.Lit[4 * k] = 1.0 / ctx->a[k];
+    }
+    bn[k] = sqrt(lat.Lit[3 * k] * lat.Lit[3 * k] + lat.Lit[3 * k + 1] * lat.Lit[3 * k + 1] +
+                 lat.Lit[3 * k + 2] * lat.Lit[3 * k + 2]);
+  }
+  k_tabulate<<<(unsigned)ctx->n_kitems, TAB64_NT, 0, st>>>(
+      reinterpret_cast<const int4 *>(D.kitems), D.qoff, D.x, D.aoff, D.alist, D.toff, D.orb, lat,
+      bn[0], bn[1], bn[2], ctx->general ? 1 : 0, D.psi);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }

@@ -108,6 +108,8 @@ struct DeviceArrays {
   // functions at the tricubic nodes (64 x 32, serendipity space only)
   int32_t *jitems = nullptr, *dunits = nullptr;
   double *Rser = nullptr;
+  // FP64 tabulation: (element, first slot, slots of one atom, first point) items
+  int32_t *kitems = nullptr;
   // mixed-path work list of the n_e > 128 elements, 3 per item (index into
   // `order`, first chunk, end chunk; chunks of 8 padded points), largest first
   int32_t *titems = nullptr;
@@ -157,6 +159,7 @@ struct pufe_ctx {
   int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
   int asm64_work = 0;         // doubles of its shared work area
   int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
+  int n_kitems = 0;           // items of the FP64 tabulation
   int n_dunits = 0;           // units of the FP64 density (0: direct form)
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
@@ -197,6 +200,8 @@ namespace pufe {
 __host__ __device__ inline bool adjoint_sf_fits(int A, int pmax) { return A <= 16 && pmax <= 10; }
 // (slot, padded point) items of the FP32 enrichment table per tabulation CTA
 constexpr int TAB_CHUNK = 2048;
+// points of one FP64 tabulation item
+constexpr int TAB64_CHUNK = 128;
 // Shared-memory stage of the E-E overlap kernel (floats): elements whose
 // slots' Psi values on one (sub)cell exceed it take the Gram form instead
 constexpr int SEE_STAGE_MAX_F = 8192;

@@ -1566,6 +1566,24 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
     sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
     pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits);
   }
+  // FP64 tabulation: runs of slots with one atom and cutoff, in chunks of points
+  std::vector<int32_t> kitems;
+  for (int64_t e = 0; e < nelem; ++e) {
+    const std::vector<int> &al = ealpha[e];
+    for (size_t a = 0; a < al.size();) {
+      const Orbital &o = S.orb[al[a]];
+      size_t b = a + 1;
+      for (; b < al.size(); ++b) {
+        const Orbital &u = S.orb[al[b]];
+        if (u.tau[0] != o.tau[0] || u.tau[1] != o.tau[1] || u.tau[2] != o.tau[2] || u.rc != o.rc)
+          break;
+      }
+      for (int32_t q = 0; q < q_e[e]; q += TAB64_CHUNK)
+        kitems.insert(kitems.end(), {(int32_t)e, (int32_t)a, (int32_t)(b - a), q});
+      a = b;
+    }
+  }
+  ctx->n_kitems = (int)(kitems.size() / 4);
   ctx->n_aitems = (int)(aitems.size() / 6);
   ctx->n_jitems = (int)(jitems.size() / 6);
   ctx->n_dunits = (int)(dunits.size() / 4);
@@ -1600,6 +1618,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   if ((st = upload(&D.order, order)) != PUFE_OK) return st;
   if (!wsplit.empty() && (st = upload(&D.wsplit, wsplit)) != PUFE_OK) return st;
   if (!aitems.empty() && (st = upload(&D.aitems, aitems)) != PUFE_OK) return st;
+  if (!kitems.empty() && (st = upload(&D.kitems, kitems)) != PUFE_OK) return st;
   if (!jitems.empty() && (st = upload(&D.jitems, jitems)) != PUFE_OK) return st;
   if (!dunits.empty() && (st = upload(&D.dunits, dunits)) != PUFE_OK) return st;
   if (ser) {
@@ -1663,7 +1682,7 @@ static void free_device(pufe_ctx *ctx) {
   void *ptrs[] = {D.qoff, D.x, D.w, D.xi, D.doff, D.dofs, D.ecol, D.eshift, D.aoff, D.alist,
                   D.toff, D.psi, D.psi32, D.qpoff, D.qdat, D.ptab, D.vpad, D.toff32, D.eorig,
                   D.Tfe, D.Sfe, D.S0, D.partoff, D.part_p, D.part_q,
-                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems, D.jitems, D.dunits, D.Rser,
+                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems, D.jitems, D.dunits, D.Rser, D.kitems,
                   D.titems, D.sitems, D.gitems32, D.gitems64, D.citems, D.pitems, D.tblk, D.eeform, D.err};
   for (void *p : ptrs)
     if (p) cudaFree(p);

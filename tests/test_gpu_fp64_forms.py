@@ -2,7 +2,8 @@
 FP64 oracle: the smallest and largest points per axis (4 and 16) that the
 factorized assembly takes and the 3 that it leaves to the direct kernel, one
 element (every node repeated by periodicity), slots of one vertex column (the
-direct enrichment blocks) and of eight (the pair form), one state, an odd count
+direct enrichment blocks) and of eight (the pair form), several images of an atom
+within its cutoff (the tabulation's sum), one state, an odd count
 and the most that a call takes.  Tolerance 1e-12 of the
 largest entry, as in the other FP64 parity tests."""
 import math
@@ -27,6 +28,8 @@ CELLS = {
     "one_vertex_slots": lambda: W.small_two_atom(nel=3, quad_p=6, r_e=0.5),
     # (an even order: an odd one puts a point on the nucleus, where the oracle's
     # direction cosines are 0/0)
+    # several periodic images within r_c of a point
+    "images": lambda: W.small_two_atom(nel=2, a=2.0, quad_p=4, r_c=1.9, r_e=1.0),
     "wide_support": lambda: W.small_two_atom(nel=3, quad_p=6, r_c=1.9, r_e=1.9),
 }
 
