@@ -180,6 +180,42 @@ pufe_status pufe_assemble_HV_adjoint_bloch(pufe_ctx *ctx, const double *k, const
   return launch_adjoint_fp64_bloch(ctx, ph, Hbar_re, Hbar_im, Vbar, (cudaStream_t)stream);
 }
 
+// N r^l Y_lm (l <= 3; real, as solid_harmonic) as at most three monomials
+static void projector_terms(int l, int m, double N, ProjDev &d) {
+  struct Mono {
+    double c;
+    int x, y, z;
+  };
+  const double c1 = 0.48860251190291992;                            // sqrt(3 / (4 pi))
+  const double a = 1.0925484305920792, b = 0.31539156525252005;     // sqrt(15/pi)/2, sqrt(5/pi)/4
+  const double g = 0.59004358992664352, e = 2.8906114426405538;     // sqrt(35/2pi)/4, sqrt(105/pi)/2
+  const double f = 0.45704579946446572, h = 0.37317633259011540;    // sqrt(21/2pi)/4, sqrt(7/pi)/4
+  const std::vector<Mono> t[4][7] = {
+      {{{0.28209479177387814, 0, 0, 0}}},
+      {{{c1, 0, 1, 0}}, {{c1, 0, 0, 1}}, {{c1, 1, 0, 0}}},
+      {{{a, 1, 1, 0}},
+       {{a, 0, 1, 1}},
+       {{2 * b, 0, 0, 2}, {-b, 2, 0, 0}, {-b, 0, 2, 0}},
+       {{a, 1, 0, 1}},
+       {{a / 2, 2, 0, 0}, {-a / 2, 0, 2, 0}}},
+      {{{3 * g, 2, 1, 0}, {-g, 0, 3, 0}},
+       {{e, 1, 1, 1}},
+       {{4 * f, 0, 1, 2}, {-f, 2, 1, 0}, {-f, 0, 3, 0}},
+       {{2 * h, 0, 0, 3}, {-3 * h, 2, 0, 1}, {-3 * h, 0, 2, 1}},
+       {{4 * f, 1, 0, 2}, {-f, 3, 0, 0}, {-f, 1, 2, 0}},
+       {{e / 2, 2, 0, 1}, {-e / 2, 0, 2, 1}},
+       {{g, 3, 0, 0}, {-3 * g, 1, 2, 0}}}};
+  const std::vector<Mono> &v = t[l][m + l];
+  d.nterm = (int)v.size();
+  for (int u = 0; u < 3; ++u) {
+    const bool on = u < d.nterm;
+    d.coef[u] = on ? N * v[u].c : 0.0;
+    d.pw[u][0] = on ? v[u].x : 0;
+    d.pw[u][1] = on ? v[u].y : 0;
+    d.pw[u][2] = on ? v[u].z : 0;
+  }
+}
+
 // checks the projector list and copies it to the device (blocking copy)
 static pufe_status upload_projectors(pufe_ctx *ctx, int nproj, const pufe_projector *proj) {
   if (nproj < 1 || nproj > 64 || !proj) return fail(PUFE_EINVAL, "need 1 <= nproj <= 64 and proj");
@@ -190,10 +226,9 @@ static pufe_status upload_projectors(pufe_ctx *ctx, int nproj, const pufe_projec
       return fail(PUFE_EINVAL, "projector needs 0 <= l <= 3, |m| <= l, r_p > 0");
     ProjDev d;
     for (int c = 0; c < 3; ++c) d.tau[c] = q.tau[c];
-    d.l = q.l;
-    d.m = q.m;
     d.rp = q.r_p;
-    d.N = std::sqrt(2.0 / (std::tgamma(q.l + 1.5) * std::pow(q.r_p, 2 * q.l + 3)));
+    const double N = std::sqrt(2.0 / (std::tgamma(q.l + 1.5) * std::pow(q.r_p, 2 * q.l + 3)));
+    projector_terms(q.l, q.m, N, d);
     d.rcut = q.r_p * std::sqrt(2.0 * 20.0 * std::log(10.0));   // Gaussian below 1e-20
     pd[p] = d;
   }

@@ -421,12 +421,12 @@ pufe_status launch_tabulate(pufe_ctx *ctx, cudaStream_t s);
 pufe_status launch_density_fp64(pufe_ctx *ctx, const double *C, int64_t ldc, const double *f,
                                 int nocc, double *rho, cudaStream_t s);
 pufe_status launch_adjoint_fp64(pufe_ctx *ctx, const double *Hbar, double *Vbar, cudaStream_t s);
-// Gaussian nonlocal projector on the device: N r^l exp(-r^2/(2 rp^2)) Y_lm,
-// images within rcut
+// Gaussian nonlocal projector on the device: N r^l Y_lm exp(-r^2/(2 rp^2)) as
+// sum_u coef_u x^pw[u][0] y^pw[u][1] z^pw[u][2] exp(...), images within rcut per axis
 struct ProjDev {
   double tau[3];
-  double rp, N, rcut;
-  int l, m;
+  double rp, rcut, coef[3];
+  int nterm, pw[3][3];
 };
 // k == nullptr: Gamma point, F real; else F + i Fi at wavevector k
 pufe_status launch_projections(pufe_ctx *ctx, const ProjDev *pj, int P, const double *k, double *F,

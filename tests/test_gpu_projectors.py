@@ -105,3 +105,26 @@ def test_bloch_projections_match_oracle(name):
     ctx.pufe_sync_status()
     assert np.abs(Fi.cpu().numpy()).max() == 0.0
     assert np.abs(Fr.cpu().numpy() - F0.cpu().numpy()).max() < 1e-14 * np.abs(Fo).max()
+
+
+@pytest.mark.parametrize("quad_p,nel", [(1, 2), (3, 2), (16, 1)])
+def test_every_harmonic_at_the_edges_of_the_rules(quad_p, nel):
+    """All (l, m) up to l = 3 (each a sum of up to three products of 1D
+    functions), one to 16 points per axis, a projector count that is no multiple
+    of a CTA's group, at the Gamma point and at a wavevector; 1e-12 as above."""
+    wl = W.small_two_atom(nel=nel, quad_p=quad_p)
+    m = omesh.Mesh(wl)
+    rules = oq.all_rules(m)
+    ctx = pufe.pufe_build_mesh(wl)
+    ctx.pufe_tabulate(pufe.PUFE_FP64)
+    ps = [dict(tau=wl["atoms"][(l + m_) % 2][1], l=l, m=m_, rp=0.5 + 0.1 * l)
+          for l in range(4) for m_ in range(-l, l + 1)] + [dict(tau=(0.3, 1.1, 2.0), l=0, m=0, rp=0.9)]
+    F, G, Gi = (torch.full((ctx.n_dof, len(ps)), 3.0, dtype=torch.float64, device="cuda:0")
+                for _ in range(3))
+    k = 2.0 * np.pi / wl["a"] * np.array([0.3, -0.2, 0.1])
+    ctx.pufe_nonlocal_projections(ps, F)
+    ctx.pufe_nonlocal_projections_bloch(k, ps, (G, Gi))
+    ctx.pufe_sync_status()
+    Fo, Go = onl.projections(m, rules, ps), onl.projections_k(m, rules, ps, k)
+    assert np.abs(F.cpu().numpy() - Fo).max() < 1e-12 * np.abs(Fo).max()
+    assert np.abs(G.cpu().numpy() + 1j * Gi.cpu().numpy() - Go).max() < 1e-12 * np.abs(Go).max()
