@@ -1,7 +1,6 @@
 // FP64 CUDA-core kernels of the PUFE hot path:
 //   K0  enrichment tabulation (Sec. 5.1, eqs. Psitilde/Psi)
 //   K1+K2+K3  element basis tile, contraction and scatter (Sec. 4, eq. disceig3d)
-//   K5  adjoint of V -> H (derivative of sum Hbar_ij H_ij with respect to V_q)
 //
 // The element basis (the FE columns -- 64 tricubic or 32 cubic serendipity
 // functions -- then phi_v^PU Psi_alpha columns) is rebuilt on chip from the reference coordinates of each quadrature point
@@ -16,7 +15,6 @@ namespace {
 
 constexpr int QC = 8;         // quadrature points per chunk
 constexpr int ASM_NT = 256;   // threads of the assembly kernel
-constexpr int ADJ_NT = 256;   // threads of the adjoint kernel
 
 __device__ __forceinline__ void set_err(unsigned *err, unsigned bit) { atomicOr(err, bit); }
 
@@ -390,117 +388,6 @@ __global__ void __launch_bounds__(ASM_NT) k_assemble_fp64(
   }
 }
 
-// ---------------------------------------------------------------------------
-// K5 (FP64): Vbar_q = w_q b_q^T Hbar_e b_q.  One CTA per work item (an
-// element, or the point range [qa, qb) of one, as in the assembly): the
-// element block Hbar_e is gathered into shared memory (or read through the
-// scatter map when it does not fit); per chunk of QC points the basis rows are
-// built in shared memory and each thread reduces one (q, i) pair over j.
-// ---------------------------------------------------------------------------
-// BLOCH: complex cotangent Hbar + i Hbi; the element block used is
-// Re(conj(Hbar) exp(i k.(R_j - R_i))) = Hbar pr + Hbi pi.
-template <bool BLOCH>
-__global__ void __launch_bounds__(ADJ_NT) k_adjoint_fp64(
-    const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
-    const double *__restrict__ w, const double *__restrict__ xi_all,
-    const int64_t *__restrict__ doff, const int32_t *__restrict__ ecol,
-    const int64_t *__restrict__ toff, const double *__restrict__ psi,
-    const int64_t *__restrict__ soff, const int32_t *__restrict__ smap,
-    const double *__restrict__ Hbar, int hs_in_smem, double *__restrict__ Vbar,
-    const uint8_t *__restrict__ eshift, PhaseTab ph, const double *__restrict__ Hbi,
-    const int32_t *__restrict__ wsplit, int nfe) {
-  extern __shared__ __align__(16) double smem[];
-  // work item: a whole element, or the point range [qa, qb) of one
-  const int e = wsplit ? wsplit[3 * blockIdx.x] : order[blockIdx.x];
-  const int64_t q0 = qoff[e];
-  const int Q = (int)(qoff[e + 1] - q0);
-  const int qa = wsplit ? max(wsplit[3 * blockIdx.x + 1], 0) : 0;
-  const int qb = wsplit ? min(wsplit[3 * blockIdx.x + 2], Q) : Q;
-  const int n = (int)(doff[e + 1] - doff[e]);
-  const int32_t *ec = ecol + (doff[e] - (int64_t)nfe * e);
-  const double *pe = psi + 4 * toff[e];
-  const int32_t *m = smap + soff[e];
-  double *Bc = smem;                 // QC x n
-  double *acc = Bc + QC * n;         // QC
-  Tab1D *tab = reinterpret_cast<Tab1D *>(acc + QC);
-  double *Hs = reinterpret_cast<double *>(tab + QC);  // n x n when it fits
-  // element entry (i, j) of the cotangent (phased real part for BLOCH)
-  auto hval = [&](int i, int j) -> double {
-    const int32_t sl = m[(int64_t)i * n + j];
-    if (!BLOCH) return Hbar[sl];
-    const int ci = eshift[doff[e] + i], cj = eshift[doff[e] + j];
-    double pr = 1.0, pim = 0.0;
-    if (ci != cj) {
-      pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
-      pim = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
-    }
-    return Hbar[sl] * pr + Hbi[sl] * pim;
-  };
-  if (hs_in_smem)
-    for (int k = threadIdx.x; k < n * n; k += ADJ_NT) Hs[k] = hval(k / n, k % n);
-  const double s[3] = {0, 0, 0};
-  for (int qc = qa; qc < qb; qc += QC) {
-    __syncthreads();
-    for (int k = threadIdx.x; k < QC * 3; k += ADJ_NT) {
-      const int qq = k / 3, d = k - 3 * qq;
-      const int q = qc + qq;
-      const double xv = (q < qb) ? xi_all[3 * (q0 + q) + d] : 0.0;
-      double L[4], dL[4];
-      lagrange3(xv, L, dL);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        tab[qq].L[d][c] = L[c];
-        tab[qq].dL[d][c] = dL[c];
-      }
-    }
-    if (threadIdx.x < QC) acc[threadIdx.x] = 0.0;
-    __syncthreads();
-    for (int k = threadIdx.x; k < QC * n; k += ADJ_NT) {
-      const int qq = k / n, c = k - qq * n;
-      const int q = qc + qq;
-      double b = 0, gx, gy, gz;
-      if (q < qb) {
-        if (c < nfe) {   // FE column: tricubic (64) or serendipity (32)
-          if (nfe == 64) {
-            fe_column(tab[qq], c, s, b, gx, gy, gz);
-          } else {
-            const double xq[3] = {xi_all[3 * (q0 + q)], xi_all[3 * (q0 + q) + 1],
-                                  xi_all[3 * (q0 + q) + 2]};
-            double g3[3];
-            serendipity32(c, xq, b, g3);
-          }
-        } else {
-          const int code = ec[c - nfe];
-          const int slot = code >> 3, lv = code & 7;
-          const double *pp = pe + (int64_t)slot * 4 * Q + q;
-          const double ps[4] = {pp[0], 0.0, 0.0, 0.0};
-          const double xq[3] = {xi_all[3 * (q0 + q)], xi_all[3 * (q0 + q) + 1],
-                                xi_all[3 * (q0 + q) + 2]};
-          pu_column(xq, lv, s, ps, b, gx, gy, gz);
-        }
-      }
-      Bc[k] = b;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < QC * n; k += ADJ_NT) {
-      const int qq = k / n, i = k - qq * n;
-      if (qc + qq >= qb) continue;
-      const double *brow = Bc + qq * n;
-      double t = 0.0;
-      if (hs_in_smem) {
-        const double *hr = Hs + (int64_t)i * n;
-        for (int j = 0; j < n; ++j) t = fma(hr[j], brow[j], t);
-      } else {
-        for (int j = 0; j < n; ++j) t = fma(hval(i, j), brow[j], t);
-      }
-      atomicAdd(acc + qq, brow[i] * t);
-    }
-    __syncthreads();
-    if (threadIdx.x < QC && qc + (int)threadIdx.x < qb)
-      Vbar[q0 + qc + threadIdx.x] = w[q0 + qc + threadIdx.x] * acc[threadIdx.x];
-  }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -602,20 +489,7 @@ pufe_status launch_density_fp64(pufe_ctx *ctx, const double *C, int64_t ldc, con
 }
 
 pufe_status launch_adjoint_fp64(pufe_ctx *ctx, const double *Hbar, double *Vbar, cudaStream_t st) {
-  if (ctx->n_jitems > 0) return launch_adjoint_sf64(ctx, nullptr, Hbar, nullptr, Vbar, st);
-  auto &D = ctx->d;
-  const int n = ctx->max_basis;
-  size_t sm = (size_t)QC * n * sizeof(double) + QC * sizeof(double) + QC * sizeof(Tab1D);
-  const size_t hs = (size_t)n * n * sizeof(double);
-  int in_smem = (sm + hs <= 200 * 1024) ? 1 : 0;
-  if (in_smem) sm += hs;
-  PUFE_CUDA_TRY(cudaFuncSetAttribute(k_adjoint_fp64<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_adjoint_fp64<false><<<fp64_items(ctx), ADJ_NT, sm, st>>>(
-      D.order, D.qoff, D.w, D.xi, D.doff, D.ecol, D.toff, D.psi, D.soff, D.smap, Hbar, in_smem,
-      Vbar, nullptr, PhaseTab{}, nullptr, D.wsplit, ctx->nfe_e);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
+  return launch_adjoint_sf64(ctx, nullptr, Hbar, nullptr, Vbar, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -650,20 +524,7 @@ pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const d
 
 pufe_status launch_adjoint_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Hr,
                                       const double *Hi, double *Vbar, cudaStream_t st) {
-  if (ctx->n_jitems > 0) return launch_adjoint_sf64(ctx, &ph, Hr, Hi, Vbar, st);
-  auto &D = ctx->d;
-  const int n = ctx->max_basis;
-  size_t sm = (size_t)QC * n * sizeof(double) + QC * sizeof(double) + QC * sizeof(Tab1D);
-  const size_t hs = (size_t)n * n * sizeof(double);
-  int in_smem = (sm + hs <= 200 * 1024) ? 1 : 0;
-  if (in_smem) sm += hs;
-  PUFE_CUDA_TRY(cudaFuncSetAttribute(k_adjoint_fp64<true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_adjoint_fp64<true><<<fp64_items(ctx), ADJ_NT, sm, st>>>(
-      D.order, D.qoff, D.w, D.xi, D.doff, D.ecol, D.toff, D.psi, D.soff, D.smap, Hr, in_smem,
-      Vbar, D.eshift, ph, Hi, D.wsplit, ctx->nfe_e);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
+  return launch_adjoint_sf64(ctx, &ph, Hr, Hi, Vbar, st);
 }
 
 }  // namespace pufe

@@ -86,8 +86,8 @@ struct DeviceArrays {
   float *psi32 = nullptr;     // per element [q/8][slot][comp][q%8]: 32-float blocks
   float *eorig = nullptr;     // per (element, slot): displacement of the element
                               // origin from the nearest atom image, hi[3], lo[3], 0, 0
-  double *Tfe = nullptr;      // 64 x 64: kinetic block of the tricubic functions (any element)
-  double *Sfe = nullptr;      // 64 x 64: overlap block of the tricubic functions (any element)
+  double *Tfe = nullptr;      // nfe x nfe: kinetic block of the FE functions (any element)
+  double *Sfe = nullptr;      // nfe x nfe: overlap block of the FE functions (any element)
   double *S0 = nullptr;       // nnz: overlap FE-FE constants summed over elements (mixed path)
   Orbital *orb = nullptr;     // n_alpha
   OrbitalF *orbf = nullptr;   // n_alpha

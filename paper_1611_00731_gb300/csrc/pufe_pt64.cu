@@ -57,7 +57,8 @@ struct Adj64 {
   const uint8_t *eshift;
   PhaseTab ph;
   double *out;
-  int work;
+  const double *Rser;   // serendipity space: nodal values 64 x 32 (nfe = 32)
+  int nfe, work;
 };
 
 // the element's cotangent entries (the phased real part at a wavevector)
@@ -99,8 +100,33 @@ __device__ void adj_fefe(const Adj64 &P, int e, int cb, int ce, double *sm) {
   const int tid = threadIdx.x;
   const CotElem<BLOCH> H = cot_elem<BLOCH>(P, e);
   double *C = sm, *X = sm + 1000;   // coefficients [z][y][x]; the gathered block, then the stages
+  if (P.nfe == 64) {
 #pragma unroll 4
-  for (int o = tid; o < 4096; o += P64_NT) X[o] = H(o >> 6, o & 63);
+    for (int o = tid; o < 4096; o += P64_NT) X[o] = H(o >> 6, o & 63);
+  } else {   // serendipity: R Hbar R^T, R the nodal values of its functions
+    double *Y = X + 4096;
+    for (int o = tid; o < 1024; o += P64_NT) X[o] = H(o >> 5, o & 31);
+    __syncthreads();
+    for (int o = tid; o < 2048; o += P64_NT) {
+      const int j = o >> 5, d = o & 31;
+      double s = 0.0;
+      for (int c = 0; c < 32; ++c) {
+        const double r = P.Rser[j * 32 + c];
+        if (r != 0.0) s = fma(r, X[c * 32 + d], s);
+      }
+      Y[o] = s;
+    }
+    __syncthreads();
+    for (int o = tid; o < 4096; o += P64_NT) {
+      const int j = o & 63, i = o >> 6;
+      double s = 0.0;
+      for (int c = 0; c < 32; ++c) {
+        const double r = P.Rser[j * 32 + c];
+        if (r != 0.0) s = fma(r, Y[i * 32 + c], s);
+      }
+      X[o] = s;
+    }
+  }
   __syncthreads();
   for (int o = tid; o < 1000; o += P64_NT) {
     const int x = o % 10, y = (o / 10) % 10, z = o / 100;
@@ -155,7 +181,9 @@ __device__ void adj_fefe(const Adj64 &P, int e, int cb, int ce, double *sm) {
 }
 
 // shared doubles of the FE x FE part and, per slot and per pair, of the others
-int adj_fefe_doubles(int p) { return 1000 + std::max(4096, 130 * p + 10 * p * p); }
+int adj_fefe_doubles(int p, bool ser) {
+  return 1000 + std::max(ser ? 6144 : 4096, 130 * p + 10 * p * p);
+}
 __host__ __device__ inline int adj_slot_doubles(int p) {
   const int ev = 25 * p + 5 * p * p;
   return 125 + (ev > 832 ? ev : 832);
@@ -166,11 +194,11 @@ template <bool BLOCH>
 __device__ void adj_slots(const Adj64 &P, int e, int s0, int s1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x, G = s1 - s0;
   const CotElem<BLOCH> H = cot_elem<BLOCH>(P, e);
-  const int nE = H.n - 64;
+  const int nE = H.n - P.nfe;
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   int *scol = reinterpret_cast<int *>(sm);   // [G][8]
   double *K = sm + 4 * G, *base = K + 125 * G;
   double *R = base, *X = R + 512 * G, *Y = R;   // [g][z 8][y 8][x 8] -> [g][zy][5] -> [g][z 8][25]
@@ -181,10 +209,25 @@ __device__ void adj_slots(const Adj64 &P, int e, int s0, int s1, int cb, int ce,
     if (c >= 0 && c < 8 * G) scol[c] = o;
   }
   __syncthreads();
+  if (P.nfe == 32) {   // serendipity: its 32 coefficients per vertex first
+    for (int o = tid; o < 256 * G; o += P64_NT) {
+      const int j = o & 31, r = scol[o >> 5];
+      X[o] = r < 0 ? 0.0 : H(32 + r, j) + H(j, 32 + r);
+    }
+    __syncthreads();
+  }
 #pragma unroll 4
-  for (int o = tid; o < 512 * G; o += P64_NT) {   // (vertex, FE function) coefficients
+  for (int o = tid; o < 512 * G; o += P64_NT) {   // (vertex, tricubic function) coefficients
     const int j = o & 63, gv = o >> 6, v = gv & 7, r = scol[gv];
-    const double c = r < 0 ? 0.0 : H(64 + r, j) + H(j, 64 + r);
+    double c = 0.0;
+    if (P.nfe == 64) {
+      if (r >= 0) c = H(64 + r, j) + H(j, 64 + r);
+    } else {
+      for (int k = 0; k < 32; ++k) {
+        const double w = P.Rser[j * 32 + k];
+        if (w != 0.0) c = fma(w, X[gv * 32 + k], c);
+      }
+    }
     const int x = (j & 3) + 4 * (v & 1), y = ((j >> 2) & 3) + 4 * ((v >> 1) & 1),
               z = (j >> 4) + 4 * (v >> 2);
     R[(gv >> 3) * 512 + (z * 8 + y) * 8 + x] = c;
@@ -270,11 +313,11 @@ template <bool BLOCH>
 __device__ void adj_pairs(const Adj64 &P, int e, int k0, int k1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x;
   const CotElem<BLOCH> H = cot_elem<BLOCH>(P, e);
-  const int nE = H.n - 64, A = P.aoff[e + 1] - P.aoff[e];
+  const int nE = H.n - P.nfe, A = P.aoff[e + 1] - P.aoff[e];
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   int *scol = reinterpret_cast<int *>(sm);   // [A][8]
   for (int o = tid; o < 8 * A; o += P64_NT) scol[o] = -1;
   __syncthreads();
@@ -306,8 +349,8 @@ __device__ void adj_pairs(const Adj64 &P, int e, int k0, int k1, int cb, int ce,
         if ((unsigned)cx > 1u || (unsigned)cy > 1u || (unsigned)cz > 1u) continue;
         const int r = scol[al * 8 + u], c = scol[be * 8 + (cx | (cy << 1) | (cz << 2))];
         if (r < 0 || c < 0) continue;
-        s += H(64 + r, 64 + c);
-        if (al != be) s += H(64 + c, 64 + r);
+        s += H(P.nfe + r, P.nfe + c);
+        if (al != be) s += H(P.nfe + c, P.nfe + r);
       }
       K[o] = s * (1.0 / 64.0);
     }
@@ -359,16 +402,16 @@ template <bool BLOCH>
 __device__ void adj_direct(const Adj64 &P, int e, int qa, int qb, double *sm) {
   const int tid = threadIdx.x;
   const CotElem<BLOCH> H = cot_elem<BLOCH>(P, e);
-  const int nE = H.n - 64, nent = nE * (nE + 1) / 2;
+  const int nE = H.n - P.nfe, nent = nE * (nE + 1) / 2;
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   double *Hs = sm, *B = sm + nent;
   for (int o = tid; o < nE * nE; o += P64_NT) {
     const int r = o / nE, c = o - r * nE;
     if (c > r) continue;
-    Hs[r * (r + 1) / 2 + c] = r == c ? H(64 + r, 64 + r) : H(64 + r, 64 + c) + H(64 + c, 64 + r);
+    Hs[r * (r + 1) / 2 + c] = r == c ? H(P.nfe + r, P.nfe + r) : H(P.nfe + r, P.nfe + c) + H(P.nfe + c, P.nfe + r);
   }
   const int QC = max(1, min(min((P.work - nent) / nE, P64_NT), qb - qa)), PG = P64_NT / QC;
   const int qq = tid % QC, grp = tid / QC;
@@ -566,7 +609,7 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
     std::stable_sort(L.begin(), L.end(), [](const Item &x, const Item &y) { return x.c > y.c; });
     for (const Item &i : L) out.insert(out.end(), i.v, i.v + width);
   };
-  if (!ctx->ser) {
+  {
     std::vector<double> cf(ne), cs(ne), cp(ne), cd(ne);
     double total = 0.0;
     for (int64_t e = 0; e < ne; ++e) {
@@ -578,7 +621,7 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
         cs[e] += 125 * d + 25 * d * d + 6 * d * d * d;
         cp[e] += 27 * d + 9 * d * d + 5 * d * d * d;
       }
-      const double nE = ctx->n_e[e] - 64, A = ctx->n_slot[e];
+      const double nE = ctx->n_e[e] - ctx->nfe_e, A = ctx->n_slot[e];
       cd[e] = (double)ctx->q_e[e] * (0.5 * nE * (nE + 1) + 5 * nE);
       total += cf[e] + A * cs[e] + std::min(0.5 * A * (A + 1) * cp[e], cd[e]);
     }
@@ -596,8 +639,8 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
     for (int64_t e = 0; e < ne; ++e) {
       int p = 1;
       for (int d : ctx->part_p_host[e]) p = std::max(p, d);
-      const int A = ctx->n_slot[e], np = A * (A + 1) / 2, nE = ctx->n_e[e] - 64;
-      adj_work = std::max(adj_work, adj_fefe_doubles(p));
+      const int A = ctx->n_slot[e], np = A * (A + 1) / 2, nE = ctx->n_e[e] - ctx->nfe_e;
+      adj_work = std::max(adj_work, adj_fefe_doubles(p, ctx->ser));
       cells(e, 0, 0, 0, cf[e], 30000.0);
       if (A == 0) continue;
       int G = std::max(1, std::min(A, (int)std::min(1e6, target / cs[e])));
@@ -675,6 +718,8 @@ pufe_status launch_adjoint_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double 
   P.eshift = D.eshift;
   if (ph) P.ph = *ph;
   P.out = Vbar;
+  P.Rser = D.Rser;
+  P.nfe = ctx->nfe_e;
   P.work = ctx->adj64_work;
   const size_t sm = (size_t)ctx->adj64_work * sizeof(double);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "element too large for the FP64 adjoint");

@@ -1060,8 +1060,20 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   int min_p = 1 << 30;
   for (auto &parts : rule)
     for (auto &pt : parts) min_p = std::min(min_p, pt.p);
-  // (the exact FE-FE constants serve the mixed path, which takes the tricubic space)
-  const bool fe_exact = min_p >= 4 && !ser;
+  const bool fe_exact = min_p >= 4;
+  std::vector<double> Rser;   // values of the serendipity functions at the tricubic nodes
+  if (ser) {
+    Rser.resize(64 * 32);
+    for (int j = 0; j < 64; ++j) {
+      const double nd[4] = {-1.0, -1.0 / 3.0, 1.0 / 3.0, 1.0};
+      const double xi[3] = {nd[j & 3], nd[(j >> 2) & 3], nd[j >> 4]};
+      double g[3];
+      for (int c = 0; c < 32; ++c) {
+        serendipity32(c, xi, Rser[32 * j + c], g);
+        if (std::fabs(Rser[32 * j + c]) < 1e-15) Rser[32 * j + c] = 0.0;   // zeros up to rounding
+      }
+    }
+  }
   std::vector<double> TF, SF, S0;
   if (fe_exact) {
     double M1[4][4] = {{0}}, K1[4][4] = {{0}}, D1[4][4] = {{0}};   // D1[a][b] = int L'_a L_b
@@ -1121,13 +1133,27 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
           TF[i * 64 + j] = 0.5 * S.detJ * t;
         }
     }
+    if (ser) {   // the serendipity functions in the tricubic ones: R^T X R
+      auto lift = [&](std::vector<double> &X) {
+        std::vector<double> Y(32 * 64, 0.0), Z(32 * 32, 0.0);
+        for (int c = 0; c < 32; ++c)
+          for (int j = 0; j < 64; ++j)
+            for (int k = 0; k < 64; ++k) Y[c * 64 + k] += Rser[j * 32 + c] * X[j * 64 + k];
+        for (int c = 0; c < 32; ++c)
+          for (int d = 0; d < 32; ++d)
+            for (int k = 0; k < 64; ++k) Z[c * 32 + d] += Y[c * 64 + k] * Rser[k * 32 + d];
+        X.swap(Z);
+      };
+      lift(SF);
+      lift(TF);
+    }
     // the overlap constants summed over the elements through the scatter map
     S0.assign(nnz, 0.0);
     for (int64_t e = 0; e < nelem; ++e) {
       const int n = n_e[e];
       const int32_t *m = &smap[soff[e]];
-      for (int i = 0; i < 64; ++i)
-        for (int j = 0; j < 64; ++j) S0[m[(int64_t)i * n + j]] += SF[i * 64 + j];
+      for (int i = 0; i < nfe_e; ++i)
+        for (int j = 0; j < nfe_e; ++j) S0[m[(int64_t)i * n + j]] += SF[i * nfe_e + j];
     }
   }
 
@@ -1621,19 +1647,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   if (!kitems.empty() && (st = upload(&D.kitems, kitems)) != PUFE_OK) return st;
   if (!jitems.empty() && (st = upload(&D.jitems, jitems)) != PUFE_OK) return st;
   if (!dunits.empty() && (st = upload(&D.dunits, dunits)) != PUFE_OK) return st;
-  if (ser) {
-    std::vector<double> R(64 * 32);
-    for (int j = 0; j < 64; ++j) {
-      const double nd[4] = {-1.0, -1.0 / 3.0, 1.0 / 3.0, 1.0};
-      const double xi[3] = {nd[j & 3], nd[(j >> 2) & 3], nd[j >> 4]};
-      double g[3];
-      for (int c = 0; c < 32; ++c) {
-        serendipity32(c, xi, R[32 * j + c], g);
-        if (std::fabs(R[32 * j + c]) < 1e-15) R[32 * j + c] = 0.0;   // zeros up to rounding
-      }
-    }
-    if ((st = upload(&D.Rser, R)) != PUFE_OK) return st;
-  }
+  if (ser && (st = upload(&D.Rser, Rser)) != PUFE_OK) return st;
   if (!titems.empty() && (st = upload(&D.titems, titems)) != PUFE_OK) return st;
   if (!sitems.empty() && (st = upload(&D.sitems, sitems)) != PUFE_OK) return st;
   if (!gitems32.empty() && (st = upload(&D.gitems32, gitems32)) != PUFE_OK) return st;

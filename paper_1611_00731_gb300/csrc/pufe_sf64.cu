@@ -1,5 +1,5 @@
-// FP64 assembly of H and S by sum factorization (orthorhombic cells, tricubic
-// space, rules of >= 4 points per axis on every (sub)cell).
+// FP64 assembly of H and S by sum factorization (rules of >= 4 points per axis on
+// every (sub)cell).
 //
 // What bounds it: GB300 issues two FP64 multiply-adds per clock and SM (1/64
 // of the FP32 rate), so a kernel of this kind is as fast as the number of FP64
@@ -40,6 +40,12 @@
 //    Elements whose slots hold few vertex columns take the direct products of
 //    their columns where those are fewer operations (sf64_work_list).
 //
+// General (triclinic) cells: the fields are (J^-1 grad Psi)_d and the metric
+// G = J^-1 J^-T replaces (2/h_d)^2; its off-diagonal terms pair a slope on one axis
+// with a slope on another, projections of w Psi (of A) that the same moments hold.
+// The serendipity functions are sums of tricubic ones (their nodal values, R), so
+// their rows are R^T times the tricubic rows.
+//
 // One launch over a work list of (element, kind, range) items, largest first:
 // FE x FE blocks, slot ranges, pair ranges and the direct blocks' point ranges,
 // cut so that the items of small meshes still fill the chip.  All blocks meet in
@@ -47,7 +53,8 @@
 //
 // Measured (kernel time, direct kernel before): 12^3 rocksalt cell 18.8 -> 1.37 ms,
 // CsCl-like 16^3 cell 23.7 -> 2.65 ms, two-atom 4^3 cell 1.72 -> 0.096 ms, eight
-// elements of 6^3 points 377 -> 33 us.
+// elements of 6^3 points 377 -> 33 us; triclinic serendipity 6^3 at a wavevector 1.15
+// -> 0.48 ms.
 #include <algorithm>
 
 #include "pufe_internal.h"
@@ -72,7 +79,12 @@ struct Asm64 {
   double *H, *Hi, *S, *Si;
   const uint8_t *eshift;
   PhaseTab ph;
-  double sc[3];   // 2 / h_d
+  // first and second order factors of the fields: orthorhombic cells 2 / h_d with
+  // the physical gradients; general cells (GEN) jit = J^-T, the fields
+  // (J^-1 grad Psi)_d and the metric G = J^-1 J^-T
+  double sc[3], jit[9], G[9];
+  const double *Rser;   // serendipity space: nodal values 64 x 32 (nfe = 32)
+  int nfe;
   int want, work;   // PUFE_WANT_* mask; doubles of the shared work area
   unsigned *err;
 };
@@ -190,13 +202,38 @@ __device__ void fefe_item(const Asm64 &P, int e, int cb, int ce, double *sm) {
   const int n = (int)(P.doff[e + 1] - P.doff[e]);
   const int32_t *m = P.smap + P.soff[e];
   const uint8_t *es = P.eshift + P.doff[e];
+  auto tri = [&](int i, int j) -> double {   // tricubic entry
+    return M[pidx64(i & 3, j & 3) * 100 + pidx64((i >> 2) & 3, (j >> 2) & 3) * 10 +
+             pidx64(i >> 4, j >> 4)];
+  };
+  double *Y = M + 1000;   // serendipity: R^T M (32 x 64), R the nodal values of its functions
+  if (P.nfe == 32 && h) {
+    for (int o = tid; o < 2048; o += A64_NT) {
+      const int c = o >> 6, k = o & 63;
+      double s = 0.0;
+      for (int j = 0; j < 64; ++j) {
+        const double r = P.Rser[j * 32 + c];
+        if (r != 0.0) s = fma(r, tri(j, k), s);
+      }
+      Y[o] = s;
+    }
+    __syncthreads();
+  }
   // the constants come with the element's first (sub)cell range; at the Gamma
   // point S starts as their sum, so only H is added
   const bool s = BLOCH && (P.want & PUFE_WANT_S) && cb == 0;
-  for (int o = tid; o < 4096; o += A64_NT) {
-    const int i = o >> 6, j = o & 63;
-    const double v = M[pidx64(i & 3, j & 3) * 100 + pidx64((i >> 2) & 3, (j >> 2) & 3) * 10 +
-                       pidx64(i >> 4, j >> 4)];
+  const int nf = P.nfe;
+  for (int o = tid; o < nf * nf; o += A64_NT) {
+    const int i = o / nf, j = o - i * nf;
+    double v = 0.0;
+    if (nf == 64) {
+      v = tri(i, j);
+    } else if (h) {
+      for (int k = 0; k < 64; ++k) {
+        const double r = P.Rser[k * 32 + j];
+        if (r != 0.0) v = fma(r, Y[i * 64 + k], v);
+      }
+    }
     add_entry<BLOCH>(P, m[i * n + j], h && cb == 0 ? P.Tfe[o] + v : v, s ? P.Sfe[o] : 0.0, h, s,
                      BLOCH ? es[i] : 0, BLOCH ? es[j] : 0);
   }
@@ -219,30 +256,50 @@ __device__ __forceinline__ void expand_m(const double *m, int st, double s, doub
 #pragma unroll
   for (int a = 0; a < 4; ++a) o[a] = fma(kappa1(a), om, (1.0 + s * node1(a)) * m[a * st]);
 }
-// adds sum_j L'_a(x_j) (cf (1 + s x_j) F_j + cs s S_j) to o[a]
+// adds sum_j L'_a(x_j) (cf (1 + s x_j) F_j + cs s S_j) to o[a]; general cells: with
+// x1, x2 their cross terms' moments, (1 + s x_j) (c1 x1_j + c2 x2_j) too
+template <bool GEN = false>
 __device__ __forceinline__ void expand_d(const double *F, int fst, const double *S, int sst,
-                                         double s, double cf, double cs, double o[4]) {
+                                         double s, double cf, double cs, double o[4],
+                                         const double *x1 = nullptr, int st1 = 0, double c1 = 0.0,
+                                         const double *x2 = nullptr, int st2 = 0, double c2 = 0.0) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const double g = fma(cf * (1.0 + s * node1(j)), F[j * fst], cs * s * S[j * sst]);
+    double t = cf * F[j * fst];
+    if (GEN) t = fma(c1, x1[j * st1], t);
+    if (GEN && x2) t = fma(c2, x2[j * st2], t);
+    const double g = fma(1.0 + s * node1(j), t, cs * s * S[j * sst]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) o[a] = fma(c_d1[a * 4 + j], g, o[a]);
+  }
+}
+// sum_j L'_a(x_j) (1 + s x_j) S_j
+__device__ __forceinline__ void slope_m(const double *S, int st, double s, double o[4]) {
+#pragma unroll
+  for (int a = 0; a < 4; ++a) o[a] = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const double g = (1.0 + s * node1(j)) * S[j * st];
 #pragma unroll
     for (int a = 0; a < 4; ++a) o[a] = fma(c_d1[a * 4 + j], g, o[a]);
   }
 }
 
 constexpr int FXE_MOM = 550;    // moments of a slot: S 125, V 125, Fx, Fy, Fz 100 each
-constexpr int FXE_EXP = 1616;   // doubles of the expansion's intermediates
+// doubles of the expansion's intermediates: orthorhombic, general cells' cross
+// terms, the serendipity space's tricubic rows of H and S
+constexpr int FXE_EXP = 1616, FXE_EXP_GEN = 1160, FXE_EXP_SER = 1024;
 constexpr int EXE_MOM = 162;    // moments of a slot pair
 
-template <bool BLOCH>
+template <bool BLOCH, bool GEN>
 __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x, G = s1 - s0;
   const bool h = (P.want & PUFE_WANT_H) != 0, ws = (P.want & PUFE_WANT_S) != 0;
-  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - 64;
+  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - P.nfe;
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   double *mom = sm;                                        // [G][550]
   int *scol = reinterpret_cast<int *>(mom + FXE_MOM * G);  // [G][8]
   double *base = mom + FXE_MOM * G + 4 * G;
@@ -287,8 +344,17 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
 #pragma unroll
         for (int u = 0; u < 5; ++u) a[u] = fma(fS, fk[u], a[u]);
         if (h) {
-          const double fV = fS * P.V[q], fx = w * ps[Q + p2 * qz], fy = w * ps[2 * Q + p2 * qz],
-                       fz = w * ps[3 * Q + p2 * qz];
+          const double fV = fS * P.V[q];
+          double fx = ps[Q + p2 * qz], fy = ps[2 * Q + p2 * qz], fz = ps[3 * Q + p2 * qz];
+          if (GEN) {   // J^-1 grad
+            const double gx = fx, gy = fy, gz = fz;
+            fx = P.jit[0] * gx + P.jit[3] * gy + P.jit[6] * gz;
+            fy = P.jit[1] * gx + P.jit[4] * gy + P.jit[7] * gz;
+            fz = P.jit[2] * gx + P.jit[5] * gy + P.jit[8] * gz;
+          }
+          fx *= w;
+          fy *= w;
+          fz *= w;
 #pragma unroll
           for (int u = 0; u < 5; ++u) {
             a[5 + u] = fma(fV, fk[u], a[5 + u]);
@@ -341,8 +407,16 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
   const uint8_t *es = P.eshift + P.doff[e];
   double *XS = base, *XFy = XS + 200, *XFz = XFy + 160, *R1 = XFz + 160;   // [z][y][x 8]
   double *YS = R1 + 200, *YFz = YS + 320, *R2 = YFz + 256;                 // [z][y 8][x 8]
-  const double c2[3] = {0.5 * P.sc[0], 0.5 * P.sc[1], 0.5 * P.sc[2]};
-  const double cc[3] = {c2[0] * P.sc[0], c2[1] * P.sc[1], c2[2] * P.sc[2]};
+  // general cells: D on x; its M on y; D on y of M on x; M on y of s_x L on x
+  double *XD = R2 + 320, *YXD = XD + 200, *YD = YXD + 320, *YXL = YD + 320;
+  double *HS = base + FXE_EXP + (GEN ? FXE_EXP_GEN : 0);   // serendipity: [H, S][vertex][64]
+  // 1/2 of the first and second order factors
+  const double c2[3] = {GEN ? 0.5 : 0.5 * P.sc[0], GEN ? 0.5 : 0.5 * P.sc[1],
+                        GEN ? 0.5 : 0.5 * P.sc[2]};
+  const double cc[3] = {GEN ? 0.5 * P.G[0] : c2[0] * P.sc[0], GEN ? 0.5 * P.G[4] : c2[1] * P.sc[1],
+                        GEN ? 0.5 * P.G[8] : c2[2] * P.sc[2]};
+  const double gxy = 0.5 * P.G[1], gxz = 0.5 * P.G[2], gyz = 0.5 * P.G[5];
+  const bool ser = P.nfe == 32;
   for (int g = 0; g < G; ++g) {
     const double *S = mom + g * FXE_MOM, *Vm = S + 125, *Fx = S + 250, *Fy = S + 350, *Fz = S + 450;
     const int *sc8 = scol + 8 * g;
@@ -365,6 +439,10 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
           expand_m(Vm + 5 * r, 1, s, o);
           expand_d(Fx + 4 * r, 1, S + 5 * r, 1, s, c2[0], cc[0], o);
           for (int a = 0; a < 4; ++a) R1[r * 8 + 4 * t + a] = o[a];
+          if (GEN) {
+            slope_m(S + 5 * r, 1, s, o);
+            for (int a = 0; a < 4; ++a) XD[r * 8 + 4 * t + a] = o[a];
+          }
         }
       } else if (h) {
         const bool y = r < 45;
@@ -384,8 +462,25 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
         for (int b = 0; b < 4; ++b) YS[z * 64 + (4 * t + b) * 8 + x] = o[b];
         if (h) {
           expand_m(R1 + z * 40 + x, 8, s, o);
-          expand_d(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, s, c2[1], cc[1], o);
-          for (int b = 0; b < 4; ++b) R2[z * 64 + (4 * t + b) * 8 + x] = o[b];
+          if (GEN) {
+            // s_x L_a on x: the moments of L_a themselves, signed
+            const double sx = x >> 2 ? 1.0 : -1.0, *xl = S + z * 25 + (x & 3);
+            expand_d<true>(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, s, c2[1], cc[1], o, xl, 5,
+                           gxy * sx);
+            for (int b = 0; b < 4; ++b) {
+              o[b] = fma(gxy * s, XD[z * 40 + b * 8 + x], o[b]);
+              R2[z * 64 + (4 * t + b) * 8 + x] = o[b];
+            }
+            expand_m(XD + z * 40 + x, 8, s, o);
+            for (int b = 0; b < 4; ++b) YXD[z * 64 + (4 * t + b) * 8 + x] = o[b];
+            slope_m(XS + z * 40 + x, 8, s, o);
+            for (int b = 0; b < 4; ++b) YD[z * 64 + (4 * t + b) * 8 + x] = o[b];
+            expand_m(xl, 5, s, o);
+            for (int b = 0; b < 4; ++b) YXL[z * 64 + (4 * t + b) * 8 + x] = sx * o[b];
+          } else {
+            expand_d(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, s, c2[1], cc[1], o);
+            for (int b = 0; b < 4; ++b) R2[z * 64 + (4 * t + b) * 8 + x] = o[b];
+          }
         }
       } else if (h) {
         expand_m(XFz + (z - 5) * 40 + x, 8, s, o);
@@ -395,36 +490,67 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
     __syncthreads();
     for (int it = tid; it < 128; it += A64_NT) {   // z and the scatter: (t_z, y 8, x 8)
       const int xy = it & 63, t = it >> 6, x = xy & 7, y = xy >> 3;
-      const int r = sc8[(x >> 2) | ((y >> 2) << 1) | (t << 2)];
+      const int v = (x >> 2) | ((y >> 2) << 1) | (t << 2), r = sc8[v];
       if (r < 0) continue;
       const double s = t ? 1.0 : -1.0;
       double so[4], ho[4] = {0, 0, 0, 0};
       expand_m(YS + xy, 64, s, so);
       if (h) {
         expand_m(R2 + xy, 64, s, ho);
-        expand_d(YFz + xy, 64, YS + xy, 64, s, c2[2], cc[2], ho);
+        if (GEN) {
+          const double sy = y >> 2 ? 1.0 : -1.0;
+          expand_d<true>(YFz + xy, 64, YS + xy, 64, s, c2[2], cc[2], ho, YXL + xy, 64, gxz,
+                         XS + (y & 3) * 8 + x, 40, gyz * sy);
+          for (int c = 0; c < 4; ++c)
+            ho[c] = fma(s, fma(gxz, YXD[c * 64 + xy], gyz * YD[c * 64 + xy]), ho[c]);
+        } else {
+          expand_d(YFz + xy, 64, YS + xy, 64, s, c2[2], cc[2], ho);
+        }
       }
       for (int c = 0; c < 4; ++c) {
-        const int i = (x & 3) + 4 * (y & 3) + 16 * c, j = 64 + r;
+        const int i = (x & 3) + 4 * (y & 3) + 16 * c;
+        if (ser) {
+          HS[v * 64 + i] = ho[c];
+          HS[512 + v * 64 + i] = so[c];
+          continue;
+        }
+        const int j = 64 + r;
         const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
         add_entry<BLOCH>(P, m[i * n + j], 0.125 * ho[c], 0.125 * so[c], h, ws, ci, cj);
         add_entry<BLOCH>(P, m[j * n + i], 0.125 * ho[c], 0.125 * so[c], h, ws, cj, ci);
       }
+    }
+    if (!ser) continue;
+    __syncthreads();
+    for (int it = tid; it < 256; it += A64_NT) {   // rows of the serendipity functions
+      const int v = it >> 5, i = it & 31, r = sc8[v];
+      if (r < 0) continue;
+      double hv = 0.0, sv = 0.0;
+      for (int k = 0; k < 64; ++k) {
+        const double w = P.Rser[k * 32 + i];
+        if (w == 0.0) continue;
+        hv = fma(w, HS[v * 64 + k], hv);
+        sv = fma(w, HS[512 + v * 64 + k], sv);
+      }
+      const int j = 32 + r;
+      const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
+      add_entry<BLOCH>(P, m[i * n + j], 0.125 * hv, 0.125 * sv, h, ws, ci, cj);
+      add_entry<BLOCH>(P, m[j * n + i], 0.125 * hv, 0.125 * sv, h, ws, cj, ci);
     }
   }
 }
 
 // ---- enrichment x enrichment block of the slot pairs [k0, k1) ------------------
 // z rows: A u (3), E u (3), B_x u, C_x u, B_y u, C_y u (3 each), B_z l, C_z l (2 each)
-template <bool BLOCH>
+template <bool BLOCH, bool GEN>
 __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, double *sm) {
   const int tid = threadIdx.x;
   const bool h = (P.want & PUFE_WANT_H) != 0, ws = (P.want & PUFE_WANT_S) != 0;
-  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - 64;
+  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - P.nfe;
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0), A = P.aoff[e + 1] - P.aoff[e];
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   const int32_t *m = P.smap + P.soff[e];
   const uint8_t *es = P.eshift + P.doff[e];
   int *scol = reinterpret_cast<int *>(sm);   // [A][8]
@@ -438,9 +564,12 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
   const int fit = max(1, avail / (22 * pmax * pmax + 60 * pmax + EXE_MOM + 1));
   const int nch = (k1 - k0 + fit - 1) / fit, npc = (k1 - k0 + nch - 1) / nch;
   const int nr1 = h ? 22 : 3, nr2 = h ? 60 : 9;
-  const double c2[3] = {0.5 * P.sc[0], 0.5 * P.sc[1], 0.5 * P.sc[2]};
-  // 1/8 (2/h_d)^2: one half times the quarter of <., 1>
-  const double cq[3] = {0.25 * c2[0] * P.sc[0], 0.25 * c2[1] * P.sc[1], 0.25 * c2[2] * P.sc[2]};
+  const double c2[3] = {GEN ? 0.5 : 0.5 * P.sc[0], GEN ? 0.5 : 0.5 * P.sc[1],
+                        GEN ? 0.5 : 0.5 * P.sc[2]};
+  // 1/8 (2/h_d)^2 (general cells: G_dd / 8): one half times the quarter of <., 1>
+  const double cq[3] = {GEN ? 0.125 * P.G[0] : 0.25 * c2[0] * P.sc[0],
+                        GEN ? 0.125 * P.G[4] : 0.25 * c2[1] * P.sc[1],
+                        GEN ? 0.125 * P.G[8] : 0.25 * c2[2] * P.sc[2]};
   for (int c0 = k0; c0 < k1; c0 += npc) {
     const int nc = min(npc, k1 - c0);
     double *mom = base;                                         // [nc][162]
@@ -489,13 +618,22 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
           a[1] = fma(fA, u1, a[1]);
           a[2] = fma(fA, u2, a[2]);
           if (h) {
-            const double a1 = pa[Q + z], a2 = pa[2 * Q + z], a3 = pa[3 * Q + z];
-            const double b1 = pb[Q + z], b2 = pb[2 * Q + z], b3 = pb[3 * Q + z];
+            double a1 = pa[Q + z], a2 = pa[2 * Q + z], a3 = pa[3 * Q + z];
+            double b1 = pb[Q + z], b2 = pb[2 * Q + z], b3 = pb[3 * Q + z];
             const double wa = w * a0, l0 = f[4 * p + qz], l1 = f[5 * p + qz];
             const double fE = fma(P.V[q], fA, 0.5 * w * fma(a1, b1, fma(a2, b2, a3 * b3)));
             a[3] = fma(fE, u0, a[3]);
             a[4] = fma(fE, u1, a[4]);
             a[5] = fma(fE, u2, a[5]);
+            if (GEN) {   // J^-1 grad
+              const double ax = a1, ay = a2, az = a3, bx = b1, by = b2, bz = b3;
+              a1 = P.jit[0] * ax + P.jit[3] * ay + P.jit[6] * az;
+              a2 = P.jit[1] * ax + P.jit[4] * ay + P.jit[7] * az;
+              a3 = P.jit[2] * ax + P.jit[5] * ay + P.jit[8] * az;
+              b1 = P.jit[0] * bx + P.jit[3] * by + P.jit[6] * bz;
+              b2 = P.jit[1] * bx + P.jit[4] * by + P.jit[7] * bz;
+              b3 = P.jit[2] * bx + P.jit[5] * by + P.jit[8] * bz;
+            }
             const double f4[4] = {wb * a1, wa * b1, wb * a2, wa * b2};
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -580,9 +718,27 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
         hv = fma(c2[1] * qy, M[90 + (kz * 2 + by) * 3 + kx], hv);
         hv = fma(c2[2] * pz, M[144 + (cz * 3 + ky) * 3 + kx], hv);
         hv = fma(c2[2] * qz, M[126 + (bz * 3 + ky) * 3 + kx], hv);
+        if (GEN) {
+          // 1/2 G_de s_d s'_e <A, l_b'd on d, l_be on e> for d != e, with
+          // l_t = (u_t + u_(t+1)) / 2
+          const double px[3] = {bx ? 1.0 : -1.0, by ? 1.0 : -1.0, bz ? 1.0 : -1.0};
+          const double pq[3] = {cx ? 1.0 : -1.0, cy ? 1.0 : -1.0, cz ? 1.0 : -1.0};
+          const int b3[3] = {bx, by, bz}, c3[3] = {cx, cy, cz}, k3[3] = {kx, ky, kz},
+                    st[3] = {1, 3, 9};
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+              if (d == f) continue;
+              const int o = 3 - d - f;
+              const double *q = M + k3[o] * st[o] + c3[d] * st[d] + b3[f] * st[f];
+              hv = fma(0.125 * P.G[3 * d + f] * px[d] * pq[f],
+                       q[0] + q[st[d]] + q[st[f]] + q[st[d] + st[f]], hv);
+            }
+        }
         hv *= 1.0 / 64.0;
       }
-      const int i = 64 + r, j = 64 + c;
+      const int i = P.nfe + r, j = P.nfe + c;
       const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
       add_entry<BLOCH>(P, m[i * n + j], hv, sv, h, ws, ci, cj);
       if (al != be) add_entry<BLOCH>(P, m[j * n + i], hv, sv, h, ws, cj, ci);
@@ -599,15 +755,15 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
 // reads are not what bounds it, and no lane works on a tile's padding.
 constexpr int EED_PER = 4;
 
-template <bool BLOCH>
+template <bool BLOCH, bool GEN>
 __device__ void eed_item(const Asm64 &P, int e, int qa, int qb, double *sm) {
   const int tid = threadIdx.x;
   const bool h = (P.want & PUFE_WANT_H) != 0, ws = (P.want & PUFE_WANT_S) != 0;
-  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - 64, nent = nE * (nE + 1) / 2;
+  const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - P.nfe, nent = nE * (nE + 1) / 2;
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
-  const int32_t *ec = P.ecol + (P.doff[e] - 64ll * e);
+  const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   const int32_t *m = P.smap + P.soff[e];
   const uint8_t *es = P.eshift + P.doff[e];
   const int QC = max(1, min((P.work - 2 * A64_NT) / (5 * nE), qb - qa));
@@ -644,9 +800,20 @@ __device__ void eed_item(const Asm64 &P, int e, int qa, int qb, double *sm) {
         const double yz = ly * lz, phi = lx * yz, v = ps[0], b = w1 * phi * v;
         double *o = X + qq * 5 * nE + j;
         if (h) {
-          o[0] = w2 * fma(phi, ps[Q], sx * P.sc[0] * yz * v);
-          o[nE] = w2 * fma(phi, ps[2 * Q], sy * P.sc[1] * lx * lz * v);
-          o[2 * nE] = w2 * fma(phi, ps[3 * Q], sz * P.sc[2] * lx * ly * v);
+          double dx = sx * yz, dy = sy * lx * lz, dz = sz * lx * ly;   // 8 grad_xi phi
+          if (GEN) {
+            const double gx = dx, gy = dy, gz = dz;
+            dx = P.jit[0] * gx + P.jit[1] * gy + P.jit[2] * gz;
+            dy = P.jit[3] * gx + P.jit[4] * gy + P.jit[5] * gz;
+            dz = P.jit[6] * gx + P.jit[7] * gy + P.jit[8] * gz;
+          } else {
+            dx *= P.sc[0];
+            dy *= P.sc[1];
+            dz *= P.sc[2];
+          }
+          o[0] = w2 * fma(phi, ps[Q], dx * v);
+          o[nE] = w2 * fma(phi, ps[2 * Q], dy * v);
+          o[2 * nE] = w2 * fma(phi, ps[3 * Q], dz * v);
           o[4 * nE] = P.V[q0 + q] * b;
         }
         o[3 * nE] = b;
@@ -688,7 +855,7 @@ __device__ void eed_item(const Asm64 &P, int e, int qa, int qb, double *sm) {
 #pragma unroll
     for (int u = 0; u < EED_PER; ++u) {
       if (r[u] < 0) continue;
-      const int i = 64 + r[u], j = 64 + c[u];
+      const int i = P.nfe + r[u], j = P.nfe + c[u];
       const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
       add_entry<BLOCH>(P, m[i * n + j], hs[u], ss[u], h, ws, ci, cj);
       if (i != j) add_entry<BLOCH>(P, m[j * n + i], hs[u], ss[u], h, ws, cj, ci);
@@ -696,7 +863,7 @@ __device__ void eed_item(const Asm64 &P, int e, int qa, int qb, double *sm) {
   }
 }
 
-template <bool BLOCH>
+template <bool BLOCH, bool GEN>
 __global__ void __launch_bounds__(A64_NT) k_assemble_sf64(Asm64 P) {
   extern __shared__ __align__(16) double sm64[];
   const int32_t *it = P.items + 6ll * blockIdx.x;
@@ -704,17 +871,21 @@ __global__ void __launch_bounds__(A64_NT) k_assemble_sf64(Asm64 P) {
   if (kind == 0)
     fefe_item<BLOCH>(P, e, cb, ce, sm64);
   else if (kind == 1)
-    fxe_item<BLOCH>(P, e, a, b, cb, ce, sm64);
+    fxe_item<BLOCH, GEN>(P, e, a, b, cb, ce, sm64);
   else if (kind == 2)
-    exe_item<BLOCH>(P, e, a, b, cb, ce, sm64);
+    exe_item<BLOCH, GEN>(P, e, a, b, cb, ce, sm64);
   else
-    eed_item<BLOCH>(P, e, a, b, sm64);
+    eed_item<BLOCH, GEN>(P, e, a, b, sm64);
 }
 
 // shared doubles of one item
-int fefe_doubles(int p) { return 1000 + 30 * p + 10 * p * p + 100 * p; }
-int fxe_doubles(int G, int p) {
-  return (FXE_MOM + 4) * G + std::max(FXE_EXP, 15 * p + G * (24 * p * p + 115 * p));
+int fefe_doubles(int p, bool ser) {
+  return 1000 + std::max(30 * p + 10 * p * p + 100 * p, ser ? 2048 : 0);
+}
+int fxe_doubles(int G, int p, bool gen, bool ser) {
+  return (FXE_MOM + 4) * G +
+         std::max(FXE_EXP + (gen ? FXE_EXP_GEN : 0) + (ser ? FXE_EXP_SER : 0),
+                  15 * p + G * (24 * p * p + 115 * p));
 }
 int exe_doubles(int A, int nc, int p) {
   return 4 * A + 18 * p + nc * (22 * p * p + 60 * p + EXE_MOM + 1);
@@ -753,7 +924,7 @@ static double ee_pair_ops(const std::vector<int32_t> &cells) {
 void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, int &work) {
   items.clear();
   work = 0;
-  if (ctx->general || ctx->ser || !ctx->fe_exact || ctx->max_part_p > 16) return;
+  if (!ctx->fe_exact || ctx->max_part_p > 16) return;
   const int64_t ne = (int64_t)ctx->n_e.size();
   struct Item {
     int32_t e, kind, a, b, cb, ce;
@@ -773,7 +944,7 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
     }
     const double A = ctx->n_slot[e], np = 0.5 * A * (A + 1);
     cp[e] = ee_pair_ops(ctx->part_p_host[e]);
-    cd[e] = ee_direct_ops(ctx->n_e[e] - 64, ctx->q_e[e]);
+    cd[e] = ee_direct_ops(ctx->n_e[e] - ctx->nfe_e, ctx->q_e[e]);
     total += cf[e] + A * cs[e] + std::min(np * cp[e], cd[e]);
   }
   const double target = std::max(1.0, total / (4.0 * nsm));
@@ -788,13 +959,13 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
                        (int)((int64_t)(j + 1) * nc / cuts), c / cuts});
   };
   for (int64_t e = 0; e < ne; ++e) {
-    const int A = ctx->n_slot[e], np = A * (A + 1) / 2, p = pm[e], nE = ctx->n_e[e] - 64;
+    const int A = ctx->n_slot[e], np = A * (A + 1) / 2, p = pm[e], nE = ctx->n_e[e] - ctx->nfe_e;
     cells(e, 0, 0, 0, cf[e], 40000.0);
-    work = std::max(work, fefe_doubles(p));
+    work = std::max(work, fefe_doubles(p, ctx->ser));
     if (A == 0) continue;
     int G = std::max(1, std::min(A, (int)std::min(1e6, target / cs[e])));
-    while (G > 1 && fxe_doubles(G, p) > A64_WORK) --G;
-    work = std::max(work, fxe_doubles(G, p));
+    while (G > 1 && fxe_doubles(G, p, ctx->general, ctx->ser) > A64_WORK) --G;
+    work = std::max(work, fxe_doubles(G, p, ctx->general, ctx->ser));
     for (int a = 0; a < A; a += G)
       cells(e, 1, a, std::min(A, a + G), cs[e] * std::min(G, A - a), 40000.0 * G);
     if (cd[e] < np * cp[e]) {
@@ -854,13 +1025,22 @@ pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double
   P.Si = Si;
   P.eshift = D.eshift;
   if (ph) P.ph = *ph;
-  for (int d = 0; d < 3; ++d) P.sc[d] = 2.0 / ctx->h[d];
+  for (int d = 0; d < 3 && !ctx->general; ++d) P.sc[d] = 2.0 / ctx->h[d];
+  if (ctx->general)
+    for (int d = 0; d < 3; ++d)
+      for (int c = 0; c < 3; ++c) {
+        P.jit[3 * d + c] = ctx->Jit[3 * d + c];
+        for (int r = 0; r < 3; ++r) P.G[3 * d + c] += ctx->Jit[3 * r + d] * ctx->Jit[3 * r + c];
+      }
+  P.Rser = D.Rser;
+  P.nfe = ctx->nfe_e;
   P.want = what;
   P.work = ctx->asm64_work;
   P.err = D.err;
   const size_t sm = (size_t)ctx->asm64_work * sizeof(double);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "element too large for the FP64 assembly");
-  auto kern = ph ? k_assemble_sf64<true> : k_assemble_sf64<false>;
+  auto kern = ph ? (ctx->general ? k_assemble_sf64<true, true> : k_assemble_sf64<true, false>)
+                 : (ctx->general ? k_assemble_sf64<false, true> : k_assemble_sf64<false, false>);
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   kern<<<(unsigned)ctx->n_aitems, A64_NT, sm, st>>>(P);
   PUFE_CUDA_TRY(cudaGetLastError());

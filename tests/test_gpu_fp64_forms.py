@@ -30,6 +30,14 @@ CELLS = {
     # direction cosines are 0/0)
     # several periodic images within r_c of a point
     "images": lambda: W.small_two_atom(nel=2, a=2.0, quad_p=4, r_c=1.9, r_e=1.0),
+    # general cells (the metric's cross terms) and the serendipity space (its rows
+    # lifted to the tricubic ones), alone and together, in both E x E forms
+    "triclinic": lambda: W.ceal_like(nel=2, quad_p=5),
+    "triclinic_wide": lambda: W.ceal_like(nel=3, quad_p=4, r_c=3.0, r_e=2.9),
+    "serendipity": lambda: dict(W.small_two_atom(nel=3, quad_p=6, r_c=1.9, r_e=1.9),
+                                fe="serendipity32"),
+    "triclinic_serendipity": lambda: dict(W.ceal_like(nel=2, quad_p=9), fe="serendipity32"),
+    "serendipity_p3": lambda: dict(W.small_two_atom(nel=2, quad_p=3), fe="serendipity32"),
     "wide_support": lambda: W.small_two_atom(nel=3, quad_p=6, r_c=1.9, r_e=1.9),
 }
 
@@ -74,7 +82,7 @@ def test_assembly(cell):
 
 def test_assembly_at_a_wavevector(cell):
     wl, m, rules, ctx = cell
-    k = 2.0 * math.pi / wl["a"] * np.array([0.3, -0.2, 0.1])
+    k = 2.0 * math.pi / (wl["a"] or W.CEAL_A) * np.array([0.3, -0.2, 0.1])
     V = W.random_potential(ctx.n_q, seed=6)
     Ho, So = ob.assemble_HS_k(m, rules, V, k)
     mk = lambda: torch.full((ctx.nnz,), 3.0, dtype=torch.float64, device="cuda:0")
@@ -108,7 +116,7 @@ def test_adjoint(cell):
 
 def test_density_and_adjoint_at_a_wavevector(cell):
     wl, m, rules, ctx = cell
-    k = 2.0 * math.pi / wl["a"] * np.array([0.3, -0.2, 0.1])
+    k = 2.0 * math.pi / (wl["a"] or W.CEAL_A) * np.array([0.3, -0.2, 0.1])
     Cr, Ci = (W.random_coefficients(ctx.n_dof, 7, seed=s) for s in (1, 2))
     f = W.random_occupations(7, seed=3)
     hr, hi = (W.random_symmetric_values(ctx.nnz, seed=s) for s in (4, 5))
