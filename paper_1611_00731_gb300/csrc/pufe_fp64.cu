@@ -33,8 +33,8 @@ __device__ __forceinline__ void set_err(unsigned *err, unsigned bit) { atomicOr(
 // one or two per axis instead of 27 in all.  On the 12^3 rocksalt cell that is
 // about 40 operations per value in place of 400, and the elements of 30 slots and
 // 4,096 points of the CsCl-like cell spread over 32 CTAs each instead of one.
-// Measured: 12^3 rocksalt 2.19 -> 0.21 ms, CsCl-like 16^3 30.3 -> 0.26 ms, two-atom
-// 4^3 377 -> 30 us.
+// Measured: 12^3 rocksalt 2.19 -> 0.19 ms, CsCl-like 16^3 30.3 -> 0.26 ms, two-atom
+// 4^3 377 -> 28 us.
 // ---------------------------------------------------------------------------
 constexpr int TAB64_NT = 128;
 
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(TAB64_NT) k_tabulate(
     const int4 *__restrict__ items, const int64_t *__restrict__ qoff,
     const double *__restrict__ x, const int32_t *__restrict__ aoff,
     const int32_t *__restrict__ alist, const int64_t *__restrict__ toff,
-    const Orbital *__restrict__ orb, LatticeDev lat, double b0, double b1, double b2, int gen,
+    const Orbital *__restrict__ orb, LatticeDev lat, float b0, float b1, float b2, int gen,
     double *__restrict__ psi) {
   const int4 it = items[blockIdx.x];   // element, first slot, slots, first point
   const int64_t e = it.x, q0 = qoff[e];
@@ -52,7 +52,8 @@ __global__ void __launch_bounds__(TAB64_NT) k_tabulate(
   double *out = psi + 4 * toff[e] + (int64_t)it.y * 4 * Q;
   for (int q = it.w + threadIdx.x; q < min(it.w + TAB64_CHUNK, Q); q += TAB64_NT) {
     const Orbital &o0 = orb[al[0]];   // the atom and the cutoff of the run
-    const double rc = o0.rc, irc = 1.0 / rc, bn[3] = {b0, b1, b2};
+    const double rc = o0.rc, irc = o0.inv_rc, rc2 = rc * rc;
+    const float bn[3] = {b0, b1, b2};
     double d[3], s[3];
     int lo[3], hi[3];
 #pragma unroll
@@ -61,9 +62,10 @@ __global__ void __launch_bounds__(TAB64_NT) k_tabulate(
     for (int k = 0; k < 3; ++k) {
       s[k] = gen ? lat.Lit[3 * k] * d[0] + lat.Lit[3 * k + 1] * d[1] + lat.Lit[3 * k + 2] * d[2]
                  : d[k] * lat.Lit[4 * k];
-      const double reach = rc * bn[k] * (1.0 + 1e-9);
-      lo[k] = (int)ceil(-reach - s[k]);
-      hi[k] = (int)floor(reach - s[k]);
+      // (in FP32, with a margin that covers its rounding; r < r_c decides below)
+      const float reach = (float)rc * bn[k] * 1.0001f + 1e-4f, sf = (float)s[k];
+      lo[k] = (int)ceilf(-reach - sf);
+      hi[k] = (int)floorf(reach - sf);
     }
     bool first = true;
     for (int i = lo[0]; i <= hi[0]; ++i)
@@ -80,9 +82,10 @@ __global__ void __launch_bounds__(TAB64_NT) k_tabulate(
             v[2] = d[2] + k * lat.L[8];
           }
           const double r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-          if (r2 >= rc * rc) continue;
-          const double r = sqrt(r2), t = r * irc, t3 = t * t * t, om = 1.0 - t;
-          const double ir = r > 1e-14 ? 1.0 / r : 0.0;
+          if (r2 >= rc2) continue;
+          // one reciprocal square root for r and 1 / r (0 at the nucleus)
+          const double ir = r2 > 1e-28 ? rsqrt(r2) : 0.0;
+          const double r = r2 > 1e-28 ? r2 * ir : sqrt(r2), t = r * irc, t3 = t * t * t, om = 1.0 - t;
           const double hc = 1.0 + t3 * t * (-35.0 + t * (84.0 + t * (-70.0 + 20.0 * t)));
           const double dh = -140.0 * irc * t3 * om * om * om;
           double zeta = -1.0, ex = 0.0, f = 0.0, df = 0.0;
@@ -432,7 +435,7 @@ pufe_status launch_tabulate(pufe_ctx *ctx, cudaStream_t st) {
   }
   k_tabulate<<<(unsigned)ctx->n_kitems, TAB64_NT, 0, st>>>(
       reinterpret_cast<const int4 *>(D.kitems), D.qoff, D.x, D.aoff, D.alist, D.toff, D.orb, lat,
-      bn[0], bn[1], bn[2], ctx->general ? 1 : 0, D.psi);
+      (float)bn[0], (float)bn[1], (float)bn[2], ctx->general ? 1 : 0, D.psi);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
@@ -444,8 +447,8 @@ static unsigned fp64_items(const pufe_ctx *ctx) {
 }
 
 // FP64 assembly into caller arrays: H (and Hi, Si at a wavevector, ph != nullptr)
-// zeroed here, S too -- or, on the sum-factorized path at the Gamma point, set
-// to the constant FE-FE overlap that path does not add
+// zeroed here, S too -- or, on the sum-factorized path, set to the constant FE-FE
+// overlap that path does not add
 pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
                                  double *H, double *Hi, double *S, double *Si, cudaStream_t st) {
   auto &D = ctx->d;
@@ -458,14 +461,11 @@ pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double
     if (ph) PUFE_CUDA_TRY(cudaMemsetAsync(Hi, 0, bytes, st));
   }
   if (what & PUFE_WANT_S) {
-    if (ph) {
-      PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
-      PUFE_CUDA_TRY(cudaMemsetAsync(Si, 0, bytes, st));
-    } else if (ctx->n_aitems > 0) {
+    if (ctx->n_aitems > 0)
       PUFE_CUDA_TRY(cudaMemcpyAsync(S, D.S0, bytes, cudaMemcpyDeviceToDevice, st));
-    } else {
+    else
       PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
-    }
+    if (ph) PUFE_CUDA_TRY(cudaMemsetAsync(Si, 0, bytes, st));
   }
   if (ctx->n_aitems > 0) return launch_assemble_sf64(ctx, ph, V, what, H, Hi, S, Si, st);
   auto kern = ph ? (ctx->general ? k_assemble_fp64<true, true> : k_assemble_fp64<true, false>)

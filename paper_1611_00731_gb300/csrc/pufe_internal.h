@@ -41,6 +41,7 @@ struct Orbital {
   double zeta;     // Slater exponent
   double norm;     // STO normalisation (2 zeta)^(n+1/2) / sqrt((2n)!)
   double rc;       // cutoff radius
+  double inv_rc;   // 1 / rc
   int n, l, m;
   int pad;
 };
@@ -108,6 +109,9 @@ struct DeviceArrays {
   // functions at the tricubic nodes (64 x 32, serendipity space only)
   int32_t *jitems = nullptr, *dunits = nullptr;
   double *Rser = nullptr;
+  // the same by function: node and value lists, rser_len per function
+  int32_t *rser_i = nullptr;
+  double *rser_v = nullptr;
   // FP64 tabulation: (element, first slot, slots of one atom, first point) items
   int32_t *kitems = nullptr;
   // mixed-path work list of the n_e > 128 elements, 3 per item (index into
@@ -159,12 +163,14 @@ struct pufe_ctx {
   int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
   int asm64_work = 0;         // doubles of its shared work area
   int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
+  int rser_len = 0;           // entries per serendipity function in rser_i, rser_v
   int n_kitems = 0;           // items of the FP64 tabulation
   int n_dunits = 0;           // units of the FP64 density (0: direct form)
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
   int n_gitems32 = 0, n_gitems64 = 0;   // items of the Gram-form lists
   int n_citems = 0;           // items of the strip kernel's list ((sub)cell ranges)
+  bool citems_cut = false;    // some element of that list is cut into several ranges
   int n_pitems = 0;           // items of the FP32 per-point list (point ranges of every element)
   int n_tblk = 0;             // CTAs of the FP32 tabulation (TAB_CHUNK table items each)
   int max_part_p = 0;         // largest points-per-axis of any (sub)cell
@@ -415,6 +421,22 @@ __host__ __device__ inline void enrichment_eval(const Orbital &o, const double p
         orbital_accumulate<T>(o, T(d0[0] + i * a[0]), T(d0[1] + j * a[1]), T(d0[2] + k * a[2]),
                               psi, g);
 }
+
+#ifdef __CUDACC__
+// FP64 -> FP32, round to nearest even, on the integer pipe for values in the
+// normal FP32 range (GB300 converts on the FP64 pipe, two per clock and SM: the
+// 11,000 coefficients of an 87-function element of 64 complex states would take
+// it a third of the element's multiply-adds); the others take the conversion.
+__device__ __forceinline__ float f64_to_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  if (ex - 897u > 253u) return (hi << 1 | lo) ? (float)x : __uint_as_float(hi);
+  unsigned r = ((ex - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rem = lo & 0x1fffffffu;
+  r += (rem > 0x10000000u || (rem == 0x10000000u && (r & 1u))) ? 1u : 0u;
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+#endif
 
 // launchers implemented in the .cu files
 pufe_status launch_tabulate(pufe_ctx *ctx, cudaStream_t s);

@@ -107,6 +107,8 @@ __device__ void adj_fefe(const Adj64 &P, int e, int cb, int ce, double *sm) {
     double *Y = X + 4096;
     for (int o = tid; o < 1024; o += P64_NT) X[o] = H(o >> 5, o & 31);
     __syncthreads();
+    // (a warp works on one node, whose zeros it skips as a whole; R Hbar is kept
+    // transposed, [32][64], and the result too: the sums below take both halves)
     for (int o = tid; o < 2048; o += P64_NT) {
       const int j = o >> 5, d = o & 31;
       double s = 0.0;
@@ -114,15 +116,15 @@ __device__ void adj_fefe(const Adj64 &P, int e, int cb, int ce, double *sm) {
         const double r = P.Rser[j * 32 + c];
         if (r != 0.0) s = fma(r, X[c * 32 + d], s);
       }
-      Y[o] = s;
+      Y[d * 64 + j] = s;
     }
     __syncthreads();
     for (int o = tid; o < 4096; o += P64_NT) {
-      const int j = o & 63, i = o >> 6;
+      const int j = o >> 6, i = o & 63;
       double s = 0.0;
       for (int c = 0; c < 32; ++c) {
         const double r = P.Rser[j * 32 + c];
-        if (r != 0.0) s = fma(r, Y[i * 32 + c], s);
+        if (r != 0.0) s = fma(r, Y[c * 64 + i], s);
       }
       X[o] = s;
     }
@@ -210,22 +212,25 @@ __device__ void adj_slots(const Adj64 &P, int e, int s0, int s1, int cb, int ce,
   }
   __syncthreads();
   if (P.nfe == 32) {   // serendipity: its 32 coefficients per vertex first
-    for (int o = tid; o < 256 * G; o += P64_NT) {
-      const int j = o & 31, r = scol[o >> 5];
-      X[o] = r < 0 ? 0.0 : H(32 + r, j) + H(j, 32 + r);
+    for (int o = tid; o < 256 * G; o += P64_NT) {   // [function][slot, vertex]
+      const int j = o & 31, gv = o >> 5, r = scol[gv];
+      X[j * 8 * G + gv] = r < 0 ? 0.0 : H(32 + r, j) + H(j, 32 + r);
     }
     __syncthreads();
   }
 #pragma unroll 4
   for (int o = tid; o < 512 * G; o += P64_NT) {   // (vertex, tricubic function) coefficients
-    const int j = o & 63, gv = o >> 6, v = gv & 7, r = scol[gv];
+    // lanes along the functions of one vertex, or (serendipity) along the vertices
+    // of one node, whose nonzeros they share
+    const int j = P.nfe == 64 ? o & 63 : o / (8 * G), gv = P.nfe == 64 ? o >> 6 : o % (8 * G);
+    const int v = gv & 7, r = scol[gv];
     double c = 0.0;
     if (P.nfe == 64) {
       if (r >= 0) c = H(64 + r, j) + H(j, 64 + r);
     } else {
       for (int k = 0; k < 32; ++k) {
         const double w = P.Rser[j * 32 + k];
-        if (w != 0.0) c = fma(w, X[gv * 32 + k], c);
+        if (w != 0.0) c = fma(w, X[k * 8 * G + gv], c);
       }
     }
     const int x = (j & 3) + 4 * (v & 1), y = ((j >> 2) & 3) + 4 * ((v >> 1) & 1),

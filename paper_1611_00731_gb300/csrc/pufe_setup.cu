@@ -536,6 +536,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
       ob.m = sp.m[o];
       ob.zeta = sp.zeta[o];
       ob.rc = sp.r_c;
+      ob.inv_rc = 1.0 / sp.r_c;
       ob.norm = std::pow(2.0 * ob.zeta, ob.n + 0.5) / std::sqrt(factorial(2 * ob.n));
       ob.pad = 0;
       S.orb.push_back(ob);
@@ -1515,6 +1516,11 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
     }
   }
   ctx->n_citems = (int)(citems.size() / 3);
+  {
+    int64_t strip = 0;
+    for (int64_t e = 0; e < nelem; ++e) strip += n_e[e] > 64 && n_e[e] <= 128;
+    ctx->citems_cut = ctx->n_citems > strip;
+  }
 
   // Work list of the FP32 per-point kernels (density; adjoint of the strip in
   // its per-point form): every element, cut into ranges of multiples of 256
@@ -1647,7 +1653,28 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   if (!kitems.empty() && (st = upload(&D.kitems, kitems)) != PUFE_OK) return st;
   if (!jitems.empty() && (st = upload(&D.jitems, jitems)) != PUFE_OK) return st;
   if (!dunits.empty() && (st = upload(&D.dunits, dunits)) != PUFE_OK) return st;
-  if (ser && (st = upload(&D.Rser, Rser)) != PUFE_OK) return st;
+  if (ser) {
+    int len = 0;
+    for (int c = 0; c < 32; ++c) {
+      int k = 0;
+      for (int j = 0; j < 64; ++j) k += Rser[32 * j + c] != 0.0;
+      len = std::max(len, k);
+    }
+    std::vector<int32_t> ri(32 * len, 0);
+    std::vector<double> rv(32 * len, 0.0);
+    for (int c = 0; c < 32; ++c) {
+      int k = 0;
+      for (int j = 0; j < 64; ++j)
+        if (Rser[32 * j + c] != 0.0) {
+          ri[c * len + k] = j;
+          rv[c * len + k++] = Rser[32 * j + c];
+        }
+    }
+    ctx->rser_len = len;
+    if ((st = upload(&D.Rser, Rser)) != PUFE_OK) return st;
+    if ((st = upload(&D.rser_i, ri)) != PUFE_OK) return st;
+    if ((st = upload(&D.rser_v, rv)) != PUFE_OK) return st;
+  }
   if (!titems.empty() && (st = upload(&D.titems, titems)) != PUFE_OK) return st;
   if (!sitems.empty() && (st = upload(&D.sitems, sitems)) != PUFE_OK) return st;
   if (!gitems32.empty() && (st = upload(&D.gitems32, gitems32)) != PUFE_OK) return st;
@@ -1696,7 +1723,7 @@ static void free_device(pufe_ctx *ctx) {
   void *ptrs[] = {D.qoff, D.x, D.w, D.xi, D.doff, D.dofs, D.ecol, D.eshift, D.aoff, D.alist,
                   D.toff, D.psi, D.psi32, D.qpoff, D.qdat, D.ptab, D.vpad, D.toff32, D.eorig,
                   D.Tfe, D.Sfe, D.S0, D.partoff, D.part_p, D.part_q,
-                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems, D.jitems, D.dunits, D.Rser, D.kitems,
+                  D.orb, D.orbf, D.rowptr, D.col, D.soff, D.smap, D.order, D.wsplit, D.aitems, D.jitems, D.dunits, D.Rser, D.rser_i, D.rser_v, D.kitems,
                   D.titems, D.sitems, D.gitems32, D.gitems64, D.citems, D.pitems, D.tblk, D.eeform, D.err};
   for (void *p : ptrs)
     if (p) cudaFree(p);

@@ -51,10 +51,10 @@
 // cut so that the items of small meshes still fill the chip.  All blocks meet in
 // FP64 atomics.
 //
-// Measured (kernel time, direct kernel before): 12^3 rocksalt cell 18.8 -> 1.37 ms,
-// CsCl-like 16^3 cell 23.7 -> 2.65 ms, two-atom 4^3 cell 1.72 -> 0.096 ms, eight
-// elements of 6^3 points 377 -> 33 us; triclinic serendipity 6^3 at a wavevector 1.15
-// -> 0.48 ms.
+// Measured (kernel time, direct kernel before): 12^3 rocksalt cell 18.8 -> 1.31 ms,
+// CsCl-like 16^3 cell 23.7 -> 2.62 ms, two-atom 4^3 cell 1.72 -> 0.094 ms, eight
+// elements of 6^3 points 377 -> 35 us; triclinic serendipity 6^3 at a wavevector 1.15
+// -> 0.21 ms.
 #include <algorithm>
 
 #include "pufe_internal.h"
@@ -83,8 +83,11 @@ struct Asm64 {
   // the physical gradients; general cells (GEN) jit = J^-T, the fields
   // (J^-1 grad Psi)_d and the metric G = J^-1 J^-T
   double sc[3], jit[9], G[9];
-  const double *Rser;   // serendipity space: nodal values 64 x 32 (nfe = 32)
-  int nfe;
+  // serendipity space (nfe = 32): the tricubic nodes where function c is not zero
+  // and its values there, rl per function (padded with zeros)
+  const int32_t *ri;
+  const double *rv;
+  int rl, nfe;
   int want, work;   // PUFE_WANT_* mask; doubles of the shared work area
   unsigned *err;
 };
@@ -206,21 +209,20 @@ __device__ void fefe_item(const Asm64 &P, int e, int cb, int ce, double *sm) {
     return M[pidx64(i & 3, j & 3) * 100 + pidx64((i >> 2) & 3, (j >> 2) & 3) * 10 +
              pidx64(i >> 4, j >> 4)];
   };
-  double *Y = M + 1000;   // serendipity: R^T M (32 x 64), R the nodal values of its functions
+  // serendipity: R^T M, R the nodal values of its functions, transposed [64][32];
+  // a warp works on one function's nodes, so that its list is uniform
+  double *Y = M + 1000;
   if (P.nfe == 32 && h) {
     for (int o = tid; o < 2048; o += A64_NT) {
       const int c = o >> 6, k = o & 63;
       double s = 0.0;
-      for (int j = 0; j < 64; ++j) {
-        const double r = P.Rser[j * 32 + c];
-        if (r != 0.0) s = fma(r, tri(j, k), s);
-      }
-      Y[o] = s;
+      for (int u = 0; u < P.rl; ++u) s = fma(P.rv[c * P.rl + u], tri(P.ri[c * P.rl + u], k), s);
+      Y[k * 32 + c] = s;
     }
     __syncthreads();
   }
-  // the constants come with the element's first (sub)cell range; at the Gamma
-  // point S starts as their sum, so only H is added
+  // the constants come with the element's first (sub)cell range; S starts as their
+  // sum at the Gamma point, so a wavevector adds only what the phases change
   const bool s = BLOCH && (P.want & PUFE_WANT_S) && cb == 0;
   const int nf = P.nfe;
   for (int o = tid; o < nf * nf; o += A64_NT) {
@@ -228,67 +230,78 @@ __device__ void fefe_item(const Asm64 &P, int e, int cb, int ce, double *sm) {
     double v = 0.0;
     if (nf == 64) {
       v = tri(i, j);
-    } else if (h) {
-      for (int k = 0; k < 64; ++k) {
-        const double r = P.Rser[k * 32 + j];
-        if (r != 0.0) v = fma(r, Y[i * 64 + k], v);
-      }
+    } else if (h) {   // (symmetric: row i from function i's list, column j from Y)
+      for (int u = 0; u < P.rl; ++u)
+        v = fma(P.rv[i * P.rl + u], Y[P.ri[i * P.rl + u] * 32 + j], v);
     }
-    add_entry<BLOCH>(P, m[i * n + j], h && cb == 0 ? P.Tfe[o] + v : v, s ? P.Sfe[o] : 0.0, h, s,
-                     BLOCH ? es[i] : 0, BLOCH ? es[j] : 0);
+    const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
+    add_entry<BLOCH>(P, m[i * n + j], h && cb == 0 ? P.Tfe[o] + v : v, 0.0, h, false, ci, cj);
+    if (s && ci != cj) {
+      const double pr = P.ph.re[ci] * P.ph.re[cj] + P.ph.im[ci] * P.ph.im[cj];
+      const double pi = P.ph.re[ci] * P.ph.im[cj] - P.ph.im[ci] * P.ph.re[cj];
+      atomicAdd(P.S + m[i * n + j], P.Sfe[o] * (pr - 1.0));
+      atomicAdd(P.Si + m[i * n + j], P.Sfe[o] * pi);
+    }
   }
 }
 
 // ---- FE x enrichment blocks of the slots [s0, s1) ------------------------------
-// 1D constants: nodes x_a, kappa_a, L'_a(x_j)
-__device__ __forceinline__ double node1(int a) { return -1.0 + a * (2.0 / 3.0); }
-__device__ __forceinline__ double kappa1(int a) {
-  return (a & 1 ? 1.0 : -1.0) * (a == 0 || a == 3 ? 0.5625 : 1.6875);
+// 1D constants.  With s = -1, +1 for t = 0, 1: M_a,t = L_a (1 + s x) =
+// alpha_a,t L_a + s kappa_a omega, alpha_a,t = 1 + s x_a = 0, 2/3, 4/3 or 2.  Both
+// values of each constant are known at compile time and picked by t, so that no
+// FP64 operation is spent on them.
+__device__ __forceinline__ double alpha1(int a, bool t) {
+  return t ? (a == 0 ? 0.0 : (a == 1 ? 2.0 / 3.0 : (a == 2 ? 4.0 / 3.0 : 2.0)))
+           : (a == 3 ? 0.0 : (a == 2 ? 2.0 / 3.0 : (a == 1 ? 4.0 / 3.0 : 2.0)));
+}
+__device__ __forceinline__ double kappa1(int a, bool t) {   // s kappa_a
+  const double k = (a & 1 ? 1.0 : -1.0) * (a == 0 || a == 3 ? 0.5625 : 1.6875);
+  return t ? k : -k;
 }
 // L'_a(x_j), row a
 __constant__ double c_d1[16] = {-2.75, -0.5, 0.25, -0.5, 4.5,  -0.75, -1.5, 2.25,
                                 -2.25, 1.5,  0.75, -4.5, 0.5,  -0.25, 0.5,  2.75};
 
-// the four M_a,t of an axis from the five moments at stride `st`:
-// M_a,t = (1 + s x_a) L_a + s kappa_a omega
-__device__ __forceinline__ void expand_m(const double *m, int st, double s, double o[4]) {
-  const double om = s * m[4 * st];
+// the four M_a,t of an axis from the five moments at stride `st`
+__device__ __forceinline__ void expand_m(const double *m, int st, bool t, double o[4]) {
+  const double om = m[4 * st];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) o[a] = fma(kappa1(a), om, (1.0 + s * node1(a)) * m[a * st]);
+  for (int a = 0; a < 4; ++a) o[a] = fma(kappa1(a, t), om, alpha1(a, t) * m[a * st]);
 }
-// adds sum_j L'_a(x_j) (cf (1 + s x_j) F_j + cs s S_j) to o[a]; general cells: with
-// x1, x2 their cross terms' moments, (1 + s x_j) (c1 x1_j + c2 x2_j) too
+// adds sum_j L'_a(x_j) ((1 + s x_j) F_j + ss S_j) to o[a] (ss: the second order
+// factor times s); general cells: with x1, x2 their cross terms' moments,
+// (1 + s x_j) (c1 x1_j + c2 x2_j) too
 template <bool GEN = false>
 __device__ __forceinline__ void expand_d(const double *F, int fst, const double *S, int sst,
-                                         double s, double cf, double cs, double o[4],
+                                         bool t, double ss, double o[4],
                                          const double *x1 = nullptr, int st1 = 0, double c1 = 0.0,
                                          const double *x2 = nullptr, int st2 = 0, double c2 = 0.0) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    double t = cf * F[j * fst];
-    if (GEN) t = fma(c1, x1[j * st1], t);
-    if (GEN && x2) t = fma(c2, x2[j * st2], t);
-    const double g = fma(1.0 + s * node1(j), t, cs * s * S[j * sst]);
+    double f = F[j * fst];
+    if (GEN) f = fma(c1, x1[j * st1], f);
+    if (GEN && x2) f = fma(c2, x2[j * st2], f);
+    const double g = fma(alpha1(j, t), f, ss * S[j * sst]);
 #pragma unroll
     for (int a = 0; a < 4; ++a) o[a] = fma(c_d1[a * 4 + j], g, o[a]);
   }
 }
 // sum_j L'_a(x_j) (1 + s x_j) S_j
-__device__ __forceinline__ void slope_m(const double *S, int st, double s, double o[4]) {
+__device__ __forceinline__ void slope_m(const double *S, int st, bool t, double o[4]) {
 #pragma unroll
   for (int a = 0; a < 4; ++a) o[a] = 0.0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const double g = (1.0 + s * node1(j)) * S[j * st];
+    const double g = alpha1(j, t) * S[j * st];
 #pragma unroll
     for (int a = 0; a < 4; ++a) o[a] = fma(c_d1[a * 4 + j], g, o[a]);
   }
 }
 
-constexpr int FXE_MOM = 550;    // moments of a slot: S 125, V 125, Fx, Fy, Fz 100 each
 // doubles of the expansion's intermediates: orthorhombic, general cells' cross
 // terms, the serendipity space's tricubic rows of H and S
 constexpr int FXE_EXP = 1616, FXE_EXP_GEN = 1160, FXE_EXP_SER = 1024;
+constexpr int FXE_MOM = 550;    // moments of a slot: S 125, V 125, Fx, Fy, Fz 100 each
 constexpr int EXE_MOM = 162;    // moments of a slot pair
 
 template <bool BLOCH, bool GEN>
@@ -324,8 +337,9 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
       double L[4], dL[4];
       lagrange3(x, L, dL);
       double *f = F + d * 5 * p + t;
-      for (int a = 0; a < 4; ++a) f[a * p] = L[a];
-      f[4 * p] = (x + 1.0) * (x + 1.0 / 3.0) * (x - 1.0 / 3.0) * (x - 1.0);
+      const double c8 = d == 2 ? 0.125 : 1.0;   // the 1/8 of phi_v, once
+      for (int a = 0; a < 4; ++a) f[a * p] = c8 * L[a];
+      f[4 * p] = c8 * ((x + 1.0) * (x + 1.0 / 3.0) * (x - 1.0 / 3.0) * (x - 1.0));
     }
     __syncthreads();
     for (int it = tid; it < GP2; it += A64_NT) {   // z: one thread per (slot, qx, qy)
@@ -377,7 +391,8 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
       for (int qy = 0; qy < p; ++qy) {
         const double t = t1[p * qy];
 #pragma unroll
-        for (int u = 0; u < 5; ++u) a[u] = fma(t, f[u * p + qy], a[u]);
+        for (int u = 0; u < 4; ++u) a[u] = fma(t, f[u * p + qy], a[u]);
+        if (r < 15 || r >= 20) a[4] = fma(t, f[4 * p + qy], a[4]);
       }
       // rows 0-14 and 20-23 keep five y moments, Fy (15-19) four
       const int o = r < 15 ? 5 * r : (r < 20 ? 75 + 4 * (r - 15) : 95 + 5 * (r - 20));
@@ -393,7 +408,8 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
       for (int qx = 0; qx < p; ++qx) {
         const double t = t2[qx];
 #pragma unroll
-        for (int u = 0; u < 5; ++u) a[u] = fma(t, f[u * p + qx], a[u]);
+        for (int u = 0; u < 4; ++u) a[u] = fma(t, f[u * p + qx], a[u]);
+        if (r < 50 || r >= 75) a[4] = fma(t, f[4 * p + qx], a[4]);
       }
       // rows 50-74 (Fx) keep four x moments, the others five
       double *mo = mom + g * FXE_MOM + (r < 50 ? 5 * r : (r < 75 ? 250 + 4 * (r - 50) : 350 + 5 * (r - 75)));
@@ -409,12 +425,19 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
   double *YS = R1 + 200, *YFz = YS + 320, *R2 = YFz + 256;                 // [z][y 8][x 8]
   // general cells: D on x; its M on y; D on y of M on x; M on y of s_x L on x
   double *XD = R2 + 320, *YXD = XD + 200, *YD = YXD + 320, *YXL = YD + 320;
-  double *HS = base + FXE_EXP + (GEN ? FXE_EXP_GEN : 0);   // serendipity: [H, S][vertex][64]
-  // 1/2 of the first and second order factors
-  const double c2[3] = {GEN ? 0.5 : 0.5 * P.sc[0], GEN ? 0.5 : 0.5 * P.sc[1],
-                        GEN ? 0.5 : 0.5 * P.sc[2]};
-  const double cc[3] = {GEN ? 0.5 * P.G[0] : c2[0] * P.sc[0], GEN ? 0.5 * P.G[4] : c2[1] * P.sc[1],
-                        GEN ? 0.5 * P.G[8] : c2[2] * P.sc[2]};
+  double *HS = base + FXE_EXP + (GEN ? FXE_EXP_GEN : 0);   // serendipity: [64][H, S][vertex]
+  // 1/2 of the first order factor goes into the moments of Fx, Fy, Fz, 1/2 of the
+  // second into cc
+  const double cc[3] = {0.5 * (GEN ? P.G[0] : P.sc[0] * P.sc[0]),
+                        0.5 * (GEN ? P.G[4] : P.sc[1] * P.sc[1]),
+                        0.5 * (GEN ? P.G[8] : P.sc[2] * P.sc[2])};
+  if (h) {
+    __syncthreads();
+    for (int o = tid; o < 300 * G; o += A64_NT) {
+      const int g = o / 300, i = o - 300 * g;
+      mom[g * FXE_MOM + 250 + i] *= GEN ? 0.5 : 0.5 * P.sc[i / 100];
+    }
+  }
   const double gxy = 0.5 * P.G[1], gxz = 0.5 * P.G[2], gyz = 0.5 * P.G[5];
   const bool ser = P.nfe == 32;
   for (int g = 0; g < G; ++g) {
@@ -430,24 +453,23 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
     for (int it = tid; it < 130; it += A64_NT) {   // x
       const int t = it & 1, r = it >> 1;
       if (!(xm >> t & 1)) continue;
-      const double s = t ? 1.0 : -1.0;
       double o[4];
       if (r < 25) {
-        expand_m(S + 5 * r, 1, s, o);
+        expand_m(S + 5 * r, 1, t, o);
         for (int a = 0; a < 4; ++a) XS[r * 8 + 4 * t + a] = o[a];
         if (h) {
-          expand_m(Vm + 5 * r, 1, s, o);
-          expand_d(Fx + 4 * r, 1, S + 5 * r, 1, s, c2[0], cc[0], o);
+          expand_m(Vm + 5 * r, 1, t, o);
+          expand_d(Fx + 4 * r, 1, S + 5 * r, 1, t, t ? cc[0] : -cc[0], o);
           for (int a = 0; a < 4; ++a) R1[r * 8 + 4 * t + a] = o[a];
           if (GEN) {
-            slope_m(S + 5 * r, 1, s, o);
+            slope_m(S + 5 * r, 1, t, o);
             for (int a = 0; a < 4; ++a) XD[r * 8 + 4 * t + a] = o[a];
           }
         }
       } else if (h) {
         const bool y = r < 45;
         const int rr = y ? r - 25 : r - 45;
-        expand_m((y ? Fy : Fz) + 5 * rr, 1, s, o);
+        expand_m((y ? Fy : Fz) + 5 * rr, 1, t, o);
         for (int a = 0; a < 4; ++a) (y ? XFy : XFz)[rr * 8 + 4 * t + a] = o[a];
       }
     }
@@ -458,32 +480,32 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
       const double s = t ? 1.0 : -1.0;
       double o[4];
       if (z < 5) {
-        expand_m(XS + z * 40 + x, 8, s, o);
+        expand_m(XS + z * 40 + x, 8, t, o);
         for (int b = 0; b < 4; ++b) YS[z * 64 + (4 * t + b) * 8 + x] = o[b];
         if (h) {
-          expand_m(R1 + z * 40 + x, 8, s, o);
+          expand_m(R1 + z * 40 + x, 8, t, o);
           if (GEN) {
             // s_x L_a on x: the moments of L_a themselves, signed
             const double sx = x >> 2 ? 1.0 : -1.0, *xl = S + z * 25 + (x & 3);
-            expand_d<true>(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, s, c2[1], cc[1], o, xl, 5,
+            expand_d<true>(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, t, s * cc[1], o, xl, 5,
                            gxy * sx);
             for (int b = 0; b < 4; ++b) {
               o[b] = fma(gxy * s, XD[z * 40 + b * 8 + x], o[b]);
               R2[z * 64 + (4 * t + b) * 8 + x] = o[b];
             }
-            expand_m(XD + z * 40 + x, 8, s, o);
+            expand_m(XD + z * 40 + x, 8, t, o);
             for (int b = 0; b < 4; ++b) YXD[z * 64 + (4 * t + b) * 8 + x] = o[b];
-            slope_m(XS + z * 40 + x, 8, s, o);
+            slope_m(XS + z * 40 + x, 8, t, o);
             for (int b = 0; b < 4; ++b) YD[z * 64 + (4 * t + b) * 8 + x] = o[b];
-            expand_m(xl, 5, s, o);
+            expand_m(xl, 5, t, o);
             for (int b = 0; b < 4; ++b) YXL[z * 64 + (4 * t + b) * 8 + x] = sx * o[b];
           } else {
-            expand_d(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, s, c2[1], cc[1], o);
+            expand_d(XFy + z * 32 + x, 8, XS + z * 40 + x, 8, t, t ? cc[1] : -cc[1], o);
             for (int b = 0; b < 4; ++b) R2[z * 64 + (4 * t + b) * 8 + x] = o[b];
           }
         }
       } else if (h) {
-        expand_m(XFz + (z - 5) * 40 + x, 8, s, o);
+        expand_m(XFz + (z - 5) * 40 + x, 8, t, o);
         for (int b = 0; b < 4; ++b) YFz[(z - 5) * 64 + (4 * t + b) * 8 + x] = o[b];
       }
     }
@@ -494,48 +516,46 @@ __device__ void fxe_item(const Asm64 &P, int e, int s0, int s1, int cb, int ce, 
       if (r < 0) continue;
       const double s = t ? 1.0 : -1.0;
       double so[4], ho[4] = {0, 0, 0, 0};
-      expand_m(YS + xy, 64, s, so);
+      expand_m(YS + xy, 64, t, so);
       if (h) {
-        expand_m(R2 + xy, 64, s, ho);
+        expand_m(R2 + xy, 64, t, ho);
         if (GEN) {
           const double sy = y >> 2 ? 1.0 : -1.0;
-          expand_d<true>(YFz + xy, 64, YS + xy, 64, s, c2[2], cc[2], ho, YXL + xy, 64, gxz,
+          expand_d<true>(YFz + xy, 64, YS + xy, 64, t, s * cc[2], ho, YXL + xy, 64, gxz,
                          XS + (y & 3) * 8 + x, 40, gyz * sy);
           for (int c = 0; c < 4; ++c)
             ho[c] = fma(s, fma(gxz, YXD[c * 64 + xy], gyz * YD[c * 64 + xy]), ho[c]);
         } else {
-          expand_d(YFz + xy, 64, YS + xy, 64, s, c2[2], cc[2], ho);
+          expand_d(YFz + xy, 64, YS + xy, 64, t, t ? cc[2] : -cc[2], ho);
         }
       }
       for (int c = 0; c < 4; ++c) {
         const int i = (x & 3) + 4 * (y & 3) + 16 * c;
         if (ser) {
-          HS[v * 64 + i] = ho[c];
-          HS[512 + v * 64 + i] = so[c];
+          HS[i * 16 + v] = ho[c];
+          HS[i * 16 + 8 + v] = so[c];
           continue;
         }
         const int j = 64 + r;
         const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
-        add_entry<BLOCH>(P, m[i * n + j], 0.125 * ho[c], 0.125 * so[c], h, ws, ci, cj);
-        add_entry<BLOCH>(P, m[j * n + i], 0.125 * ho[c], 0.125 * so[c], h, ws, cj, ci);
+        add_entry<BLOCH>(P, m[i * n + j], ho[c], so[c], h, ws, ci, cj);
+        add_entry<BLOCH>(P, m[j * n + i], ho[c], so[c], h, ws, cj, ci);
       }
     }
     if (!ser) continue;
     __syncthreads();
-    for (int it = tid; it < 256; it += A64_NT) {   // rows of the serendipity functions
-      const int v = it >> 5, i = it & 31, r = sc8[v];
-      if (r < 0) continue;
-      double hv = 0.0, sv = 0.0;
-      for (int k = 0; k < 64; ++k) {
-        const double w = P.Rser[k * 32 + i];
-        if (w == 0.0) continue;
-        hv = fma(w, HS[v * 64 + k], hv);
-        sv = fma(w, HS[512 + v * 64 + k], sv);
-      }
+    // rows of the serendipity functions: half a warp per function (its H and S of
+    // the eight vertices), whose list is uniform there
+    for (int it = tid; it < 512; it += A64_NT) {
+      const int i = it >> 4, hsv = it & 15, r = sc8[hsv & 7];
+      if (r < 0 || !(hsv < 8 ? h : ws)) continue;
+      double t = 0.0;
+      for (int u = 0; u < P.rl; ++u)
+        t = fma(P.rv[i * P.rl + u], HS[P.ri[i * P.rl + u] * 16 + hsv], t);
       const int j = 32 + r;
       const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
-      add_entry<BLOCH>(P, m[i * n + j], 0.125 * hv, 0.125 * sv, h, ws, ci, cj);
-      add_entry<BLOCH>(P, m[j * n + i], 0.125 * hv, 0.125 * sv, h, ws, cj, ci);
+      add_entry<BLOCH>(P, m[i * n + j], t, t, hsv < 8, hsv >= 8, ci, cj);
+      add_entry<BLOCH>(P, m[j * n + i], t, t, hsv < 8, hsv >= 8, cj, ci);
     }
   }
 }
@@ -564,12 +584,13 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
   const int fit = max(1, avail / (22 * pmax * pmax + 60 * pmax + EXE_MOM + 1));
   const int nch = (k1 - k0 + fit - 1) / fit, npc = (k1 - k0 + nch - 1) / nch;
   const int nr1 = h ? 22 : 3, nr2 = h ? 60 : 9;
-  const double c2[3] = {GEN ? 0.5 : 0.5 * P.sc[0], GEN ? 0.5 : 0.5 * P.sc[1],
-                        GEN ? 0.5 : 0.5 * P.sc[2]};
-  // 1/8 (2/h_d)^2 (general cells: G_dd / 8): one half times the quarter of <., 1>
-  const double cq[3] = {GEN ? 0.125 * P.G[0] : 0.25 * c2[0] * P.sc[0],
-                        GEN ? 0.125 * P.G[4] : 0.25 * c2[1] * P.sc[1],
-                        GEN ? 0.125 * P.G[8] : 0.25 * c2[2] * P.sc[2]};
+  // factors of the entries' terms with the scaled 1D functions: 1/4 (2/h_d) (first
+  // order; general cells: 1/4) and 1/8 (2/h_d)^2 (G_dd / 8)
+  const double c1[3] = {GEN ? 0.25 : 0.25 * P.sc[0], GEN ? 0.25 : 0.25 * P.sc[1],
+                        GEN ? 0.25 : 0.25 * P.sc[2]};
+  const double cq[3] = {0.125 * (GEN ? P.G[0] : P.sc[0] * P.sc[0]),
+                        0.125 * (GEN ? P.G[4] : P.sc[1] * P.sc[1]),
+                        0.125 * (GEN ? P.G[8] : P.sc[2] * P.sc[2])};
   for (int c0 = k0; c0 < k1; c0 += npc) {
     const int nc = min(npc, k1 - c0);
     double *mom = base;                                         // [nc][162]
@@ -591,7 +612,8 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
       __syncthreads();
       for (int o = tid; o < 3 * p; o += A64_NT) {
         const int d = o / p, t = o - d * p;
-        const double x = axis_xi(P, qs, p, d, t), l0 = 1.0 - x, l1 = 1.0 + x;
+        // (halved linears: u_k / 4 and l_t / 2, so the 1/64 of phi_v phi_v' is in them)
+        const double x = axis_xi(P, qs, p, d, t), l0 = 0.5 - 0.5 * x, l1 = 0.5 + 0.5 * x;
         double *f = F + d * 6 * p + t;
         f[0] = l0 * l0;
         f[p] = l0 * l1;
@@ -605,6 +627,7 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
         const int g = it / p2, qxy = it - g * p2;
         const double *pa = pe + (int64_t)pr[2 * g] * 4 * Q + pq + qxy;
         const double *pb = pe + (int64_t)pr[2 * g + 1] * 4 * Q + pq + qxy;
+        const bool diag = pa == pb;
         const double *f = F + 12 * p;
         double a[22];
 #pragma unroll
@@ -620,7 +643,7 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
           if (h) {
             double a1 = pa[Q + z], a2 = pa[2 * Q + z], a3 = pa[3 * Q + z];
             double b1 = pb[Q + z], b2 = pb[2 * Q + z], b3 = pb[3 * Q + z];
-            const double wa = w * a0, l0 = f[4 * p + qz], l1 = f[5 * p + qz];
+            const double l0 = f[4 * p + qz], l1 = f[5 * p + qz];
             const double fE = fma(P.V[q], fA, 0.5 * w * fma(a1, b1, fma(a2, b2, a3 * b3)));
             a[3] = fma(fE, u0, a[3]);
             a[4] = fma(fE, u1, a[4]);
@@ -634,19 +657,36 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
               b2 = P.jit[1] * bx + P.jit[4] * by + P.jit[7] * bz;
               b3 = P.jit[2] * bx + P.jit[5] * by + P.jit[8] * bz;
             }
-            const double f4[4] = {wb * a1, wa * b1, wb * a2, wa * b2};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              a[6 + 3 * v] = fma(f4[v], u0, a[6 + 3 * v]);
-              a[7 + 3 * v] = fma(f4[v], u1, a[7 + 3 * v]);
-              a[8 + 3 * v] = fma(f4[v], u2, a[8 + 3 * v]);
-            }
-            const double Bz = wb * a3, Cz = wa * b3;
+            const double Bx = wb * a1, By = wb * a2, Bz = wb * a3;
+            a[6] = fma(Bx, u0, a[6]);
+            a[7] = fma(Bx, u1, a[7]);
+            a[8] = fma(Bx, u2, a[8]);
+            a[12] = fma(By, u0, a[12]);
+            a[13] = fma(By, u1, a[13]);
+            a[14] = fma(By, u2, a[14]);
             a[18] = fma(Bz, l0, a[18]);
             a[19] = fma(Bz, l1, a[19]);
-            a[20] = fma(Cz, l0, a[20]);
-            a[21] = fma(Cz, l1, a[21]);
+            if (!diag) {   // C of a pair alpha = beta is its B
+              const double wa = w * a0, Cx = wa * b1, Cy = wa * b2, Cz = wa * b3;
+              a[9] = fma(Cx, u0, a[9]);
+              a[10] = fma(Cx, u1, a[10]);
+              a[11] = fma(Cx, u2, a[11]);
+              a[15] = fma(Cy, u0, a[15]);
+              a[16] = fma(Cy, u1, a[16]);
+              a[17] = fma(Cy, u2, a[17]);
+              a[20] = fma(Cz, l0, a[20]);
+              a[21] = fma(Cz, l1, a[21]);
+            }
           }
+        }
+        if (diag) {
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            a[9 + u] = a[6 + u];
+            a[15 + u] = a[12 + u];
+          }
+          a[20] = a[18];
+          a[21] = a[19];
         }
 #pragma unroll
         for (int u = 0; u < 22; ++u)
@@ -658,13 +698,13 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
         const double *t1 = T1 + r * NP2 + g * p2 + qx;
         // B_y, C_y (rows 12-17) on the two linears, the others on the quadratics
         const bool lin = r >= 12 && r < 18;
-        const double *f = F + (6 + (lin ? 4 : 0)) * p, *f2 = F + (6 + (lin ? 3 : 2)) * p;
+        const double *f = F + (6 + (lin ? 4 : 0)) * p;
         double x0 = 0.0, x1 = 0.0, x2 = 0.0;
         for (int qy = 0; qy < p; ++qy) {
           const double t = t1[p * qy];
           x0 = fma(t, f[qy], x0);
           x1 = fma(t, f[p + qy], x1);
-          x2 = fma(t, f2[qy], x2);
+          if (!lin) x2 = fma(t, f[2 * p + qy], x2);
         }
         const int o = r < 12 ? 3 * r : (lin ? 36 + 2 * (r - 12) : 48 + 3 * (r - 18));
         T2[o * NP + gq] = x0;
@@ -676,13 +716,13 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
         const int r = it / nc, g = it - r * nc;
         const double *t2 = T2 + r * NP + g * p;
         const bool lin = r >= 18 && r < 36;   // B_x, C_x
-        const double *f = F + (lin ? 4 : 0) * p, *f2 = F + (lin ? 3 : 2) * p;
+        const double *f = F + (lin ? 4 : 0) * p;
         double x0 = 0.0, x1 = 0.0, x2 = 0.0;
         for (int qx = 0; qx < p; ++qx) {
           const double t = t2[qx];
           x0 = fma(t, f[qx], x0);
           x1 = fma(t, f[p + qx], x1);
-          x2 = fma(t, f2[qx], x2);
+          if (!lin) x2 = fma(t, f[2 * p + qx], x2);
         }
         double *mo = mom + g * EXE_MOM + (r < 18 ? 3 * r : (lin ? 54 + 2 * (r - 18) : 90 + 3 * (r - 36)));
         mo[0] += x0;
@@ -691,38 +731,42 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
       }
     }
     __syncthreads();
+    // <A, 1 on d> = A_0 + 2 A_1 + A_2 along d (scaled u), for the other two indices
+    double *ones = F;   // [nc][3][9]; the 1D factors and stages are done with
+    if (h) {
+      for (int o = tid; o < 27 * nc; o += A64_NT) {
+        const int g = o / 27, r = o - 27 * g, d = r / 9, u = (r % 9) / 3, w = r % 3;
+        const double *a = mom + g * EXE_MOM + (d == 0 ? u * 9 + w * 3 : (d == 1 ? u * 9 + w : u * 3 + w));
+        const int st = d == 0 ? 1 : (d == 1 ? 3 : 9);
+        ones[o] = fma(2.0, a[st], a[0] + a[2 * st]);
+      }
+      __syncthreads();
+    }
     // entries (v, alpha) x (v', beta) and, for alpha != beta, their transposes
     for (int it = tid; it < nc * 64; it += A64_NT) {
       const int g = it >> 6, v = (it >> 3) & 7, vp = it & 7;
       const int al = pr[2 * g], be = pr[2 * g + 1];
       const int r = scol[al * 8 + v], c = scol[be * 8 + vp];
       if (r < 0 || c < 0) continue;
-      const double *M = mom + g * EXE_MOM;
+      const double *M = mom + g * EXE_MOM, *A1 = ones + 27 * g;
       const int bx = v & 1, by = (v >> 1) & 1, bz = v >> 2, cx = vp & 1, cy = (vp >> 1) & 1, cz = vp >> 2;
       const int kx = bx + cx, ky = by + cy, kz = bz + cz, kzy = (kz * 3 + ky);
-      const double sv = M[kzy * 3 + kx] * (1.0 / 64.0);
+      const double sv = M[kzy * 3 + kx];
       double hv = 0.0;
-      if (h) {
-        const double px = bx ? 1.0 : -1.0, py = by ? 1.0 : -1.0, pz = bz ? 1.0 : -1.0;
-        const double qx = cx ? 1.0 : -1.0, qy = cy ? 1.0 : -1.0, qz = cz ? 1.0 : -1.0;
-        const double *a = M + kzy * 3;
+      if (h) {   // (signs picked, not multiplied: no FP64 operation goes into them)
         hv = M[27 + kzy * 3 + kx];
-        hv = fma(cq[0] * px * qx, a[0] + 2.0 * a[1] + a[2], hv);
-        a = M + kz * 9 + kx;
-        hv = fma(cq[1] * py * qy, a[0] + 2.0 * a[3] + a[6], hv);
-        a = M + ky * 3 + kx;
-        hv = fma(cq[2] * pz * qz, a[0] + 2.0 * a[9] + a[18], hv);
-        hv = fma(c2[0] * px, M[72 + kzy * 2 + cx], hv);
-        hv = fma(c2[0] * qx, M[54 + kzy * 2 + bx], hv);
-        hv = fma(c2[1] * py, M[108 + (kz * 2 + cy) * 3 + kx], hv);
-        hv = fma(c2[1] * qy, M[90 + (kz * 2 + by) * 3 + kx], hv);
-        hv = fma(c2[2] * pz, M[144 + (cz * 3 + ky) * 3 + kx], hv);
-        hv = fma(c2[2] * qz, M[126 + (bz * 3 + ky) * 3 + kx], hv);
+        hv = fma(bx == cx ? cq[0] : -cq[0], A1[kzy], hv);
+        hv = fma(by == cy ? cq[1] : -cq[1], A1[9 + kz * 3 + kx], hv);
+        hv = fma(bz == cz ? cq[2] : -cq[2], A1[18 + ky * 3 + kx], hv);
+        hv = fma(bx ? c1[0] : -c1[0], M[72 + kzy * 2 + cx], hv);
+        hv = fma(cx ? c1[0] : -c1[0], M[54 + kzy * 2 + bx], hv);
+        hv = fma(by ? c1[1] : -c1[1], M[108 + (kz * 2 + cy) * 3 + kx], hv);
+        hv = fma(cy ? c1[1] : -c1[1], M[90 + (kz * 2 + by) * 3 + kx], hv);
+        hv = fma(bz ? c1[2] : -c1[2], M[144 + (cz * 3 + ky) * 3 + kx], hv);
+        hv = fma(cz ? c1[2] : -c1[2], M[126 + (bz * 3 + ky) * 3 + kx], hv);
         if (GEN) {
           // 1/2 G_de s_d s'_e <A, l_b'd on d, l_be on e> for d != e, with
           // l_t = (u_t + u_(t+1)) / 2
-          const double px[3] = {bx ? 1.0 : -1.0, by ? 1.0 : -1.0, bz ? 1.0 : -1.0};
-          const double pq[3] = {cx ? 1.0 : -1.0, cy ? 1.0 : -1.0, cz ? 1.0 : -1.0};
           const int b3[3] = {bx, by, bz}, c3[3] = {cx, cy, cz}, k3[3] = {kx, ky, kz},
                     st[3] = {1, 3, 9};
 #pragma unroll
@@ -732,11 +776,11 @@ __device__ void exe_item(const Asm64 &P, int e, int k0, int k1, int cb, int ce, 
               if (d == f) continue;
               const int o = 3 - d - f;
               const double *q = M + k3[o] * st[o] + c3[d] * st[d] + b3[f] * st[f];
-              hv = fma(0.125 * P.G[3 * d + f] * px[d] * pq[f],
+              const double gdf = 0.125 * P.G[3 * d + f];
+              hv = fma(b3[d] == c3[f] ? gdf : -gdf,
                        q[0] + q[st[d]] + q[st[f]] + q[st[d] + st[f]], hv);
             }
         }
-        hv *= 1.0 / 64.0;
       }
       const int i = P.nfe + r, j = P.nfe + c;
       const int ci = BLOCH ? es[i] : 0, cj = BLOCH ? es[j] : 0;
@@ -996,8 +1040,8 @@ void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, i
   for (const Item &i : L) items.insert(items.end(), {i.e, i.kind, i.a, i.b, i.cb, i.ce});
 }
 
-// H, S (and Hi, Si at a wavevector: ph != nullptr) must hold zeros, S at the
-// Gamma point the FE-FE overlap constants
+// H (and Hi, Si at a wavevector: ph != nullptr) must hold zeros, S the summed
+// FE-FE overlap constants
 pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
                                  double *H, double *Hi, double *S, double *Si, cudaStream_t st) {
   auto &D = ctx->d;
@@ -1032,7 +1076,9 @@ pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double
         P.jit[3 * d + c] = ctx->Jit[3 * d + c];
         for (int r = 0; r < 3; ++r) P.G[3 * d + c] += ctx->Jit[3 * r + d] * ctx->Jit[3 * r + c];
       }
-  P.Rser = D.Rser;
+  P.ri = D.rser_i;
+  P.rv = D.rser_v;
+  P.rl = ctx->rser_len;
   P.nfe = ctx->nfe_e;
   P.want = what;
   P.work = ctx->asm64_work;
