@@ -27,13 +27,15 @@
 namespace pufe {
 
 // per-context work arrays of the SCF calls (allocated on first use)
+constexpr int SCF_SUMS = 4, SCF_SLOTS = 32;   // reductions, partial sums of each
 struct ScfState {
   int n1[3] = {0, 0, 0};
   double *X[3] = {nullptr, nullptr, nullptr};     // n1 x n1, row-major X[node][mode]
   double *lam[3] = {nullptr, nullptr, nullptr};   // n1, ascending
   double *b = nullptr, *t0 = nullptr, *t1 = nullptr;   // n_fe each
-  double *n_out = nullptr, *vc = nullptr, *exc = nullptr, *vxc = nullptr;   // n_q each
-  double *sums = nullptr;   // 8 reduction slots
+  double *n_out = nullptr;  // n_q: output density of a step
+  double *sums = nullptr;   // SCF_SUMS x SCF_SLOTS partial sums of the energies
+  double *h_sums = nullptr; // pinned host copy
   double *f = nullptr;      // occupations: 64 states x up to 64 k-points (k-major)
   double *nk = nullptr;     // n_q: one k-point's density (k-point steps)
   double *atoms = nullptr;  // 5 per atom: tau (3), Z, sigma
@@ -214,227 +216,320 @@ __global__ void k_ion_density(int64_t nq, const double *__restrict__ x, int nato
 }
 
 constexpr int SCF_PMAX = 16;   // largest points per axis of a (sub)cell
+constexpr int SCF_NT = 128;
 
 // 1D Lagrange factors of one p^3 (sub)cell along its three axes:
-// L1[(d * 4 + a) * SCF_PMAX + t] for axis d, function a, axis point t
+// L1[(d * 4 + a) * p + t] for axis d, function a, axis point t
 __device__ __forceinline__ void cell_tables(const double *__restrict__ xi, int64_t qs, int p,
                                             double *L1) {
-  for (int o = threadIdx.x; o < 3 * p; o += blockDim.x) {
+  for (int o = threadIdx.x; o < 3 * p; o += SCF_NT) {
     const int d = o / p, t = o - d * p;
     const int64_t stride = d == 0 ? 1 : (d == 1 ? p : (int64_t)p * p);
     double L[4], dL[4];
     lagrange3(xi[3 * (qs + t * stride) + d], L, dL);
-    for (int a = 0; a < 4; ++a) L1[(d * 4 + a) * SCF_PMAX + t] = L[a];
+    for (int a = 0; a < 4; ++a) L1[(d * 4 + a) * p + t] = L[a];
   }
 }
 
-// b_i += scale sum_q w_q phi_i(x_q) f_q over the 64 FE functions of every
-// element, by sum factorization over each p^3 (sub)cell (contract z, then
-// y, then x: 4 p^3 + 16 p^2 + 64 p multiply-adds per cell)
-__global__ void __launch_bounds__(128) k_fe_load(
+// b_i += scale sum_q w_q phi_i(x_q) (n_q - rho_I,q) over the 64 FE functions of
+// every element, by sum factorization over each p^3 (sub)cell (contract z, then y,
+// then x: 5 p^3 + 16 p^2 + 64 p FP64 operations per cell, which bind it; a column
+// of points is read once for its four z functions).  Also clears the energy sums
+// of the step.
+__global__ void __launch_bounds__(SCF_NT) k_fe_load(
     const int64_t *__restrict__ qoff, const double *__restrict__ w, const double *__restrict__ xi,
     const int32_t *__restrict__ partoff, const int32_t *__restrict__ part_p,
     const int32_t *__restrict__ part_q, const int64_t *__restrict__ doff,
-    const int32_t *__restrict__ dofs, const double *__restrict__ f, double scale,
-    double *__restrict__ b, unsigned *err) {
-  __shared__ double L1[12 * SCF_PMAX];
-  __shared__ double T1[SCF_PMAX * SCF_PMAX * 4];   // [qx + p qy][c]
-  __shared__ double T2[SCF_PMAX * 16];             // [qx][b + 4 c]
-  __shared__ double bl[64];
+    const int32_t *__restrict__ dofs, const double *__restrict__ n,
+    const double *__restrict__ rho_I, double scale, int pm, double *__restrict__ b,
+    double *__restrict__ sums) {
+  extern __shared__ __align__(16) double sml[];
+  double *L1 = sml, *T1 = L1 + 12 * pm, *T2 = T1 + 4 * pm * pm, *bl = T2 + 16 * pm;
   const int e = blockIdx.x, tid = threadIdx.x;
-  if (tid < 64) bl[tid] = 0.0;
+  if (e == 0)
+    for (int o = tid; o < SCF_SUMS * SCF_SLOTS; o += SCF_NT) sums[o] = 0.0;
+  for (int o = tid; o < 64; o += SCF_NT) bl[o] = 0.0;
   for (int k = partoff[e]; k < partoff[e + 1]; ++k) {
     const int p = part_p[k], p2 = p * p;
-    if (p > SCF_PMAX) {
-      if (tid == 0) atomicOr(err, DEVERR_SHAPE);
-      return;
-    }
     const int64_t qs = qoff[e] + part_q[k];
     __syncthreads();
     cell_tables(xi, qs, p, L1);
     __syncthreads();
-    for (int it = tid; it < p2 * 4; it += blockDim.x) {   // z
-      const int qxy = it >> 2, c = it & 3;
-      double s = 0.0;
+    for (int it = tid; it < p2; it += SCF_NT) {   // z: [c][qx + p qy]
+      double s[4] = {0, 0, 0, 0};
+#pragma unroll 4
       for (int qz = 0; qz < p; ++qz) {
-        const int64_t q = qs + qxy + (int64_t)p2 * qz;
-        s += w[q] * f[q] * L1[(8 + c) * SCF_PMAX + qz];
+        const int64_t q = qs + it + (int64_t)p2 * qz;
+        const double v = w[q] * (n[q] - rho_I[q]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] = fma(v, L1[(8 + c) * p + qz], s[c]);
       }
-      T1[it] = s;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) T1[c * p2 + it] = s[c];
     }
     __syncthreads();
-    for (int it = tid; it < p * 16; it += blockDim.x) {   // y
-      const int qx = it >> 4, bc = it & 15, bb = bc & 3, c = bc >> 2;
+    for (int it = tid; it < p * 16; it += SCF_NT) {   // y: [b + 4 c][qx]
+      const int bc = it / p, qx = it - bc * p, bb = bc & 3, c = bc >> 2;
       double s = 0.0;
-      for (int qy = 0; qy < p; ++qy) s += T1[(qx + p * qy) * 4 + c] * L1[(4 + bb) * SCF_PMAX + qy];
+      for (int qy = 0; qy < p; ++qy) s = fma(T1[c * p2 + p * qy + qx], L1[(4 + bb) * p + qy], s);
       T2[it] = s;
     }
     __syncthreads();
-    if (tid < 64) {                                       // x
-      const int a = tid & 3, bc = tid >> 2;
+    for (int it = tid; it < 64; it += SCF_NT) {       // x
+      const int a = it & 3, bc = it >> 2;
       double s = 0.0;
-      for (int qx = 0; qx < p; ++qx) s += T2[qx * 16 + bc] * L1[a * SCF_PMAX + qx];
-      bl[tid] += s;
+      for (int qx = 0; qx < p; ++qx) s = fma(T2[bc * p + qx], L1[a * p + qx], s);
+      bl[it] += s;
     }
   }
   __syncthreads();
-  if (tid < 64) atomicAdd(b + dofs[doff[e] + tid], scale * bl[tid]);
+  for (int o = tid; o < 64; o += SCF_NT) atomicAdd(b + dofs[doff[e] + o], scale * bl[o]);
 }
 
-// out = A applied along axis `axis` of the (n0, n1, n2) node array (x fastest):
-// out[.., j, ..] = sum_k A[k][j] in[.., k, ..] (transpose = true: A^T, i.e.
-// sum_k A[k][j]; transpose = false: sum_k A[j][k])
-__global__ void k_axis(int n0, int n1, int n2, int axis, const double *__restrict__ A,
-                       bool transpose, const double *__restrict__ in, double *__restrict__ out) {
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t total = (int64_t)n0 * n1 * n2;
-  if (id >= total) return;
-  const int i0 = (int)(id % n0), i1 = (int)((id / n0) % n1), i2 = (int)(id / ((int64_t)n0 * n1));
-  const int n = axis == 0 ? n0 : (axis == 1 ? n1 : n2);
-  const int j = axis == 0 ? i0 : (axis == 1 ? i1 : i2);
-  const int64_t stride = axis == 0 ? 1 : (axis == 1 ? n0 : (int64_t)n0 * n1);
-  const int64_t base = id - (int64_t)j * stride;
-  double s = 0.0;
-  for (int k = 0; k < n; ++k) {
-    const double a = transpose ? A[(size_t)k * n + j] : A[(size_t)j * n + k];
-    s += a * in[base + (int64_t)k * stride];
+// One axis of the (n0, n1, n2) node array (x fastest): out[.., j, ..] =
+// sum_k M[k][j] in[.., k, ..] with M = X (fwd) or X^T (back), X row-major
+// [node][mode].  A CTA takes `nb` lines (8; fewer on very long axes).  n FP64
+// multiply-adds per node bind it (2.7 us for 36^3 nodes) as long as nothing waits:
+// M is staged in shared memory by one round of independent loads (reading it from
+// L2 inside the sums, a few values ahead, took 13-25 us), and a sum runs in four
+// chains.  M too large for the stage (over 112 nodes per axis) is read in place.
+// `clear` (may be null): an array of the same size set to zero.
+constexpr int AX_NT = 256;
+
+__device__ __forceinline__ int64_t line_base(int n0, int n1, int axis, int64_t line) {
+  if (axis == 0) return line * n0;
+  if (axis == 1) return (line % n0) + (line / n0) * ((int64_t)n0 * n1);
+  return line;
+}
+
+// M into shared memory as [k][j] (staged) or left in place; entry (k, j) then is at
+// k sk + j sj of the returned pointer
+__device__ __forceinline__ const double *axis_matrix(const double *__restrict__ X, bool fwd, int n,
+                                                     bool staged, double *M, int &sk, int &sj) {
+  if (!staged) {
+    sk = fwd ? n : 1;
+    sj = fwd ? 1 : n;
+    return X;
   }
-  out[id] = s;
+  if (fwd)
+    for (int o = threadIdx.x; o < n * n; o += AX_NT) M[o] = X[o];
+  else
+    for (int o = threadIdx.x; o < n * n; o += AX_NT) {
+      const int j = o / n, k = o - j * n;
+      M[k * n + j] = X[o];
+    }
+  sk = n;
+  sj = 1;
+  return M;
 }
 
-// c_abc /= (lx_a + ly_b + lz_c); the constant mode (0, 0, 0) -> 0
-__global__ void k_modal_scale(int n0, int n1, int n2, const double *__restrict__ l0,
-                              const double *__restrict__ l1, const double *__restrict__ l2,
-                              double *__restrict__ c) {
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t total = (int64_t)n0 * n1 * n2;
-  if (id >= total) return;
-  const int i0 = (int)(id % n0), i1 = (int)((id / n0) % n1), i2 = (int)(id / ((int64_t)n0 * n1));
-  c[id] = (id == 0) ? 0.0 : c[id] / (l0[i0] + l1[i1] + l2[i2]);
+__device__ __forceinline__ double line_sum(const double *m, int sk, int n, const double *in,
+                                           int nb) {
+  double s[4] = {0, 0, 0, 0};
+  int k = 0;
+  for (; k + 4 <= n; k += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] = fma(m[(int64_t)(k + u) * sk], in[(k + u) * nb], s[u]);
+  }
+  for (; k < n; ++k) s[0] = fma(m[(int64_t)k * sk], in[k * nb], s[0]);
+  return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// V(x_q) = sum_i v_i phi_i(x_q) over the 64 FE functions, by sum
-// factorization over each p^3 (sub)cell (x, then y, then z)
-__global__ void __launch_bounds__(128) k_fe_interp(
+__global__ void __launch_bounds__(AX_NT) k_axis(int n0, int n1, int n2, int axis, int nb,
+                                                bool staged, const double *__restrict__ X,
+                                                bool fwd, const double *__restrict__ in,
+                                                double *__restrict__ out,
+                                                double *__restrict__ clear) {
+  extern __shared__ __align__(16) double smx[];   // [k][line], then M
+  const int n = axis == 0 ? n0 : (axis == 1 ? n1 : n2);
+  const int64_t lines = (int64_t)n0 * n1 * n2 / n, l0 = (int64_t)blockIdx.x * nb;
+  const int nl = (int)min((int64_t)nb, lines - l0);
+  const int64_t stride = axis == 0 ? 1 : (axis == 1 ? n0 : (int64_t)n0 * n1);
+  int sk, sj;
+  const double *M = axis_matrix(X, fwd, n, staged, smx + n * nb, sk, sj);
+  for (int o = threadIdx.x; o < nl * n; o += AX_NT) {
+    const int l = axis == 0 ? o / n : o % nl, k = axis == 0 ? o - l * n : o / nl;
+    smx[k * nb + l] = in[line_base(n0, n1, axis, l0 + l) + k * stride];
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < nl * n; o += AX_NT) {
+    const int l = axis == 0 ? o / n : o % nl, j = axis == 0 ? o - l * n : o / nl;
+    const int64_t at = line_base(n0, n1, axis, l0 + l) + j * stride;
+    out[at] = line_sum(M + (int64_t)j * sj, sk, n, smx + l, nb);
+    if (clear) clear[at] = 0.0;
+  }
+}
+
+// The z axis both ways around the modal scaling: forward, c_abc / (lx_a + ly_b +
+// lz_c) with the constant mode (0, 0, 0) set to zero, and back, on the same lines
+// (back reads the same staged matrix by rows).
+__global__ void __launch_bounds__(AX_NT) k_axis_z(int n0, int n1, int n2, int nb, bool staged,
+                                                  const double *__restrict__ X,
+                                                  const double *__restrict__ lx,
+                                                  const double *__restrict__ ly,
+                                                  const double *__restrict__ lz,
+                                                  const double *__restrict__ in,
+                                                  double *__restrict__ out) {
+  extern __shared__ __align__(16) double smx[];   // [k][line], twice, then X
+  double *c = smx + n2 * nb;
+  const int64_t plane = (int64_t)n0 * n1, l0 = (int64_t)blockIdx.x * nb;
+  const int nl = (int)min((int64_t)nb, plane - l0);
+  int sk, sj;
+  const double *M = axis_matrix(X, true, n2, staged, c + n2 * nb, sk, sj);
+  for (int o = threadIdx.x; o < nl * n2; o += AX_NT) {
+    const int l = o % nl, k = o / nl;
+    smx[k * nb + l] = in[l0 + l + k * plane];
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < nl * n2; o += AX_NT) {
+    const int l = o % nl, j = o / nl;
+    const int64_t xy = l0 + l;
+    const double s = line_sum(M + (int64_t)j * sj, sk, n2, smx + l, nb);
+    c[j * nb + l] = (xy == 0 && j == 0) ? 0.0 : s / (lx[xy % n0] + ly[xy / n0] + lz[j]);
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < nl * n2; o += AX_NT) {
+    const int l = o % nl, j = o / nl;
+    out[l0 + l + j * plane] = line_sum(M + (int64_t)j * sk, sj, n2, c + l, nb);
+  }
+}
+
+// Powers for the LDA from their FP32 values, each refined once by Householder's
+// iteration of third order (the residual r of an FP32 start is about 2^-22, so the
+// terms left out are below 2^-62): a handful of FP64 operations each, where the
+// library's cbrt, square root and division take tens -- and FP64 operations are what
+// binds a pass over the points.
+// n^(-1/3), 1e-30 < n: y <- y (1 + r / 3 + 2 r^2 / 9), r = 1 - n y^3 (values beyond
+// the FP32 range take cbrt)
+__device__ __forceinline__ double inv_cbrt(double n) {
+  if (!(n < 1e37)) return 1.0 / cbrt(n);
+  const double y = (double)rcbrtf((float)n);
+  const double r = fma(-n * y, y * y, 1.0);
+  return fma(y * r, fma(r, 2.0 / 9.0, 1.0 / 3.0), y);
+}
+// x^(-1/2), 1 <= x < 1e30: y <- y (1 + r / 2 + 3 r^2 / 8), r = 1 - x y^2
+__device__ __forceinline__ double inv_sqrt(double x) {
+  const double y = (double)rsqrtf((float)x);
+  const double r = fma(-x * y, y, 1.0);
+  return fma(y * r, fma(r, 0.375, 0.5), y);
+}
+// 1 / x, 1 <= x < 1e30: y <- y (1 + r + r^2), r = 1 - x y
+__device__ __forceinline__ double inverse(double x) {
+  const double y = (double)(1.0f / (float)x);
+  const double r = fma(-x, y, 1.0);
+  return fma(y * r, r + 1.0, y);
+}
+
+// Dirac exchange + Perdew-Zunger 1981 correlation (unpolarised); 0 for n <= 1e-30.
+// The energy per electron (v false) or the potential (v true).
+__device__ __forceinline__ double lda_pz81(double n, bool v) {
+  if (!(n > 1e-30)) return 0.0;
+  const double y = inv_cbrt(n);
+  const double rs = 0.62035049089940009 * y;           // (3 / (4 pi))^(1/3) n^(-1/3)
+  const double ex = -0.73855876638202240 * (n * y * y);   // -3/4 (3 / pi)^(1/3) n^(1/3)
+  if (rs >= 1.0) {
+    const double sq = rs * inv_sqrt(rs);
+    const double inv = inverse(fma(1.0529, sq, fma(0.3334, rs, 1.0)));
+    if (!v) return fma(-0.1423, inv, ex);
+    return fma(4.0 / 3.0, ex,
+               -0.1423 * fma(7.0 / 6.0 * 1.0529, sq, fma(4.0 / 3.0 * 0.3334, rs, 1.0)) * inv * inv);
+  }
+  const double lr = log(rs);
+  if (!v) return ex + (0.0311 * lr - 0.048 + 0.0020 * rs * lr - 0.0116 * rs);
+  return fma(4.0 / 3.0, ex,
+             0.0311 * lr + (-0.048 - 0.0311 / 3.0) + 2.0 / 3.0 * 0.0020 * rs * lr +
+                 (2.0 * -0.0116 - 0.0020) / 3.0 * rs);
+}
+
+// V_C(x_q) = sum_i v_i phi_i(x_q) over the 64 FE functions, by sum factorization
+// over each p^3 (sub)cell (x, then y, then z), and what the caller makes of it at
+// the point while it is in a register:
+//  * V_eff != nullptr: V_eff = V_C + v_xc(n), and V_C, eps_xc where wanted;
+//  * else the energies of n (an output density) and its mixing: partial sums
+//    [0] += w n V_in, [1] += w (rho_I - n) V_C, [2] += w n eps_xc, [3] += w |n - n_in|
+//    (32 partial sums each: thousands of atomics on one address would take longer
+//    than the sums themselves), then n_in <- n_in + alpha (n - n_in).
+struct InterpOut {
+  const double *n;
+  double *V_eff, *V_C, *eps_xc;
+  const double *w, *V_in, *rho_I;
+  double alpha;
+  double *n_in, *sums;
+};
+
+__global__ void __launch_bounds__(SCF_NT) k_fe_interp(
     const int64_t *__restrict__ qoff, const double *__restrict__ xi,
     const int32_t *__restrict__ partoff, const int32_t *__restrict__ part_p,
     const int32_t *__restrict__ part_q, const int64_t *__restrict__ doff,
-    const int32_t *__restrict__ dofs, const double *__restrict__ v, double *__restrict__ out,
-    unsigned *err) {
-  __shared__ double L1[12 * SCF_PMAX];
-  __shared__ double ve[64];
-  __shared__ double T1[16 * SCF_PMAX];              // [b + 4 c][qx]
-  __shared__ double T2[4 * SCF_PMAX * SCF_PMAX];    // [c][qx + p qy]
+    const int32_t *__restrict__ dofs, const double *__restrict__ v, int pm, InterpOut O) {
+  extern __shared__ __align__(16) double smi[];
+  double *L1 = smi, *ve = L1 + 12 * pm, *T1 = ve + 64, *T2 = T1 + 16 * pm;   // T2: [c][qx + p qy]
+  double *red = T2 + 4 * pm * pm;                                            // [4][warps]
   const int e = blockIdx.x, tid = threadIdx.x;
-  if (tid < 64) ve[tid] = v[dofs[doff[e] + tid]];
+  for (int o = tid; o < 64; o += SCF_NT) ve[o] = v[dofs[doff[e] + o]];
+  double s4[SCF_SUMS] = {0.0, 0.0, 0.0, 0.0};
   for (int k = partoff[e]; k < partoff[e + 1]; ++k) {
     const int p = part_p[k], p2 = p * p;
-    if (p > SCF_PMAX) {
-      if (tid == 0) atomicOr(err, DEVERR_SHAPE);
-      return;
-    }
     const int64_t qs = qoff[e] + part_q[k];
     __syncthreads();
     cell_tables(xi, qs, p, L1);
     __syncthreads();
-    for (int it = tid; it < 16 * p; it += blockDim.x) {   // x
+    for (int it = tid; it < 16 * p; it += SCF_NT) {   // x
       const int bc = it / p, qx = it - bc * p;
       double s = 0.0;
-      for (int a = 0; a < 4; ++a) s += ve[a + 4 * bc] * L1[a * SCF_PMAX + qx];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) s = fma(ve[a + 4 * bc], L1[a * p + qx], s);
       T1[it] = s;
     }
     __syncthreads();
-    for (int it = tid; it < 4 * p2; it += blockDim.x) {   // y
+    for (int it = tid; it < 4 * p2; it += SCF_NT) {   // y
       const int c = it / p2, qxy = it - c * p2, qy = qxy / p, qx = qxy - qy * p;
       double s = 0.0;
-      for (int bb = 0; bb < 4; ++bb) s += T1[(bb + 4 * c) * p + qx] * L1[(4 + bb) * SCF_PMAX + qy];
+#pragma unroll
+      for (int bb = 0; bb < 4; ++bb) s = fma(T1[(bb + 4 * c) * p + qx], L1[(4 + bb) * p + qy], s);
       T2[it] = s;
     }
     __syncthreads();
-    for (int it = tid; it < p2 * p; it += blockDim.x) {   // z
+    for (int it = tid; it < p2 * p; it += SCF_NT) {   // z
       const int qz = it / p2, qxy = it - qz * p2;
-      double s = 0.0;
-      for (int c = 0; c < 4; ++c) s += T2[c * p2 + qxy] * L1[(8 + c) * SCF_PMAX + qz];
-      out[qs + it] = s;
+      const int64_t q = qs + it;
+      double vc = 0.0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) vc = fma(T2[c * p2 + qxy], L1[(8 + c) * p + qz], vc);
+      const double n = O.n[q];
+      if (O.V_eff) {
+        if (O.V_C) O.V_C[q] = vc;
+        if (O.eps_xc) O.eps_xc[q] = lda_pz81(n, false);
+        O.V_eff[q] = vc + lda_pz81(n, true);
+      } else {
+        const double w = O.w[q], wn = w * n, ni = O.n_in[q];
+        s4[0] = fma(wn, O.V_in[q], s4[0]);
+        s4[1] = fma(w * (O.rho_I[q] - n), vc, s4[1]);
+        s4[2] = fma(wn, lda_pz81(n, false), s4[2]);
+        s4[3] = fma(w, fabs(n - ni), s4[3]);
+        O.n_in[q] = ni + O.alpha * (n - ni);
+      }
     }
   }
-}
-
-// Dirac exchange + Perdew-Zunger 1981 correlation (unpolarised); 0 for n <= 1e-30
-__device__ inline void lda_pz81(double n, double &e, double &v) {
-  if (!(n > 1e-30)) {
-    e = v = 0.0;
-    return;
+  if (O.V_eff) return;
+  const int lane = tid & 31, warp = tid >> 5, nw = (SCF_NT + 31) / 32;
+  for (int k = 0; k < SCF_SUMS; ++k) {
+    double t = s4[k];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (lane == 0) red[k * nw + warp] = t;
   }
-  const double rs = cbrt(3.0 / (4.0 * PI * n));
-  const double ex = -0.75 * cbrt(3.0 * n / PI);
-  double ec, vc;
-  if (rs >= 1.0) {
-    const double sq = sqrt(rs), den = 1.0 + 1.0529 * sq + 0.3334 * rs;
-    ec = -0.1423 / den;
-    vc = ec * (1.0 + 7.0 / 6.0 * 1.0529 * sq + 4.0 / 3.0 * 0.3334 * rs) / den;
-  } else {
-    const double lr = log(rs);
-    ec = 0.0311 * lr - 0.048 + 0.0020 * rs * lr - 0.0116 * rs;
-    vc = 0.0311 * lr + (-0.048 - 0.0311 / 3.0) + 2.0 / 3.0 * 0.0020 * rs * lr +
-         (2.0 * -0.0116 - 0.0020) / 3.0 * rs;
+  __syncthreads();
+  for (int k = tid; k < SCF_SUMS; k += SCF_NT) {
+    double t = 0.0;
+    for (int i = 0; i < nw; ++i) t += red[k * nw + i];
+    atomicAdd(O.sums + k * SCF_SLOTS + (e & (SCF_SLOTS - 1)), t);
   }
-  e = ex + ec;
-  v = 4.0 / 3.0 * ex + vc;
-}
-
-__global__ void k_xc(int64_t nq, const double *__restrict__ n, double *__restrict__ exc,
-                     double *__restrict__ vxc) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  double e, v;
-  lda_pz81(n[q], e, v);
-  if (exc) exc[q] = e;
-  if (vxc) vxc[q] = v;
-}
-
-__global__ void k_diff(int64_t nq, const double *__restrict__ a, const double *__restrict__ b,
-                       double *__restrict__ out) {   // out = a - b
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < nq) out[q] = a[q] - b[q];
 }
 
 __global__ void k_add(int64_t nq, const double *__restrict__ a, const double *__restrict__ b,
                       double *__restrict__ out) {    // out = a + b
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q < nq) out[q] = a[q] + b[q];
-}
-
-// energies of n_out and the residual, one pass over the points:
-// sums[0] += w n_out V_in, sums[1] += w (rho_I - n_out) V_C, sums[2] += w n_out eps_xc,
-// sums[3] += w |n_out - n_in|; then n_in <- n_in + alpha (n_out - n_in)
-__global__ void k_energy_mix(int64_t nq, const double *__restrict__ w, const double *__restrict__ n_out,
-                             const double *__restrict__ V_in, const double *__restrict__ rho_I,
-                             const double *__restrict__ vc, const double *__restrict__ exc,
-                             double alpha, double *__restrict__ n_in, double *__restrict__ sums) {
-  __shared__ double red[4][32];
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  if (q < nq) {
-    const double no = n_out[q], wq = w[q], ni = n_in[q];
-    s[0] = wq * no * V_in[q];
-    s[1] = wq * (rho_I[q] - no) * vc[q];
-    s[2] = wq * no * exc[q];
-    s[3] = wq * fabs(no - ni);
-    n_in[q] = ni + alpha * (no - ni);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int k = 0; k < 4; ++k) {
-    double t = s[k];
-    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-    if (lane == 0) red[k][warp] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    double t = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[threadIdx.x][i];
-    atomicAdd(sums + threadIdx.x, t);
-  }
 }
 
 constexpr int PULAY_MAX = 8;
@@ -543,13 +638,12 @@ pufe_status scf_prepare(pufe_ctx *ctx) {
   }
   const size_t nfe = (size_t)ctx->n_fe * sizeof(double), nq = (size_t)ctx->nq * sizeof(double);
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->b, nfe));
+  PUFE_CUDA_TRY(cudaMemset(S->b, 0, nfe));   // every solve leaves it zero again
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->t0, nfe));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->t1, nfe));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->n_out, nq));
-  PUFE_CUDA_TRY(cudaMalloc((void **)&S->vc, nq));
-  PUFE_CUDA_TRY(cudaMalloc((void **)&S->exc, nq));
-  PUFE_CUDA_TRY(cudaMalloc((void **)&S->vxc, nq));
-  PUFE_CUDA_TRY(cudaMalloc((void **)&S->sums, 8 * sizeof(double)));
+  PUFE_CUDA_TRY(cudaMalloc((void **)&S->sums, SCF_SUMS * SCF_SLOTS * sizeof(double)));
+  PUFE_CUDA_TRY(cudaMallocHost((void **)&S->h_sums, SCF_SUMS * SCF_SLOTS * sizeof(double)));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->f, 64 * 64 * sizeof(double)));
   return PUFE_OK;
 }
@@ -558,10 +652,11 @@ void scf_free(pufe_ctx *ctx) {
   ScfState *S = ctx->scf;
   if (!S) return;
   void *ptrs[] = {S->X[0], S->X[1], S->X[2], S->lam[0], S->lam[1], S->lam[2], S->b, S->t0,
-                  S->t1, S->n_out, S->vc, S->exc, S->vxc, S->sums, S->f, S->nk, S->atoms,
+                  S->t1, S->n_out, S->sums, S->f, S->nk, S->atoms,
                   S->hist_n, S->hist_R, S->dots};
   for (void *p : ptrs)
     if (p) cudaFree(p);
+  if (S->h_sums) cudaFreeHost(S->h_sums);
   delete S;
   ctx->scf = nullptr;
 }
@@ -593,30 +688,42 @@ pufe_status launch_ion_density(pufe_ctx *ctx, int natoms, const double *tau, con
   return PUFE_OK;
 }
 
-// V_C with del^2 V_C = 4 pi (rho_I - n), zero cell average, at the points
-static pufe_status coulomb(pufe_ctx *ctx, const double *n, const double *rho_I, double *VC,
+// V_C with del^2 V_C = 4 pi (rho_I - n), zero cell average, and at every point what
+// `O` asks for (its n is this n)
+static pufe_status coulomb(pufe_ctx *ctx, const double *rho_I, const InterpOut &O,
                            cudaStream_t st) {
   ScfState *S = ctx->scf;
   auto &D = ctx->d;
-  const int n0 = S->n1[0], n1 = S->n1[1], n2 = S->n1[2];
+  const int n0 = S->n1[0], n1 = S->n1[1], n2 = S->n1[2], pm = std::max(1, ctx->max_part_p);
   const int64_t nfe = ctx->n_fe;
-  // f = n - rho_I at the points (in vc as scratch), b = int phi f
-  k_diff<<<blocks(ctx->nq, 256), 256, 0, st>>>(ctx->nq, n, rho_I, VC);
-  PUFE_CUDA_TRY(cudaMemsetAsync(S->b, 0, nfe * sizeof(double), st));
+  const size_t sm_load = (size_t)(12 * pm + 4 * pm * pm + 16 * pm + 64) * sizeof(double);
+  const size_t sm_out = (size_t)(12 * pm + 64 + 16 * pm + 4 * pm * pm + 16) * sizeof(double);
+  int nb = 8;   // lines per CTA: what two copies of the longest axis' lines leave
+  const int nmax = std::max(n0, std::max(n1, n2));
+  while (nb > 1 && (size_t)2 * nmax * nb * sizeof(double) > 96 * 1024) nb /= 2;
+  const bool staged = nmax <= 112;   // the matrix beside the lines
+  const size_t sm_ax = ((size_t)2 * nmax * nb + (staged ? (size_t)nmax * nmax : 0)) * sizeof(double);
+  if (sm_ax > 227 * 1024)
+    return fail(PUFE_EINVAL, "more nodes per axis than the Poisson solve takes");
+  auto lines = [&](int n) { return (unsigned)((nfe / n + nb - 1) / nb); };
+  PUFE_CUDA_TRY(cudaFuncSetAttribute(k_axis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ax));
+  PUFE_CUDA_TRY(cudaFuncSetAttribute(k_axis_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ax));
   // -K v = 4 pi int phi (rho_I - n)  <=>  K v = 4 pi int phi (n - rho_I)
-  k_fe_load<<<(unsigned)ctx->nelem, 128, 0, st>>>(D.qoff, D.w, D.xi, D.partoff, D.part_p,
-                                                  D.part_q, D.doff, D.dofs, VC, 4.0 * PI, S->b,
-                                                  D.err);
-  const unsigned nb = blocks(nfe, 256);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 0, S->X[0], true, S->b, S->t0);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 1, S->X[1], true, S->t0, S->t1);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 2, S->X[2], true, S->t1, S->t0);
-  k_modal_scale<<<nb, 256, 0, st>>>(n0, n1, n2, S->lam[0], S->lam[1], S->lam[2], S->t0);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 2, S->X[2], false, S->t0, S->t1);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 1, S->X[1], false, S->t1, S->t0);
-  k_axis<<<nb, 256, 0, st>>>(n0, n1, n2, 0, S->X[0], false, S->t0, S->t1);
-  k_fe_interp<<<(unsigned)ctx->nelem, 128, 0, st>>>(D.qoff, D.xi, D.partoff, D.part_p,
-                                                    D.part_q, D.doff, D.dofs, S->t1, VC, D.err);
+  k_fe_load<<<(unsigned)ctx->nelem, SCF_NT, sm_load, st>>>(
+      D.qoff, D.w, D.xi, D.partoff, D.part_p, D.part_q, D.doff, D.dofs, O.n, rho_I, 4.0 * PI, pm,
+      S->b, S->sums);
+  k_axis<<<lines(n0), AX_NT, sm_ax, st>>>(n0, n1, n2, 0, nb, staged, S->X[0], true, S->b, S->t0,
+                                                    nullptr);
+  k_axis<<<lines(n1), AX_NT, sm_ax, st>>>(n0, n1, n2, 1, nb, staged, S->X[1], true, S->t0, S->t1,
+                                                    S->b);
+  k_axis_z<<<lines(n2), AX_NT, sm_ax, st>>>(n0, n1, n2, nb, staged, S->X[2], S->lam[0], S->lam[1],
+                                                      S->lam[2], S->t1, S->t0);
+  k_axis<<<lines(n1), AX_NT, sm_ax, st>>>(n0, n1, n2, 1, nb, staged, S->X[1], false, S->t0, S->t1,
+                                                    nullptr);
+  k_axis<<<lines(n0), AX_NT, sm_ax, st>>>(n0, n1, n2, 0, nb, staged, S->X[0], false, S->t1, S->t0,
+                                                    nullptr);
+  k_fe_interp<<<(unsigned)ctx->nelem, SCF_NT, sm_out, st>>>(
+      D.qoff, D.xi, D.partoff, D.part_p, D.part_q, D.doff, D.dofs, S->t0, pm, O);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
@@ -625,13 +732,12 @@ pufe_status launch_effective_potential(pufe_ctx *ctx, const double *n, const dou
                                        double *V_eff, double *V_C, double *eps_xc,
                                        cudaStream_t st) {
   if (pufe_status e0 = scf_prepare(ctx)) return e0;
-  ScfState *S = ctx->scf;
-  double *vc = V_C ? V_C : S->vc;
-  if (pufe_status e1 = coulomb(ctx, n, rho_I, vc, st)) return e1;
-  k_xc<<<blocks(ctx->nq, 256), 256, 0, st>>>(ctx->nq, n, eps_xc, S->vxc);
-  k_add<<<blocks(ctx->nq, 256), 256, 0, st>>>(ctx->nq, vc, S->vxc, V_eff);
-  PUFE_CUDA_TRY(cudaGetLastError());
-  return PUFE_OK;
+  InterpOut O{};
+  O.n = n;
+  O.V_eff = V_eff;
+  O.V_C = V_C;
+  O.eps_xc = eps_xc;
+  return coulomb(ctx, rho_I, O, st);
 }
 
 void scf_reset(pufe_ctx *ctx) {
@@ -751,14 +857,19 @@ static pufe_status scf_finish(pufe_ctx *ctx, double mu, double e_band, double ts
                               const double *V_eff_in, double *n, double *V_eff_out,
                               pufe_scf_info *info, cudaStream_t st) {
   ScfState *S = ctx->scf;
-  if (pufe_status e2 = coulomb(ctx, S->n_out, rho_I, S->vc, st)) return e2;
-  k_xc<<<blocks(ctx->nq, 256), 256, 0, st>>>(ctx->nq, S->n_out, S->exc, nullptr);
-  PUFE_CUDA_TRY(cudaMemsetAsync(S->sums, 0, 8 * sizeof(double), st));
   const bool use_pulay = pulay > 1;
-  k_energy_mix<<<blocks(ctx->nq, 256), 256, 0, st>>>(ctx->nq, ctx->d.w, S->n_out, V_eff_in, rho_I,
-                                                     S->vc, S->exc, use_pulay ? 0.0 : alpha, n,
-                                                     S->sums);
-  PUFE_CUDA_TRY(cudaGetLastError());
+  InterpOut O{};
+  O.n = S->n_out;
+  O.w = ctx->d.w;
+  O.V_in = V_eff_in;
+  O.rho_I = rho_I;
+  O.alpha = use_pulay ? 0.0 : alpha;
+  O.n_in = n;
+  O.sums = S->sums;
+  if (pufe_status e2 = coulomb(ctx, rho_I, O, st)) return e2;
+  // (before the second solve, which clears the sums)
+  PUFE_CUDA_TRY(cudaMemcpyAsync(S->h_sums, S->sums, SCF_SUMS * SCF_SLOTS * sizeof(double),
+                                cudaMemcpyDeviceToHost, st));
   if (use_pulay) {
     const int depth = std::min(pulay, PULAY_MAX);
     if (!S->hist_n) {
@@ -792,9 +903,12 @@ static pufe_status scf_finish(pufe_ctx *ctx, double mu, double e_band, double ts
   // the new effective potential of the mixed density
   if (pufe_status e3 = launch_effective_potential(ctx, n, rho_I, V_eff_out, nullptr, nullptr, st))
     return e3;
-  double sums[4];
-  PUFE_CUDA_TRY(cudaMemcpyAsync(sums, S->sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
   PUFE_CUDA_TRY(cudaStreamSynchronize(st));
+  double sums[SCF_SUMS];
+  for (int k = 0; k < SCF_SUMS; ++k) {
+    sums[k] = 0.0;
+    for (int i = 0; i < SCF_SLOTS; ++i) sums[k] += S->h_sums[k * SCF_SLOTS + i];
+  }
   if (info) {
     info->mu = mu;
     info->e_band = e_band;
