@@ -39,7 +39,8 @@ __device__ __forceinline__ void lag3(float t, float L[4]) {
 
 // BLOCH (Sec. 4, eqs. bloch, strong): entry (i, j) goes into H(k) and S(k)
 // with the phase conj(exp(i k.R_i)) exp(i k.R_j) of the columns' lattice
-// shifts, the constant overlap block included (S(k) has no k-independent part).
+// shifts; S holds the constant overlap of the Gamma point on entry and gets the
+// difference that the phases make.
 template <bool BLOCH>
 __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
     const int64_t *__restrict__ qoff, const double *__restrict__ w, const double *__restrict__ V,
@@ -117,17 +118,23 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
     if (!BLOCH) {
       atomicAdd(H + slot, __ldg(Tfe + o) + (double)v);
     } else {
+      // S starts as the summed constants, so only pairs whose phase is not 1 (the
+      // elements on the cell's upper faces) correct it; a zero imaginary part is
+      // not added (unless the value is not finite)
       const int ci = eshift[doff[e] + i], cj = eshift[doff[e] + j];
-      const double pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
-      const double pi = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
+      double pr = 1.0, pi = 0.0;
+      if (ci != cj) {
+        pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
+        pi = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
+      }
       if (what & PUFE_WANT_H) {
         const double hv = __ldg(Tfe + o) + (double)v;
         atomicAdd(H + slot, hv * pr);
-        atomicAdd(Hi + slot, hv * pi);
+        if (pi != 0.0 || !isfinite(hv)) atomicAdd(Hi + slot, hv * pi);
       }
-      if (what & PUFE_WANT_S) {
+      if ((what & PUFE_WANT_S) && ci != cj) {
         const double sv = __ldg(Sfe + o);
-        atomicAdd(S + slot, sv * pr);
+        atomicAdd(S + slot, sv * (pr - 1.0));
         atomicAdd(Si + slot, sv * pi);
       }
     }
@@ -180,7 +187,7 @@ __global__ void __launch_bounds__(SF_NT) k_adjoint_fefe(
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (o0 + u * SF_NT < 4096) Hs[o0 + u * SF_NT] = (float)h[u];
+      if (o0 + u * SF_NT < 4096) Hs[o0 + u * SF_NT] = f64_to_f32(h[u]);
   }
   for (int k = partoff[e]; k < partoff[e + 1]; ++k) {
     const int p = part_p[k];
@@ -255,7 +262,7 @@ pufe_status launch_fefe(pufe_ctx *ctx, const double *V, double *H, cudaStream_t 
 }
 
 // Bloch form: the FE-FE blocks of H(k) (if wanted; V == NULL means V = 0) and
-// S(k) (if wanted) with the column phases, into zeroed outputs
+// S(k) (if wanted) with the column phases, into zeroed H, Hi and Si and S = S0
 pufe_status launch_fefe_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *V, int what,
                               double *H, double *Hi, double *S, double *Si, cudaStream_t st) {
   auto &D = ctx->d;

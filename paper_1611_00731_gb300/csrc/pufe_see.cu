@@ -270,10 +270,10 @@ __global__ void __launch_bounds__(SE_NT) k_see(
           const double pr_ = s_phr[a] * s_phr[b] + s_phi[a] * s_phi[b];
           const double pi_ = s_phr[a] * s_phi[b] - s_phi[a] * s_phr[b];
           atomicAdd(S + s_rs, v * pr_);
-          atomicAdd(Si + s_rs, v * pi_);
-          if (r != s) {
-            atomicAdd(S + s_sr, v * pr_);
-            atomicAdd(Si + s_sr, -v * pi_);
+          if (r != s) atomicAdd(S + s_sr, v * pr_);
+          if (pi_ != 0.0) {   // (no phase inside the cell)
+            atomicAdd(Si + s_rs, v * pi_);
+            if (r != s) atomicAdd(Si + s_sr, -v * pi_);
           }
         } else {
           atomicAdd(S + s_rs, v);
@@ -401,10 +401,10 @@ __global__ void __launch_bounds__(SE_NT) k_see_gram(
         const double pr_ = s_phr[ca] * s_phr[cb] + s_phi[ca] * s_phi[cb];
         const double pi_ = s_phr[ca] * s_phi[cb] - s_phi[ca] * s_phr[cb];
         atomicAdd(S + s_rs, v * pr_);
-        atomicAdd(Si + s_rs, v * pi_);
-        if (r != sc) {
-          atomicAdd(S + s_sr, v * pr_);
-          atomicAdd(Si + s_sr, -v * pi_);
+        if (r != sc) atomicAdd(S + s_sr, v * pr_);
+        if (pi_ != 0.0) {   // (no phase inside the cell)
+          atomicAdd(Si + s_rs, v * pi_);
+          if (r != sc) atomicAdd(Si + s_sr, -v * pi_);
         }
       } else {
         atomicAdd(S + s_rs, v);

@@ -222,15 +222,19 @@ __device__ __forceinline__ void strip_part(const StripElem &E, double *__restric
       pair_phase(E, E.esh[i], E.esh[64 + r], pr, pi);
       if (E.wantH) {
         atomicAdd(H + s_ir, (double)(hs * pr));
-        atomicAdd(E.Hi + s_ir, (double)(hs * pi));
         atomicAdd(H + s_ri, (double)(hs * pr));
-        atomicAdd(E.Hi + s_ri, (double)(-hs * pi));
+        if (pi != 0.0f || !isfinite(hs)) {   // (a zero is not added: no phase inside the cell)
+          atomicAdd(E.Hi + s_ir, (double)(hs * pi));
+          atomicAdd(E.Hi + s_ri, (double)(-hs * pi));
+        }
       }
       if (E.wantS) {
         atomicAdd(S + s_ir, (double)(ss * pr));
-        atomicAdd(E.Si + s_ir, (double)(ss * pi));
         atomicAdd(S + s_ri, (double)(ss * pr));
-        atomicAdd(E.Si + s_ri, (double)(-ss * pi));
+        if (pi != 0.0f) {
+          atomicAdd(E.Si + s_ir, (double)(ss * pi));
+          atomicAdd(E.Si + s_ri, (double)(-ss * pi));
+        }
       }
     } else {
       if (E.wantH) {
@@ -412,13 +416,13 @@ __device__ __forceinline__ void strip_part(const StripElem &E, double *__restric
         const int g = dp.div(rest), qx = rest - g * p;
         const int b = bty & 3, ty = bty >> 2;
         const float c0s = ty ? hyy : -hyy;
+        // component b of the 1D factors of vertex bit t_y
+        const float *tf = reinterpret_cast<const float *>(MT) + b;
+        const int t0 = 8 * pm + 4 * ty, t1o = t0 + 24 * pm, t2o = 52 * pm;   // M, D, D0 on y
         float4 w1 = make_float4(0.f, 0.f, 0.f, 0.f), w3 = w1, ws = w1;
         const float4 *t1 = reinterpret_cast<const float4 *>(T1 + (size_t)(g * p2 + qx) * 36) + tz;
         for (int qy = 0; qy < p; ++qy, t1 += p * 9) {
-          const float4 m4 = MT[(pm + qy) * 2 + ty], d4 = DT[(pm + qy) * 2 + ty], o4 = D0T[pm + qy];
-          const float My = b == 0 ? m4.x : (b == 1 ? m4.y : (b == 2 ? m4.z : m4.w));
-          const float Dy = hy2 * (b == 0 ? d4.x : (b == 1 ? d4.y : (b == 2 ? d4.z : d4.w)));
-          const float Oy = c0s * (b == 0 ? o4.x : (b == 1 ? o4.y : (b == 2 ? o4.z : o4.w)));
+          const float My = tf[t0 + 8 * qy], Dy = hy2 * tf[t1o + 8 * qy], Oy = c0s * tf[t2o + 4 * qy];
           const float4 zs = t1[0], zx = t1[2], zy = t1[4], zv = t1[6];
           w1.x = fmaf(My, zv.x, fmaf(Dy, zy.x, fmaf(Oy, zs.x, w1.x)));
           w1.y = fmaf(My, zv.y, fmaf(Dy, zy.y, fmaf(Oy, zs.y, w1.y)));
@@ -537,15 +541,14 @@ __device__ __forceinline__ void strip_part(const StripElem &E, double *__restric
         int j0, f0, n;
         sp_yrow(a, j0, f0, n);
         const float *t1 = T1 + ((size_t)g * p2 + qx) * 24 + a;
-        const float *fy0 = Fy + f0 * pm, *fy1 = fy0 + pm, *fy2 = Fy + min(f0 + 2, 5) * pm,
-                    *fy3 = Fy + 3 * pm;
+        const float *fy0 = Fy + f0 * pm, *fy1 = fy0 + pm, *fy2 = Fy + min(f0 + 2, 5) * pm;
         float c0v = 0.0f, c1v = 0.0f, c2v = 0.0f, c3v = 0.0f;
         for (int qy = 0; qy < p; ++qy) {
           const float t = t1[qy * p * 24];
           c0v = fmaf(fy0[qy], t, c0v);
           c1v = fmaf(fy1[qy], t, c1v);
           c2v = fmaf(fy2[qy], t, c2v);
-          c3v = fmaf(fy3[qy], t, c3v);
+          c3v += t;   // (the factor 1)
         }
         float *t2 = T2 + (g * p + qx) * 66;
         t2[j0] = c0v;
@@ -561,15 +564,14 @@ __device__ __forceinline__ void strip_part(const StripElem &E, double *__restric
         int i0, f0, n;
         sp_xrow(j, i0, f0, n);
         const float *t2 = T2 + (size_t)g * p * 66 + j;
-        const float *fx0 = Fx + f0 * pm, *fx1 = fx0 + pm, *fx2 = Fx + min(f0 + 2, 5) * pm,
-                    *fx3 = Fx + 3 * pm;
+        const float *fx0 = Fx + f0 * pm, *fx1 = fx0 + pm, *fx2 = Fx + min(f0 + 2, 5) * pm;
         float c0v = 0.0f, c1v = 0.0f, c2v = 0.0f, c3v = 0.0f;
         for (int qx = 0; qx < p; ++qx) {
           const float t = t2[qx * 66];
           c0v = fmaf(fx0[qx], t, c0v);
           c1v = fmaf(fx1[qx], t, c1v);
           c2v = fmaf(fx2[qx], t, c2v);
-          c3v = fmaf(fx3[qx], t, c3v);
+          c3v += t;   // (the factor 1)
         }
         float *pe = E.PE + (c0 + g) * 189;
         pe[i0] += c0v;
@@ -892,17 +894,13 @@ __global__ void __maxnreg__(ST_MAXREG) k_strip_sf(
   const FastDiv dne(ne);
   if (E.sp) {   // entries from the pair projections (slot of r <= slot of s by symmetry)
     const float hx = 0.5f * sx, hy = 0.5f * sy, hz = 0.5f * sz;
-    const int A = E.A;
-    for (int o = tid; o < ne * ne; o += ST_NT) {
-      const int r = dne.div(o), sc = o - r * ne;
-      int cr = ecs[r], cs = ecs[sc];
-      if ((cr >> 3) > (cs >> 3)) {
-        const int t = cr;
-        cr = cs;
-        cs = t;
-      }
-      const int al = cr >> 3, be = cs >> 3;
-      const float *P = E.PE + (al * A - al * (al - 1) / 2 + (be - al)) * 189;
+    // one thread per (pair, vertex, vertex): an entry of two different slots goes into
+    // both triangles
+    for (int o = tid; o < E.npair * 64; o += ST_NT) {
+      const int g = o >> 6, pr2 = pairs[g], al = pr2 & 0xff, be = pr2 >> 8;
+      const int cr = (o >> 3) & 7, cs = o & 7, r = scol[al * 8 + cr], sc = scol[be * 8 + cs];
+      if (r < 0 || sc < 0) continue;
+      const float *P = E.PE + g * 189;
       const int bx = cr & 1, by = (cr >> 1) & 1, bz = (cr >> 2) & 1;
       const int cx = cs & 1, cy = (cs >> 1) & 1, cz = (cs >> 2) & 1;
       const float px = bx ? 1.0f : -1.0f, py = by ? 1.0f : -1.0f, pz = bz ? 1.0f : -1.0f;
@@ -919,16 +917,20 @@ __global__ void __maxnreg__(ST_MAXREG) k_strip_sf(
       h = fmaf(hy * qy, P[117 + (kz * 2 + by) * 3 + kx], h);
       h = fmaf(hz * pz, P[171 + (cz * 3 + ky) * 3 + kx], h);
       h = fmaf(hz * qz, P[153 + (bz * 3 + ky) * 3 + kx], h);
-      const int slot = E.m[(64 + r) * E.n + 64 + sc];
       const float hv = h * (1.0f / 64.0f);
-      if (BLOCH) {
-        float pr, pi;
-        pair_phase(E, E.esh[64 + r], E.esh[64 + sc], pr, pi);
-        atomicAdd(H + slot, (double)(hv * pr));
-        atomicAdd(E.Hi + slot, (double)(hv * pi));
-      } else {
-        atomicAdd(H + slot, (double)hv);
-      }
+      auto add = [&](int i, int j) {
+        const int slot = E.m[(64 + i) * E.n + 64 + j];
+        if (BLOCH) {
+          float pr, pi;
+          pair_phase(E, E.esh[64 + i], E.esh[64 + j], pr, pi);
+          atomicAdd(H + slot, (double)(hv * pr));
+          if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, (double)(hv * pi));
+        } else {
+          atomicAdd(H + slot, (double)hv);
+        }
+      };
+      add(r, sc);
+      if (al != be) add(sc, r);
     }
     return;
   }
@@ -941,7 +943,7 @@ __global__ void __maxnreg__(ST_MAXREG) k_strip_sf(
       pair_phase(E, E.esh[64 + r], E.esh[64 + sc], pr, pi);
       const float hv = E.HE[lo * ne8 + hi];
       atomicAdd(H + slot, (double)(hv * pr));
-      atomicAdd(E.Hi + slot, (double)(hv * pi));
+      if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, (double)(hv * pi));
     } else {
       atomicAdd(H + slot, (double)E.HE[lo * ne8 + hi]);
     }
@@ -1186,7 +1188,7 @@ pufe_status launch_assemble_mixed_bloch(pufe_ctx *ctx, const PhaseTab &ph, const
     PUFE_CUDA_TRY(cudaMemsetAsync(Hi, 0, bytes, st));
   }
   if (what & PUFE_WANT_S) {
-    PUFE_CUDA_TRY(cudaMemsetAsync(S, 0, bytes, st));
+    PUFE_CUDA_TRY(cudaMemcpyAsync(S, ctx->d.S0, bytes, cudaMemcpyDeviceToDevice, st));
     PUFE_CUDA_TRY(cudaMemsetAsync(Si, 0, bytes, st));
   }
   pufe_status e0 = launch_fefe_bloch(ctx, ph, V, what, H, Hi, S, Si, st);
@@ -1235,9 +1237,17 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
     const int32_t *__restrict__ partoff, const int32_t *__restrict__ part_p,
     const int32_t *__restrict__ part_q, const int64_t *__restrict__ soff,
     const int32_t *__restrict__ smap, const double *__restrict__ Hbar, int pm, int cfloats,
-    double *__restrict__ Vbar, unsigned *err, BlochCot bc) {
+    double *__restrict__ Vbar, unsigned *err, BlochCot bc, const int32_t *__restrict__ citems) {
   extern __shared__ float4 sm_aj4[];
-  const int e = order[blockIdx.x], tid = threadIdx.x;
+  // work item: element order[k0], its (sub)cells [cb, ce) (all of them without a
+  // list); ranges of one element write different points
+  int k0 = blockIdx.x, cb = 0, ce = 1 << 30;
+  if (citems) {
+    k0 = citems[3 * blockIdx.x];
+    cb = citems[3 * blockIdx.x + 1];
+    ce = citems[3 * blockIdx.x + 2];
+  }
+  const int e = order[k0], tid = threadIdx.x;
   const int n = (int)(doff[e + 1] - doff[e]);
   const int ne = n - 64;
   if (ne <= 0) return;   // FE-only element: Vbar is already complete
@@ -1318,7 +1328,8 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
         const int atx = 2 * (j & 3) + (v & 1), bty = 2 * ((j >> 2) & 3) + ((v >> 1) & 1),
                   ctz = 2 * (j >> 4) + (v >> 2);
         float *kk = K + (code >> 3) * 512 + ctz * 64 + bty * 8 + atx;
-        *kk = half ? *kk + (float)(0.125 * h[u]) : (float)(0.125 * h[u]);
+        const float hv = 0.125f * f64_to_f32(h[u]);   // (exact scaling)
+        *kk = half ? *kk + hv : hv;
       }
     }
     __syncthreads();
@@ -1346,7 +1357,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (o0 + u * AJ_NT < ne * ne) HE[o0 + u * AJ_NT] = (float)h[u];
+      if (o0 + u * AJ_NT < ne * ne) HE[o0 + u * AJ_NT] = f64_to_f32(h[u]);
   }
   __syncthreads();
   for (int o = tid; o < npair * 27; o += AJ_NT) {
@@ -1373,7 +1384,8 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
   }
 
   const int nsc_w = AJ_W;
-  for (int kp = partoff[e]; kp < partoff[e + 1]; ++kp) {
+  const int kend = min(partoff[e + 1], partoff[e] + ce);
+  for (int kp = partoff[e] + cb; kp < kend; ++kp) {
     const int p = part_p[kp], p2 = p * p, p3 = p2 * p, qs = part_q[kp];
     const FastDiv dp(p), dp2(p2);
     __syncthreads();   // coefficients ready; previous part's readers done
@@ -1516,9 +1528,15 @@ pufe_status launch_adjoint_strip_sf(pufe_ctx *ctx, const double *Hbar, double *V
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "adjoint strip: shared memory above 227 KB");
   auto kern = bc.Hi ? k_adjoint_strip_sf<true> : k_adjoint_strip_sf<false>;
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<(unsigned)count, AJ_NT, sm, st>>>(
-      D.order + first, D.qoff, D.qpoff, D.qdat, D.w, D.doff, D.ecol, D.aoff, D.toff32, D.psi32,
-      D.partoff, D.part_p, D.part_q, D.soff, D.smap, Hbar, pm, cf, Vbar, D.err, bc);
+  // all strip elements, some of them cut: over the (sub)cell-range list of the
+  // assembly's strip (its items index `order` from its start), so that an element of
+  // eight 8^3 cells is not one CTA's work (CsCl-like cell 183 -> 45 us)
+  const bool all = first == ctx->n_big && first + count == ctx->nelem && D.citems &&
+                   ctx->citems_cut;
+  kern<<<all ? (unsigned)ctx->n_citems : (unsigned)count, AJ_NT, sm, st>>>(
+      D.order + (all ? 0 : first), D.qoff, D.qpoff, D.qdat, D.w, D.doff, D.ecol, D.aoff, D.toff32,
+      D.psi32, D.partoff, D.part_p, D.part_q, D.soff, D.smap, Hbar, pm, cf, Vbar, D.err, bc,
+      all ? D.citems : nullptr);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
