@@ -870,6 +870,180 @@ __global__ void __launch_bounds__(DEN_NT) k_density_f32(
   }
 }
 
+// Density for many columns (64 to 128 real ones: states at Gamma, real and
+// imaginary parts at a wavevector), as a tiled product of the basis values of 128
+// points with the element's coefficients, both in shared memory: a thread owns 8
+// points x 8 columns, so four 16-byte reads feed 64 multiply-adds, where
+// k_density_f32 (one point and 8 columns per thread) reads two for 8 and is bound
+// by that (shared-memory wavefronts 88 % of their peak, FMA pipe 20 %); a basis
+// value is formed once per point instead of once per 8 columns.  The columns'
+// sums run over the basis in the same order as there, and one thread per point
+// then adds the columns' f psi^2 in that kernel's order, so the values are the
+// same bit for bit.  16 x CG threads (CG = columns / 8); two CTAs share an SM.
+// Fewer columns stay with k_density_f32: its CTAs need less shared memory, and
+// more of them hide the gather of the coefficients (CsCl-like cell, 40 columns:
+// 0.26 ms there against 0.49 ms for a tiled product).
+constexpr int DT_PT = 128;   // points per tile
+constexpr int DT_J = 64;     // basis columns per stage
+
+template <bool BLOCH>
+__global__ void __launch_bounds__(256, 2) k_density_tile_f32(
+    const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
+    const int64_t *__restrict__ qpoff, const float4 *__restrict__ qdat,
+    const int64_t *__restrict__ doff, const int32_t *__restrict__ dofs,
+    const int32_t *__restrict__ ecol, const int32_t *__restrict__ aoff,
+    const int64_t *__restrict__ toff32, const float *__restrict__ psi,
+    const double *__restrict__ C, int64_t ldc, const double *__restrict__ f, int nocc, int noccp,
+    double *__restrict__ rho, const int32_t *__restrict__ pitems, const double *__restrict__ Ci,
+    const uint8_t *__restrict__ eshift, PhaseTab ph) {
+  extern __shared__ __align__(16) float fsm[];
+  const int e = order[pitems[3 * blockIdx.x]];
+  const int qb = pitems[3 * blockIdx.x + 1];
+  const int64_t q0 = qoff[e];
+  const int Q = min((int)(qoff[e + 1] - q0), pitems[3 * blockIdx.x + 2]);
+  const int A = aoff[e + 1] - aoff[e];
+  const int n = (int)(doff[e + 1] - doff[e]);
+  const int ncol = noccp * (BLOCH ? 2 : 1), CG = ncol >> 3, NT = blockDim.x, tid = threadIdx.x;
+  const int32_t *ec = ecol + (doff[e] - 64ll * e);
+  const int32_t *dl = dofs + doff[e];
+  const uint8_t *es = eshift + doff[e];
+  const float *pe = psi + 4 * toff32[e];
+  const float4 *qe = qdat + qpoff[e];
+  float *Cs = fsm;                      // [n][ncol]
+  float *Ls = Cs + n * ncol;            // [12][DT_PT] 1D factors, then [8][DT_PT] PU values
+  float *fs = Ls + 20 * DT_PT;          // [ncol]
+  float *Bs = fs + ncol;                // [DT_J][DT_PT]; then [ncol / 2][DT_PT]
+  for (int k = tid; k < ncol; k += NT) fs[k] = (k % noccp < nocc) ? (float)f[k % noccp] : 0.0f;
+  {   // coefficients, a warp along the states of four columns at a time; columns of a
+      // zero lattice shift carry no phase
+    const int lane = tid & 31, nw = NT >> 5;
+    for (int j0 = tid >> 5; j0 < n; j0 += 4 * nw) {
+      int64_t g[4];
+      int cd[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = min(j0 + u * nw, n - 1);
+        g[u] = (int64_t)dl[j] * ldc;
+        cd[u] = BLOCH ? es[j] : 0;
+      }
+      for (int k = lane; k < noccp; k += 32) {
+        double ar[4], ai[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          ar[u] = k < nocc ? C[g[u] + k] : 0.0;
+          ai[u] = BLOCH && k < nocc ? Ci[g[u] + k] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = j0 + u * nw;
+          if (j >= n) break;
+          double cr = ar[u], ci = ai[u];
+          if (BLOCH && (cd[u] != 0 || !isfinite(cr) || !isfinite(ci))) {
+            cr = ph.re[cd[u]] * ar[u] - ph.im[cd[u]] * ai[u];
+            ci = ph.re[cd[u]] * ai[u] + ph.im[cd[u]] * ar[u];
+          }
+          Cs[j * ncol + k] = f64_to_f32(cr);
+          if (BLOCH) Cs[j * ncol + noccp + k] = f64_to_f32(ci);
+        }
+      }
+    }
+  }
+  const int pg = tid / CG, g = tid - pg * CG;
+  for (int t0 = qb; t0 < Q; t0 += DT_PT) {
+    const int np = min(DT_PT, Q - t0);
+    __syncthreads();
+    for (int t = tid; t < np; t += NT) {
+      const float4 x4 = qe[t0 + t];
+      const float xq[3] = {x4.x, x4.y, x4.z};
+      float L[4], dL[4];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        lagrange3f(xq[d], L, dL);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) Ls[(d * 4 + a) * DT_PT + t] = L[a];
+      }
+#pragma unroll
+      for (int lv = 0; lv < 8; ++lv) {
+        float p = 1.0f;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+          p *= ((lv >> d) & 1) ? 0.5f * (1.0f + xq[d]) : 0.5f * (1.0f - xq[d]);
+        Ls[(12 + lv) * DT_PT + t] = p;
+      }
+    }
+    float acc[8][8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) acc[x][y] = 0.0f;
+    const bool act = 8 * pg < np;
+    for (int jb = 0; jb < n; jb += DT_J) {
+      const int nj = min(DT_J, n - jb);
+      __syncthreads();
+      // (DT_J = 64: the first stage is the FE columns, four with one L_b L_c each)
+      if (jb == 0) {
+        for (int o = tid; o < 16 * DT_PT; o += NT) {
+          const int yz = o / DT_PT, t = o - yz * DT_PT;
+          const float *l = Ls + t;
+          const float lyz = l[(4 + (yz & 3)) * DT_PT] * l[(8 + (yz >> 2)) * DT_PT];
+          float *d = Bs + 4 * yz * DT_PT + t;
+#pragma unroll
+          for (int a = 0; a < 4; ++a) d[a * DT_PT] = t < np ? l[a * DT_PT] * lyz : 0.0f;
+        }
+      } else {
+        for (int o = tid; o < nj * DT_PT; o += NT) {
+          const int jj = o / DT_PT, t = o - jj * DT_PT, code = ec[jb + jj - 64], q = t0 + t;
+          Bs[o] = t < np ? Ls[(12 + (code & 7)) * DT_PT + t] *
+                               pe[((int64_t)(q >> 3) * A + (code >> 3)) * 32 + (q & 7)]
+                         : 0.0f;
+        }
+      }
+      __syncthreads();
+      if (act) {
+        const float *bp = Bs + 8 * pg, *cp = Cs + jb * ncol + 4 * g, *cq = cp + 4 * CG;
+#pragma unroll 2
+        for (int j = 0; j < nj; ++j) {
+          const float4 b0 = *reinterpret_cast<const float4 *>(bp + j * DT_PT);
+          const float4 b1 = *reinterpret_cast<const float4 *>(bp + j * DT_PT + 4);
+          const float4 u4 = *reinterpret_cast<const float4 *>(cp + j * ncol);
+          const float4 v4 = *reinterpret_cast<const float4 *>(cq + j * ncol);
+          const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+          const float c[8] = {u4.x, u4.y, u4.z, u4.w, v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+#pragma unroll
+            for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(b[x], c[y], acc[x][y]);
+        }
+      }
+    }
+    // the columns' sums to one thread per point, half of the columns at a time
+    float r = 0.0f;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      __syncthreads();
+      if (act) {
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          float4 *d = reinterpret_cast<float4 *>(Bs + (4 * g + y) * DT_PT + 8 * pg);
+          const int c = 4 * half + y;
+          d[0] = make_float4(acc[0][c], acc[1][c], acc[2][c], acc[3][c]);
+          d[1] = make_float4(acc[4][c], acc[5][c], acc[6][c], acc[7][c]);
+        }
+      }
+      __syncthreads();
+      if (tid < np) {
+        const float *fk = fs + half * 4 * CG;
+#pragma unroll 8
+        for (int k = 0; k < 4 * CG; ++k) {
+          const float a = Bs[k * DT_PT + tid];
+          r = fmaf(fk[k] * a, a, r);
+        }
+      }
+    }
+    if (tid < np) rho[q0 + t0 + tid] = (double)r;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // K5' (FP32): Vbar_q = w_q b_q^T Hbar_e b_q.  One CTA per element: Hbar_e
 // (gathered through the scatter map) and a chunk of 32 basis rows sit in
@@ -877,10 +1051,15 @@ __global__ void __launch_bounds__(DEN_NT) k_density_f32(
 // t_qi = sum_j Hbar_ij b_qj and stores its rows' sum of b_qi t_qi per point;
 // the row tiles' sums are then added in a fixed order.
 // ---------------------------------------------------------------------------
+//
+// The element block is gathered with eight (map, value) load chains in flight per
+// thread -- one after the other they took most of the kernel on a 184-function
+// element -- and the 1D factors of a chunk's points are formed once per point.
+// QB points per chunk: 64 (46 x 16 register tiles of such an element fill three
+// passes of 256 threads) where the block leaves room in shared memory, else 32.
 constexpr int ADJ_NT = 256;
-constexpr int ADJ_QB = 32;
 
-template <bool BLOCH>
+template <bool BLOCH, int ADJ_QB>
 __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
     const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
     const int64_t *__restrict__ qpoff, const float4 *__restrict__ qdat,
@@ -909,36 +1088,53 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
   float *Hs = fsm;                 // n4 x n4, zero padded
   float *Bq = Hs + n4 * n4;        // ADJ_QB x ldb
   float *part = Bq + ADJ_QB * ldb; // (n4 / 4) x ADJ_QB: each row tile's sum per point
-  for (int k = threadIdx.x; k < n4 * n4; k += ADJ_NT) {
-    const int i = k / n4, j = k - i * n4;
-    float v = 0.0f;
-    if (i < n && j < n) {
-      const int32_t sl = m[i * n + j];
-      v = BLOCH ? (float)cot_entry(Hbar[sl], bc.Hi[sl], bc.eshift[doff[e] + i],
-                                   bc.eshift[doff[e] + j], bc.ph)
-                : (float)Hbar[sl];
+  float *Lq = part + (n4 / 4) * ADJ_QB;   // 12 x ADJ_QB: 1D factors of the chunk's points
+  for (int k = threadIdx.x; k < n4 * n4; k += ADJ_NT) Hs[k] = 0.0f;   // the padding stays 0
+  __syncthreads();
+  for (int k0 = threadIdx.x; k0 < n * n; k0 += 8 * ADJ_NT) {
+    int32_t sl[8];
+    double h[8], hi[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sl[u] = k0 + u * ADJ_NT < n * n ? m[k0 + u * ADJ_NT] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) h[u] = k0 + u * ADJ_NT < n * n ? Hbar[sl[u]] : 0.0;
+    if (BLOCH) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) hi[u] = k0 + u * ADJ_NT < n * n ? bc.Hi[sl[u]] : 0.0;
     }
-    Hs[k] = v;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = k0 + u * ADJ_NT, i = k / n, j = k - i * n;
+      if (k >= n * n) break;
+      Hs[i * n4 + j] = BLOCH ? (float)cot_entry(h[u], hi[u], bc.eshift[doff[e] + i],
+                                                bc.eshift[doff[e] + j], bc.ph)
+                             : (float)h[u];
+    }
   }
   const int nI = n4 / 4;
   const int ntile = (ADJ_QB / 4) * nI;
   for (int qc = qbeg; qc < qend; qc += ADJ_QB) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < 3 * ADJ_QB; t += ADJ_NT) {
+      const int d = t / ADJ_QB, qq = t - d * ADJ_QB;
+      if (qc + qq >= qend) continue;
+      const float4 x4 = qe[qc + qq];
+      float L[4], dL[4];
+      lagrange3f(d == 0 ? x4.x : (d == 1 ? x4.y : x4.z), L, dL);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) Lq[(4 * d + a) * ADJ_QB + qq] = L[a];
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < ADJ_QB * n4; k += ADJ_NT) {
       const int qq = k / n4, c = k - qq * n4;
       const int q = qc + qq;
       float b = 0.0f;
       if (q < qend && c < n) {
-        const float4 x4 = qe[q];
         if (c < 64) {
-          float L[4], dL[4], v = 1.0f;
-          lagrange3f(x4.x, L, dL);
-          v *= L[c & 3];
-          lagrange3f(x4.y, L, dL);
-          v *= L[(c >> 2) & 3];
-          lagrange3f(x4.z, L, dL);
-          b = v * L[c >> 4];
+          const float v = Lq[(c & 3) * ADJ_QB + qq] * Lq[(4 + ((c >> 2) & 3)) * ADJ_QB + qq];
+          b = v * Lq[(8 + (c >> 4)) * ADJ_QB + qq];
         } else {
+          const float4 x4 = qe[q];
           const int code = ec[c - 64];
           const int lv = code & 7;
           const float phi = (((lv & 1) ? 1.0f + x4.x : 1.0f - x4.x) *
@@ -1279,6 +1475,19 @@ pufe_status launch_density_tc(pufe_ctx *ctx, const double *C, int64_t ldc, const
   const size_t sm = ((size_t)ctx->max_basis * noccp * (Ci ? 2 : 1) + noccp) * sizeof(float);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "density: basis x states beyond shared memory");
   if (Ci && !ph) return fail(PUFE_EINVAL, "internal: Bloch density without phases");
+  // 64 to 128 real columns: the tiled product, where its tiles fit shared memory
+  const int ncol = noccp * (Ci ? 2 : 1);
+  const size_t st_sm =
+      ((size_t)ctx->max_basis * ncol + 20 * DT_PT + ncol + DT_J * DT_PT) * sizeof(float);
+  if (ncol >= 64 && ncol <= 128 && st_sm <= 227 * 1024 && ctx->n_pitems > 0) {
+    auto kt = Ci ? k_density_tile_f32<true> : k_density_tile_f32<false>;
+    PUFE_CUDA_TRY(cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st_sm));
+    kt<<<(unsigned)ctx->n_pitems, 2 * ncol, st_sm, st>>>(
+        D.order, D.qoff, D.qpoff, D.qdat, D.doff, D.dofs, D.ecol, D.aoff, D.toff32, D.psi32, C,
+        ldc, f, nocc, noccp, rho, D.pitems, Ci, D.eshift, ph ? *ph : PhaseTab{});
+    PUFE_CUDA_TRY(cudaGetLastError());
+    return PUFE_OK;
+  }
   auto kern = Ci ? k_density_f32<true> : k_density_f32<false>;
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   if (ctx->n_pitems <= 0) return PUFE_OK;
@@ -1297,10 +1506,15 @@ pufe_status launch_adjoint_tc(pufe_ctx *ctx, const double *Hbar, double *Vbar, c
   if (nbig > 0) {  // n_e > 128: FP32 CUDA-core kernel
     const int n4 = (ctx->max_basis + 3) & ~3;
     const int ldb = n4 + 36;
-    const size_t sm = ((size_t)n4 * n4 + (size_t)ADJ_QB * ldb + (size_t)(n4 / 4) * ADJ_QB) *
-                      sizeof(float);
-    if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e too large for the FP32 adjoint kernel");
-    auto kern = bc.Hi ? k_adjoint_f32<true> : k_adjoint_f32<false>;
+    auto need = [&](int qb) {
+      return ((size_t)n4 * n4 + (size_t)qb * ldb + (size_t)(n4 / 4) * qb + 12 * qb) * sizeof(float);
+    };
+    const bool wide = need(64) <= 227 * 1024;
+    const size_t sm = need(wide ? 64 : 32);
+    if (sm > 227 * 1024)
+      return fail(PUFE_EINVAL, "n_e too large for the FP32 adjoint kernel");
+    auto kern = wide ? (bc.Hi ? k_adjoint_f32<true, 64> : k_adjoint_f32<false, 64>)
+                     : (bc.Hi ? k_adjoint_f32<true, 32> : k_adjoint_f32<false, 32>);
     PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     kern<<<ctx->n_titems, ADJ_NT, sm, st>>>(D.order, D.qoff, D.qpoff, D.qdat, D.w,
                                                      D.doff, D.ecol, D.aoff, D.toff32, D.psi32,

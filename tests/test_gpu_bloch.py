@@ -264,3 +264,32 @@ def test_mixed_bloch_gram_form_of_the_EE_overlap_block():
     ee = float(abs(D).max() / abs(So.tocsr()[nfe:, nfe:]).max())
     print(f"\nGram form at k: S E-E block {ee:.1e}")
     assert ee < 5e-6
+
+
+@pytest.mark.parametrize("nocc", [16, 17, 64])
+def test_mixed_density_of_many_states(nocc):
+    """The FP32 density of 32 to 128 real columns (its tiled product): at a
+    wavevector and, with twice the states where the call takes them, at the Gamma
+    point, on elements of 8^3 and 4^3 points; 1e-5 of the largest value, the mixed
+    density's bound elsewhere."""
+    from oracle import assemble as oasm
+    wl = dict(W.workload("c1_two_atom_4cube"), nel=5)   # rules of both orders, up to 104 functions
+    m = omesh.Mesh(wl)
+    rules = oq.all_rules(m)
+    ctx = pufe.pufe_build_mesh(wl)
+    ctx.pufe_tabulate(pufe.PUFE_TF32X3)
+    k = 2.0 * math.pi / wl["a"] * K_FRAC
+    dev = torch.device("cuda:0")
+    Cr, Ci = (W.random_coefficients(ctx.n_dof, nocc, seed=s) for s in (31, 32))
+    f = W.random_occupations(nocc, seed=33)
+    rho = torch.empty(ctx.n_q, dtype=torch.float64, device=dev)
+    ctx.pufe_density_bloch(k, torch.tensor(Cr, device=dev), torch.tensor(Ci, device=dev),
+                           torch.tensor(f, device=dev), rho, prec=pufe.PUFE_TF32X3)
+    ctx.pufe_sync_status()
+    assert _rel(rho.cpu().numpy(), ob.density_k(m, rules, Cr + 1j * Ci, f, k)) < 1e-5
+    n2 = min(64, 2 * nocc)
+    Cm, f2 = W.random_coefficients(ctx.n_dof, n2, seed=34), W.random_occupations(n2, seed=35)
+    ctx.pufe_density(torch.tensor(Cm, device=dev), torch.tensor(f2, device=dev), rho,
+                     prec=pufe.PUFE_TF32X3)
+    ctx.pufe_sync_status()
+    assert _rel(rho.cpu().numpy(), oasm.density(m, rules, Cm, f2)) < 1e-5
