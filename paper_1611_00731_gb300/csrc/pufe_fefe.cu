@@ -41,6 +41,15 @@ __device__ __forceinline__ void lag3(float t, float L[4]) {
 // with the phase conj(exp(i k.R_i)) exp(i k.R_j) of the columns' lattice
 // shifts; S holds the constant overlap of the Gamma point on entry and gets the
 // difference that the phases make.
+//
+// What bounded it before: shared memory sized for 16 points per axis (39 KB, five
+// 128-thread CTAs per SM), one output per loop turn (three instructions per
+// multiply-add) and the widening of each entry on the FP64 pipe (two per clock and SM).
+// Now a thread owns a line of each stage with five or ten outputs, shared memory
+// follows the largest rule (12 KB at 8 points: 40 registers bind, 12 CTAs per SM) and
+// entries are widened on the integer pipe; what is left is the 7 M atomics.
+// 12^3 rocksalt (ncu) 59 -> 34 us; at a wavevector, where elements away from the upper
+// faces skip phases that are 1, 64-atom cell 2.41 -> 1.26 ms.
 template <bool BLOCH>
 __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
     const int64_t *__restrict__ qoff, const double *__restrict__ w, const double *__restrict__ V,
@@ -50,17 +59,28 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
     const int32_t *__restrict__ smap, const double *__restrict__ Tfe, double *__restrict__ H,
     unsigned *err, const double *__restrict__ Sfe, const uint8_t *__restrict__ eshift,
     PhaseTab ph, int what, double *__restrict__ Hi, double *__restrict__ S,
-    double *__restrict__ Si) {
-  __shared__ float Wq[SF_PMAX * SF_PMAX * SF_PMAX];
-  __shared__ float P[3][10][SF_PMAX];          // pair products per axis
-  __shared__ float G1[SF_PMAX * SF_PMAX * 10];  // [qx + p qy][cc]
-  __shared__ float G2[SF_PMAX * 100];           // [qx][bb * 10 + cc]
-  __shared__ float M[1000];
+    double *__restrict__ Si, int pm) {
+  // dynamic shared memory, sized for the largest per-axis count pm: P[3][pm][16], the 10
+  // pair products of each axis and point as two halves of five (pitch 8); Wq[pm^3];
+  // G1[qx + p qy][cc]; G2[qx][bb][cc]; M[aa][bb][cc]
+  extern __shared__ __align__(16) float sm_ff[];
+  float *P = sm_ff, *G2 = P + 48 * pm, *M = G2 + 100 * pm, *G1 = M + 1000, *Wq = G1 + 10 * pm * pm;
   const int e = blockIdx.x, tid = threadIdx.x;
-  for (int o = tid; o < 1000; o += SF_NT) M[o] = 0.0f;
+  float m10[10];   // this thread's (bb, cc) at every aa
+#pragma unroll
+  for (int a = 0; a < 10; ++a) m10[a] = 0.0f;
+  // acc[u] += f v over the five products of one half at one point
+  auto five = [](const float *f, float v, float *acc) {
+    const float4 f4 = *reinterpret_cast<const float4 *>(f);
+    acc[0] = fmaf(v, f4.x, acc[0]);
+    acc[1] = fmaf(v, f4.y, acc[1]);
+    acc[2] = fmaf(v, f4.z, acc[2]);
+    acc[3] = fmaf(v, f4.w, acc[3]);
+    acc[4] = fmaf(v, f[4], acc[4]);
+  };
   for (int k = partoff[e]; V != nullptr && k < partoff[e + 1]; ++k) {
     const int p = part_p[k];
-    if (p > SF_PMAX) {
+    if (p > pm) {
       if (tid == 0) atomicOr(err, DEVERR_SHAPE);
       return;
     }
@@ -71,7 +91,7 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
     for (int q = tid; q < p3; q += SF_NT) {
       const double v = V[qs + q];
       bad |= !isfinite(v);
-      Wq[q] = (float)(w[qs + q] * v);
+      Wq[q] = f64_to_f32(w[qs + q] * v);
     }
     if (bad) atomicOr(err, DEVERR_NONFINITE);
     for (int o = tid; o < 3 * p; o += SF_NT) {
@@ -79,63 +99,95 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
       const int stride = d == 0 ? 1 : (d == 1 ? p : p2);
       float L[4];
       lag3((float)xi_all[3 * (qs + (int64_t)t * stride) + d], L);
+      float *f = P + (d * pm + t) * 16;
       int c = 0;
+#pragma unroll
       for (int a = 0; a < 4; ++a)
-        for (int b = a; b < 4; ++b) P[d][c++][t] = L[a] * L[b];
+#pragma unroll
+        for (int b = a; b < 4; ++b, ++c) f[c < 5 ? c : c + 3] = L[a] * L[b];
     }
     __syncthreads();
-    for (int o = tid; o < p2 * 10; o += SF_NT) {  // contract z
-      const int qxy = o / 10, cc = o - qxy * 10;
-      float s = 0.0f;
-      for (int qz = 0; qz < p; ++qz) s = fmaf(Wq[qxy + p2 * qz], P[2][cc][qz], s);
-      G1[o] = s;
+    for (int o = tid; o < 2 * p2; o += SF_NT) {   // contract z: (half of cc, qx + p qy)
+      const int h = o >= p2, qxy = o - h * p2;
+      const float *f = P + 2 * pm * 16 + 8 * h;
+      float s[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      for (int qz = 0; qz < p; ++qz) five(f + 16 * qz, Wq[qxy + p2 * qz], s);
+#pragma unroll
+      for (int u = 0; u < 5; ++u) G1[qxy * 10 + 5 * h + u] = s[u];
     }
     __syncthreads();
-    for (int o = tid; o < p * 100; o += SF_NT) {  // contract y
-      const int qx = o / 100, r = o - qx * 100, bb = r / 10, cc = r - bb * 10;
-      float s = 0.0f;
-      for (int qy = 0; qy < p; ++qy) s = fmaf(P[1][bb][qy], G1[(qx + p * qy) * 10 + cc], s);
-      G2[o] = s;
+    for (int o = tid; o < 20 * p; o += SF_NT) {   // contract y: (half of bb, qx, cc)
+      const int h = o >= 10 * p, r = o - h * 10 * p, qx = r / 10, cc = r - qx * 10;
+      const float *f = P + pm * 16 + 8 * h;
+      float s[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      for (int qy = 0; qy < p; ++qy) five(f + 16 * qy, G1[qy * p * 10 + r], s);
+#pragma unroll
+      for (int u = 0; u < 5; ++u) G2[qx * 100 + (5 * h + u) * 10 + cc] = s[u];
     }
     __syncthreads();
-    for (int o = tid; o < 1000; o += SF_NT) {  // contract x
-      const int aa = o / 100, r = o - aa * 100;
-      float s = 0.0f;
-      for (int qx = 0; qx < p; ++qx) s = fmaf(P[0][aa][qx], G2[qx * 100 + r], s);
-      M[o] += s;
+    if (tid < 100) {   // contract x: (bb, cc)
+      float s[10];
+#pragma unroll
+      for (int a = 0; a < 10; ++a) s[a] = 0.0f;
+      for (int qx = 0; qx < p; ++qx) {
+        const float g = G2[qx * 100 + tid];
+        five(P + 16 * qx, g, s);
+        five(P + 16 * qx + 8, g, s + 5);
+      }
+#pragma unroll
+      for (int a = 0; a < 10; ++a) m10[a] += s[a];
     }
   }
+  if (tid < 100) {
+#pragma unroll
+    for (int a = 0; a < 10; ++a) M[a * 100 + tid] = m10[a];
+  }
   __syncthreads();
-  // add the 64 x 64 block into H through the scatter map: thread pairs
-  // (i, j) run along j, so consecutive lanes hit neighbouring CSR columns
+  // add the 64 x 64 block into H through the scatter map: consecutive lanes run along
+  // j and hit neighbouring CSR columns; a thread keeps its j, so its M offsets are one
+  // per node of each axis
   const int n = (int)(doff[e + 1] - doff[e]);
   const int32_t *m = smap + soff[e];
-  for (int o = tid; o < 64 * 64; o += SF_NT) {
-    const int i = o >> 6, j = o & 63;
-    const float v = M[pidx(i & 3, j & 3) * 100 + pidx((i >> 2) & 3, (j >> 2) & 3) * 10 +
-                      pidx(i >> 4, j >> 4)];
-    const int slot = m[i * n + j];
-    if (!BLOCH) {
-      atomicAdd(H + slot, __ldg(Tfe + o) + (double)v);
-    } else {
-      // S starts as the summed constants, so only pairs whose phase is not 1 (the
-      // elements on the cell's upper faces) correct it; a zero imaginary part is
-      // not added (unless the value is not finite)
-      const int ci = eshift[doff[e] + i], cj = eshift[doff[e] + j];
-      double pr = 1.0, pi = 0.0;
-      if (ci != cj) {
-        pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
-        pi = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
-      }
-      if (what & PUFE_WANT_H) {
-        const double hv = __ldg(Tfe + o) + (double)v;
-        atomicAdd(H + slot, hv * pr);
-        if (pi != 0.0 || !isfinite(hv)) atomicAdd(Hi + slot, hv * pi);
-      }
-      if ((what & PUFE_WANT_S) && ci != cj) {
-        const double sv = __ldg(Sfe + o);
-        atomicAdd(S + slot, sv * (pr - 1.0));
-        atomicAdd(Si + slot, sv * pi);
+  const int j = tid & 63, ih = tid >> 6;
+  // most elements touch no upper face of the cell: every phase is 1
+  const uint8_t *es = BLOCH ? eshift + doff[e] : nullptr;
+  const bool phased = BLOCH && __syncthreads_or(tid < 64 ? es[tid] : 0) != 0;
+  int pa[2], pb[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (u < 2) pa[u] = pidx(ih + 2 * u, j & 3) * 100;
+    pb[u] = pidx(u, (j >> 2) & 3) * 10;
+  }
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const int pc = pidx(c, j >> 4);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = 16 * c + 2 * u + ih, o = i * 64 + j;
+      const double v = f32_to_f64(M[pa[u & 1] + pb[u >> 1] + pc]);
+      const int slot = m[i * n + j];
+      if (!BLOCH) {
+        atomicAdd(H + slot, __ldg(Tfe + o) + v);
+      } else {
+        // S starts as the summed constants, so only pairs whose phase is not 1 (the
+        // elements on the cell's upper faces) correct it; a zero imaginary part is
+        // not added (unless the value is not finite)
+        const int ci = phased ? es[i] : 0, cj = phased ? es[j] : 0;
+        double pr = 1.0, pi = 0.0;
+        if (ci != cj) {
+          pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
+          pi = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
+        }
+        if (what & PUFE_WANT_H) {
+          const double hv = __ldg(Tfe + o) + v;
+          atomicAdd(H + slot, ci != cj ? hv * pr : hv);
+          if (pi != 0.0 || !isfinite(hv)) atomicAdd(Hi + slot, hv * pi);
+        }
+        if ((what & PUFE_WANT_S) && ci != cj) {
+          const double sv = __ldg(Sfe + o);
+          atomicAdd(S + slot, sv * (pr - 1.0));
+          atomicAdd(Si + slot, sv * pi);
+        }
       }
     }
   }
@@ -146,8 +198,32 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
 // (Hbar restricted to the element's 64 FE columns, general, not symmetric),
 // contracted axis by axis: 4096 p + 256 p^2 + 16 p^3 multiply-adds per cell,
 // then Vbar_q = w_q f(q) is stored (the strip kernel adds the enrichment part).
+//
+// What bounded a form with one output per loop turn was its instructions: two products
+// and three shared-memory reads per multiply-add, beside the gather.  Here a thread
+// owns a row of each stage and runs over the points: its 16 inputs stay in registers
+// (for z, the 16 gathered entries themselves, through all (sub)cells), and the 16
+// factors L_i L_i' of a point, formed once per cell, are four 16-byte reads that all
+// lanes share.  The 16 terms keep their order.  12^3 rocksalt (ncu) 40 -> 30 us.
+constexpr int AF_NT = 256;     // one thread per ((a, b), (a', b')) row
+constexpr int AF_ROW = 20;     // pitches of G1 (of a row of 16, and of a qz) that keep the
+constexpr int AF_QZ = 336;     // y stage's reads on different banks
+
+__device__ __forceinline__ float af_sum(const float (&v)[16], const float4 *l) {
+  float s = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float4 f = l[c];
+    s = fmaf(f.x, v[4 * c], s);
+    s = fmaf(f.y, v[4 * c + 1], s);
+    s = fmaf(f.z, v[4 * c + 2], s);
+    s = fmaf(f.w, v[4 * c + 3], s);
+  }
+  return s;
+}
+
 template <bool BLOCH>
-__global__ void __launch_bounds__(SF_NT) k_adjoint_fefe(
+__global__ void __launch_bounds__(AF_NT, 4) k_adjoint_fefe(
     const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
     const double *__restrict__ w, const double *__restrict__ xi_all,
     const int32_t *__restrict__ partoff, const int32_t *__restrict__ part_p,
@@ -156,38 +232,40 @@ __global__ void __launch_bounds__(SF_NT) k_adjoint_fefe(
     const double *__restrict__ Hbar, int pm, double *__restrict__ Vbar, unsigned *err,
     BlochCot bc) {
   // dynamic shared memory, sized for the largest per-axis count pm:
-  // Hs[64][64], L1[3][4][pm], G1[256 pm] = [(a,b),(a',b')][qz],
-  // G2[16 pm^2] = [(a,a')][qy + p qz]
-  extern __shared__ float sm_adj[];
-  float *Hs = sm_adj, *L1 = Hs + 4096, *G1 = L1 + 12 * pm, *G2 = G1 + 256 * pm;
+  // LL[3][pm][16] = L_i L_i', G1[qz][(a,b)][(a',b')], G2[(a,a')][qy + p qz]
+  extern __shared__ __align__(16) float sm_adj[];
+  float4 *LL = reinterpret_cast<float4 *>(sm_adj);
+  float *G1 = sm_adj + 48 * pm, *G2 = G1 + AF_QZ * pm;
   const int e = order[blockIdx.x], tid = threadIdx.x;
   const int n = (int)(doff[e + 1] - doff[e]);
   const int32_t *m = smap + soff[e];
-  // gather with eight independent (map, value) load chains in flight per thread
-  for (int o0 = tid; o0 < 4096; o0 += 8 * SF_NT) {
+  const int ab = tid >> 4, apbp = tid & 15;
+  // this row's entries, (c, c') = 0..15: eight independent (map, value) load chains
+  // in flight
+  float hz[16];
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
     int s1[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int o = o0 + u * SF_NT;
-      s1[u] = o < 4096 ? m[(o >> 6) * n + (o & 63)] : 0;
+      const int c = 2 * g + (u >> 2), cp = u & 3;
+      s1[u] = m[(ab + 16 * c) * n + apbp + 16 * cp];
     }
     double h[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) h[u] = o0 + u * SF_NT < 4096 ? Hbar[s1[u]] : 0.0;
+    for (int u = 0; u < 8; ++u) h[u] = Hbar[s1[u]];
     if (BLOCH) {   // at a wavevector: the phased real part (columns' shift codes)
       double hi[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) hi[u] = o0 + u * SF_NT < 4096 ? bc.Hi[s1[u]] : 0.0;
+      for (int u = 0; u < 8; ++u) hi[u] = bc.Hi[s1[u]];
       const uint8_t *esh = bc.eshift + doff[e];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int o = o0 + u * SF_NT;
-        if (o < 4096) h[u] = cot_entry(h[u], hi[u], esh[o >> 6], esh[o & 63], bc.ph);
-      }
+      for (int u = 0; u < 8; ++u)
+        h[u] = cot_entry(h[u], hi[u], esh[ab + 16 * (2 * g + (u >> 2))],
+                         esh[apbp + 16 * (u & 3)], bc.ph);
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (o0 + u * SF_NT < 4096) Hs[o0 + u * SF_NT] = f64_to_f32(h[u]);
+    for (int u = 0; u < 8; ++u) hz[8 * g + u] = f64_to_f32(h[u]);
   }
   for (int k = partoff[e]; k < partoff[e + 1]; ++k) {
     const int p = part_p[k];
@@ -196,54 +274,54 @@ __global__ void __launch_bounds__(SF_NT) k_adjoint_fefe(
       return;
     }
     const int64_t qs = qoff[e] + part_q[k];
-    const int p2 = p * p, p3 = p2 * p;
+    const int p2 = p * p;
     __syncthreads();
-    for (int o = tid; o < 3 * p; o += SF_NT) {
+    for (int o = tid; o < 3 * p; o += AF_NT) {
       const int d = o / p, t = o - d * p;
       const int stride = d == 0 ? 1 : (d == 1 ? p : p2);
       float L[4];
       lag3((float)xi_all[3 * (qs + (int64_t)t * stride) + d], L);
-      for (int a = 0; a < 4; ++a) L1[(d * 4 + a) * pm + t] = L[a];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        LL[(d * pm + t) * 4 + a] = make_float4(L[a] * L[0], L[a] * L[1], L[a] * L[2], L[a] * L[3]);
     }
     __syncthreads();
-    // contract (c, c') for each qz: G1[(a,b),(a',b')][qz]
-    for (int o = tid; o < 256 * p; o += SF_NT) {
-      const int pr = o / p, qz = o - pr * p;
-      const int ab = pr >> 4, apbp = pr & 15;   // (a + 4b), (a' + 4b')
-      float s = 0.0f;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int cp = 0; cp < 4; ++cp)
-          s = fmaf(L1[(8 + c) * pm + qz] * L1[(8 + cp) * pm + qz], Hs[(ab + 16 * c) * 64 + apbp + 16 * cp], s);
-      G1[o] = s;
-    }
+    // contract (c, c'): a thread's row at every qz
+    for (int qz = 0; qz < p; ++qz)
+      G1[qz * AF_QZ + ab * AF_ROW + apbp] = af_sum(hz, LL + (2 * pm + qz) * 4);
     __syncthreads();
-    // contract (b, b') for each (qy, qz): G2[(a,a')][qy + p qz]
-    for (int o = tid; o < 16 * p2; o += SF_NT) {
-      const int aa = o / p2, r = o - aa * p2, qy = r % p, qz = r / p;
-      const int a = aa >> 2, ap = aa & 3;
-      float s = 0.0f;
+    // contract (b, b'): rows (a, a', qz), their qy spread over ny threads
+    const int ny = max(1, AF_NT / (16 * p));
+    if (tid < 16 * p * ny) {
+      const int aa = tid & 15, sq = tid >> 4, sp = sq / p, qz = sq - sp * p;
+      const float *g = G1 + qz * AF_QZ + (aa >> 2) * AF_ROW + (aa & 3);
+      float v[16];
 #pragma unroll
       for (int b = 0; b < 4; ++b)
 #pragma unroll
-        for (int bp = 0; bp < 4; ++bp)
-          s = fmaf(L1[(4 + b) * pm + qy] * L1[(4 + bp) * pm + qy], G1[((a + 4 * b) * 16 + ap + 4 * bp) * p + qz], s);
-      G2[o] = s;
+        for (int bp = 0; bp < 4; ++bp) v[4 * b + bp] = g[4 * b * AF_ROW + 4 * bp];
+      for (int qy = sp; qy < p; qy += ny)
+        G2[aa * p2 + qy + p * qz] = af_sum(v, LL + (pm + qy) * 4);
     }
     __syncthreads();
-    // contract (a, a') for each point, store w_q f(q)
-    for (int q = tid; q < p3; q += SF_NT) {
-      const int qx = q % p, r = q / p;
-      float s = 0.0f;
+    // contract (a, a'): lines (qy, qz), their qx spread over nx threads; w_q f(q)
+    const int nx = min(p, AF_NT / p2);
+    if (tid < p2 * nx) {
+      const int sp = tid / p2, r = tid - sp * p2;
+      float v[16];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int ap = 0; ap < 4; ++ap)
-          s = fmaf(L1[a * pm + qx] * L1[ap * pm + qx], G2[(a * 4 + ap) * p2 + r], s);
-      Vbar[qs + q] = w[qs + q] * (double)s;
+      for (int a = 0; a < 16; ++a) v[a] = G2[a * p2 + r];
+      for (int qx = sp; qx < p; qx += nx) {
+        const int64_t q = qs + qx + p * r;
+        Vbar[q] = w[q] * f32_to_f64(af_sum(v, LL + qx * 4));
+      }
     }
   }
+}
+
+// shared bytes of k_fefe_sumfac (40 KB at the 16 points per axis that the callers allow)
+size_t fefe_bytes(int pm) {
+  return (size_t)(148 * pm + 1000 + 10 * pm * pm + pm * pm * pm) * sizeof(float);
 }
 
 }  // namespace
@@ -254,9 +332,10 @@ pufe_status launch_fefe(pufe_ctx *ctx, const double *V, double *H, cudaStream_t 
   auto &D = ctx->d;
   if (ctx->max_part_p > SF_PMAX) return fail(PUFE_EINVAL, "rule with more than 16 points per axis");
   if (!D.Tfe) return fail(PUFE_ESTATE, "no exact FE-FE blocks (a rule has < 4 points per axis)");
-  k_fefe_sumfac<false><<<(unsigned)ctx->nelem, SF_NT, 0, st>>>(
+  const int pm = std::max(1, ctx->max_part_p);
+  k_fefe_sumfac<false><<<(unsigned)ctx->nelem, SF_NT, fefe_bytes(pm), st>>>(
       D.qoff, D.w, V, D.xi, D.partoff, D.part_p, D.part_q, D.doff, D.soff, D.smap, D.Tfe, H, D.err,
-      nullptr, nullptr, PhaseTab{}, PUFE_WANT_H, nullptr, nullptr, nullptr);
+      nullptr, nullptr, PhaseTab{}, PUFE_WANT_H, nullptr, nullptr, nullptr, pm);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
@@ -268,9 +347,10 @@ pufe_status launch_fefe_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *V
   auto &D = ctx->d;
   if (ctx->max_part_p > SF_PMAX) return fail(PUFE_EINVAL, "rule with more than 16 points per axis");
   if (!D.Tfe || !D.Sfe) return fail(PUFE_ESTATE, "no exact FE-FE blocks (a rule has < 4 points per axis)");
-  k_fefe_sumfac<true><<<(unsigned)ctx->nelem, SF_NT, 0, st>>>(
+  const int pm = std::max(1, ctx->max_part_p);
+  k_fefe_sumfac<true><<<(unsigned)ctx->nelem, SF_NT, fefe_bytes(pm), st>>>(
       D.qoff, D.w, (what & PUFE_WANT_H) ? V : nullptr, D.xi, D.partoff, D.part_p, D.part_q,
-      D.doff, D.soff, D.smap, D.Tfe, H, D.err, D.Sfe, D.eshift, ph, what, Hi, S, Si);
+      D.doff, D.soff, D.smap, D.Tfe, H, D.err, D.Sfe, D.eshift, ph, what, Hi, S, Si, pm);
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
@@ -285,10 +365,10 @@ pufe_status launch_adjoint_fefe(pufe_ctx *ctx, const double *Hbar, double *Vbar,
   if (ctx->max_part_p > SF_PMAX) return fail(PUFE_EINVAL, "rule with more than 16 points per axis");
   if (count <= 0) return PUFE_OK;
   const int pm = std::max(1, ctx->max_part_p);
-  const size_t sm = (size_t)(4096 + 12 * pm + 256 * pm + 16 * pm * pm) * sizeof(float);
+  const size_t sm = (size_t)((48 + AF_QZ) * pm + 16 * pm * pm) * sizeof(float);
   auto kern = bc.Hi ? k_adjoint_fefe<true> : k_adjoint_fefe<false>;
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<(unsigned)count, SF_NT, sm, st>>>(D.order + first, D.qoff, D.w, D.xi, D.partoff, D.part_p,
+  kern<<<(unsigned)count, AF_NT, sm, st>>>(D.order + first, D.qoff, D.w, D.xi, D.partoff, D.part_p,
                                            D.part_q, D.doff, D.soff, D.smap, Hbar, pm, Vbar, D.err,
                                            bc);
   PUFE_CUDA_TRY(cudaGetLastError());

@@ -436,6 +436,13 @@ __device__ __forceinline__ float f64_to_f32(double x) {
   r += (rem > 0x10000000u || (rem == 0x10000000u && (r & 1u))) ? 1u : 0u;
   return __uint_as_float(r | (hi & 0x80000000u));
 }
+// FP32 -> FP64 (exact) the same way, for the entries added into FP64 values
+__device__ __forceinline__ double f32_to_f64(float x) {
+  const unsigned u = __float_as_uint(x), ex = (u >> 23) & 0xffu;
+  if (ex - 1u > 253u) return (u << 1) ? (double)x : __hiloint2double((int)u, 0);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u)),
+                          (int)(u << 29));
+}
 #endif
 
 // launchers implemented in the .cu files

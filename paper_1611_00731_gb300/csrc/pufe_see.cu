@@ -153,6 +153,12 @@ __global__ void __launch_bounds__(SE_NT) k_see(
   const float4 *qe = qdat + qpoff[e];
   const int32_t *m = smap + soff[e];
   const uint8_t *esh = BLOCH ? eshift + doff[e] : nullptr;
+  bool phased = false;   // some enrichment column is shifted (else every phase is 1)
+  if (BLOCH) {
+    int any = 0;
+    for (int r = tid; r < ne; r += SE_NT) any |= esh[64 + r];
+    phased = __syncthreads_or(any) != 0;
+  }
 
   for (int k = partoff[e]; k < partoff[e + 1]; ++k) {
     const int p = part_p[k], p2 = p * p, p3 = p2 * p, qs = part_q[k];
@@ -263,9 +269,9 @@ __global__ void __launch_bounds__(SE_NT) k_see(
         const int kx = (i & 1) + (j & 1), ky = ((i >> 1) & 1) + ((j >> 1) & 1),
                   kz = (i >> 2) + (j >> 2);
         const ff pv = P[g * 27 + (kz * 3 + ky) * 3 + kx];
-        const double v = (double)pv.hi + (double)pv.lo;
+        const double v = f32_to_f64(pv.hi) + f32_to_f64(pv.lo);
         const int s_rs = m[(64 + r) * n + 64 + s], s_sr = m[(64 + s) * n + 64 + r];
-        if (BLOCH) {   // (r, s) with conj(ph_r) ph_s, (s, r) with its conjugate
+        if (BLOCH && phased) {   // (r, s) with conj(ph_r) ph_s, (s, r) with its conjugate
           const int a = esh[64 + r], b = esh[64 + s];
           const double pr_ = s_phr[a] * s_phr[b] + s_phi[a] * s_phi[b];
           const double pi_ = s_phr[a] * s_phi[b] - s_phi[a] * s_phr[b];
@@ -394,7 +400,7 @@ __global__ void __launch_bounds__(SE_NT) k_see_gram(
       const int r = r0 + ti * TB + a, sc = c0 + tj * TB + b;
       if (r >= ne || sc >= ne || sc > r) continue;
       const ff pv = ff_norm(acc[a][b]);
-      const double v = (double)pv.hi + (double)pv.lo;
+      const double v = f32_to_f64(pv.hi) + f32_to_f64(pv.lo);
       const int s_rs = m[(64 + r) * n + 64 + sc], s_sr = m[(64 + sc) * n + 64 + r];
       if (BLOCH) {   // (r, s) with conj(ph_r) ph_s, (s, r) with its conjugate
         const int ca = esh[64 + r], cb = esh[64 + sc];

@@ -221,29 +221,29 @@ __device__ __forceinline__ void strip_part(const StripElem &E, double *__restric
       float pr, pi;
       pair_phase(E, E.esh[i], E.esh[64 + r], pr, pi);
       if (E.wantH) {
-        atomicAdd(H + s_ir, (double)(hs * pr));
-        atomicAdd(H + s_ri, (double)(hs * pr));
+        atomicAdd(H + s_ir, f32_to_f64(hs * pr));
+        atomicAdd(H + s_ri, f32_to_f64(hs * pr));
         if (pi != 0.0f || !isfinite(hs)) {   // (a zero is not added: no phase inside the cell)
-          atomicAdd(E.Hi + s_ir, (double)(hs * pi));
-          atomicAdd(E.Hi + s_ri, (double)(-hs * pi));
+          atomicAdd(E.Hi + s_ir, f32_to_f64(hs * pi));
+          atomicAdd(E.Hi + s_ri, f32_to_f64(-hs * pi));
         }
       }
       if (E.wantS) {
-        atomicAdd(S + s_ir, (double)(ss * pr));
-        atomicAdd(S + s_ri, (double)(ss * pr));
+        atomicAdd(S + s_ir, f32_to_f64(ss * pr));
+        atomicAdd(S + s_ri, f32_to_f64(ss * pr));
         if (pi != 0.0f) {
-          atomicAdd(E.Si + s_ir, (double)(ss * pi));
-          atomicAdd(E.Si + s_ri, (double)(-ss * pi));
+          atomicAdd(E.Si + s_ir, f32_to_f64(ss * pi));
+          atomicAdd(E.Si + s_ri, f32_to_f64(-ss * pi));
         }
       }
     } else {
       if (E.wantH) {
-        atomicAdd(H + s_ir, (double)hs);
-        atomicAdd(H + s_ri, (double)hs);
+        atomicAdd(H + s_ir, f32_to_f64(hs));
+        atomicAdd(H + s_ri, f32_to_f64(hs));
       }
       if (E.wantS) {
-        atomicAdd(S + s_ir, (double)ss);
-        atomicAdd(S + s_ri, (double)ss);
+        atomicAdd(S + s_ir, f32_to_f64(ss));
+        atomicAdd(S + s_ri, f32_to_f64(ss));
       }
     }
   };
@@ -923,10 +923,10 @@ __global__ void __maxnreg__(ST_MAXREG) k_strip_sf(
         if (BLOCH) {
           float pr, pi;
           pair_phase(E, E.esh[64 + i], E.esh[64 + j], pr, pi);
-          atomicAdd(H + slot, (double)(hv * pr));
-          if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, (double)(hv * pi));
+          atomicAdd(H + slot, f32_to_f64(hv * pr));
+          if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, f32_to_f64(hv * pi));
         } else {
-          atomicAdd(H + slot, (double)hv);
+          atomicAdd(H + slot, f32_to_f64(hv));
         }
       };
       add(r, sc);
@@ -942,10 +942,10 @@ __global__ void __maxnreg__(ST_MAXREG) k_strip_sf(
       float pr, pi;
       pair_phase(E, E.esh[64 + r], E.esh[64 + sc], pr, pi);
       const float hv = E.HE[lo * ne8 + hi];
-      atomicAdd(H + slot, (double)(hv * pr));
-      if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, (double)(hv * pi));
+      atomicAdd(H + slot, f32_to_f64(hv * pr));
+      if (pi != 0.0f || !isfinite(hv)) atomicAdd(E.Hi + slot, f32_to_f64(hv * pi));
     } else {
-      atomicAdd(H + slot, (double)E.HE[lo * ne8 + hi]);
+      atomicAdd(H + slot, f32_to_f64(E.HE[lo * ne8 + hi]));
     }
   }
 }
@@ -1507,7 +1507,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
       const int lq = tid + AJ_NT * k;
       if (lq >= p3) break;
       const int64_t q = q0 + qs + lq;
-      Vbar[q] += w[q] * (double)acc[k];
+      Vbar[q] += w[q] * f32_to_f64(acc[k]);
     }
   }
 }
