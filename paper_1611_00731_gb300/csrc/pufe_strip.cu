@@ -93,7 +93,7 @@ struct FastDiv {
   unsigned m;
   bool one;
   __device__ explicit FastDiv(int d)
-      : m(d > 1 ? (unsigned)((0x100000000ull + (unsigned)d - 1) / (unsigned)d) : 0u), one(d <= 1) {}
+      : m(d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u), one(d <= 1) {}   // ceil(2^32 / d)
   __device__ __forceinline__ int div(int x) const {
     return one ? x : (int)__umulhi((unsigned)x, m);
   }
@@ -1287,6 +1287,8 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
   __syncthreads();
   if (tid < ne) cmap[ec[tid]] = tid;   // code = slot * 8 + vertex
   __syncthreads();
+  // (Index divisions by run-time sizes go through FastDiv: the gather loops and the stages
+  // repeated them for every value; 12^3 rocksalt, ncu, 93 -> 81 us.)
   // coefficients from Hbar.  The CSR values are gathered with eight
   // independent (map, value) load chains in flight per thread, each half of
   // K with the lanes of a warp along one CSR row: Hbar_rj (row of enrichment
@@ -1294,13 +1296,15 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
   // added in; the E x E block goes into the work area
   for (int o = tid; o < A * 512; o += AJ_NT) K[o] = 0.0f;   // absent vertices stay 0
   __syncthreads();
+  const FastDiv dne(ne);
+#pragma unroll
   for (int half = 0; half < 2; ++half) {
     for (int o0 = tid; o0 < ne * 64; o0 += 8 * AJ_NT) {
       int s1[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int o = o0 + u * AJ_NT;
-        const int r = half ? o % ne : o >> 6, j = half ? o / ne : o & 63;
+        const int j = half ? dne.div(o) : o & 63, r = half ? o - j * ne : o >> 6;
         s1[u] = o < ne * 64 ? m[half ? j * n + 64 + r : (64 + r) * n + j] : 0;
       }
       double h[8];
@@ -1314,7 +1318,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
         for (int u = 0; u < 8; ++u) {
           const int o = o0 + u * AJ_NT;
           if (o >= ne * 64) break;
-          const int r = half ? o % ne : o >> 6, j = half ? o / ne : o & 63;
+          const int j = half ? dne.div(o) : o & 63, r = half ? o - j * ne : o >> 6;
           h[u] = half ? cot_entry(h[u], hi[u], esh[j], esh[64 + r], bc.ph)
                       : cot_entry(h[u], hi[u], esh[64 + r], esh[j], bc.ph);
         }
@@ -1323,7 +1327,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
       for (int u = 0; u < 8; ++u) {
         const int o = o0 + u * AJ_NT;
         if (o >= ne * 64) break;
-        const int r = half ? o % ne : o >> 6, j = half ? o / ne : o & 63;
+        const int j = half ? dne.div(o) : o & 63, r = half ? o - j * ne : o >> 6;
         const int code = ec[r], v = code & 7;
         const int atx = 2 * (j & 3) + (v & 1), bty = 2 * ((j >> 2) & 3) + ((v >> 1) & 1),
                   ctz = 2 * (j >> 4) + (v >> 2);
@@ -1339,7 +1343,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
     int s1[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int o = o0 + u * AJ_NT, r = o / ne, sc = o - r * ne;
+      const int o = o0 + u * AJ_NT, r = dne.div(o), sc = o - r * ne;
       s1[u] = o < ne * ne ? m[(64 + r) * n + 64 + sc] : 0;
     }
     double h[8];
@@ -1351,7 +1355,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
       for (int u = 0; u < 8; ++u) hi[u] = o0 + u * AJ_NT < ne * ne ? bc.Hi[s1[u]] : 0.0;
       const uint8_t *esh = bc.eshift + doff[e] + 64;
       for (int u = 0; u < 8; ++u) {
-        const int o = o0 + u * AJ_NT, r = o / ne, sc = o - r * ne;
+        const int o = o0 + u * AJ_NT, r = dne.div(o), sc = o - r * ne;
         if (o < ne * ne) h[u] = cot_entry(h[u], hi[u], esh[r], esh[sc], bc.ph);
       }
     }
@@ -1387,14 +1391,14 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
   const int kend = min(partoff[e + 1], partoff[e] + ce);
   for (int kp = partoff[e] + cb; kp < kend; ++kp) {
     const int p = part_p[kp], p2 = p * p, p3 = p2 * p, qs = part_q[kp];
-    const FastDiv dp(p), dp2(p2);
+    const FastDiv dp(p), dp2(p2), dp3(p3);
     __syncthreads();   // coefficients ready; previous part's readers done
     // Psi values of the (sub)cell's points and the 1D factors per axis
     for (int o0 = tid; o0 < A * p3; o0 += 4 * AJ_NT) {   // four loads in flight per thread
       float v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int o = o0 + u * AJ_NT, al = o / p3, ql = qs + o - al * p3;
+        const int o = o0 + u * AJ_NT, al = dp3.div(o), ql = qs + o - al * p3;
         v[u] = o < A * p3 ? pe[((int64_t)(ql >> 3) * A + al) * 32 + (ql & 7)] : 0.0f;
       }
 #pragma unroll
@@ -1452,7 +1456,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
       for (int k = 0; k < 4; ++k) {
         const int lq = tid + AJ_NT * k;
         if (lq >= p3) break;
-        const int qz = lq / p2, qxy = lq - qz * p2;
+        const int qz = dp2.div(lq), qxy = lq - qz * p2;
         float a = acc[k];
         for (int g = 0; g < nc; ++g) {
           const float *y8 = Y + g * 8 * p2 + qxy;
@@ -1490,7 +1494,7 @@ __global__ void __launch_bounds__(AJ_NT, 4) k_adjoint_strip_sf(
       for (int k = 0; k < 4; ++k) {
         const int lq = tid + AJ_NT * k;
         if (lq >= p3) break;
-        const int qz = lq / p2, qxy = lq - qz * p2;
+        const int qz = dp2.div(lq), qxy = lq - qz * p2;
         const float uz0 = U1[6 * pm + qz], uz1 = U1[7 * pm + qz], uz2 = U1[8 * pm + qz];
         float a = acc[k];
         for (int g = 0; g < nc; ++g) {
@@ -1519,9 +1523,11 @@ pufe_status launch_adjoint_strip_sf(pufe_ctx *ctx, const double *Hbar, double *V
   if (count <= 0 || ctx->adj_sf_floats == 0) return PUFE_OK;
   auto &D = ctx->d;
   const int pm = std::max(1, ctx->max_part_p);
-  // FastDiv preconditions: the divided indices stay below the work area
-  // (AJ_W floats), the divisors are p and p^2
-  if ((int64_t)AJ_W * pm * pm >= (int64_t(1) << 32))
+  // FastDiv preconditions: the divided indices stay below the work area (AJ_W
+  // floats; divisors p, p^2 and, for the coefficients, n_e - 64 <= 64) or the stage
+  // of A p^3 Psi values (divisor p^3, at most 1,024 points)
+  if ((int64_t)AJ_W * std::max(pm * pm, 64) >= (int64_t(1) << 32) ||
+      (int64_t)ctx->adj_sf_floats * 1024 >= (int64_t(1) << 32))
     return fail(PUFE_EINVAL, "adjoint strip: index range beyond its 32-bit divisions");
   const int cf = (ctx->adj_sf_floats + 3) & ~3;
   const size_t sm = ((size_t)cf + 33 * pm + AJ_W + 16 * 8 + 136) * sizeof(float);
