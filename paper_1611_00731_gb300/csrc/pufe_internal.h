@@ -112,7 +112,7 @@ struct DeviceArrays {
   // the same by function: node and value lists, rser_len per function
   int32_t *rser_i = nullptr;
   double *rser_v = nullptr;
-  // FP64 tabulation: (element, first slot, slots of one atom, first point) items
+  // tabulation: (element, first slot, slots of one atom, first point) items
   int32_t *kitems = nullptr;
   // mixed-path work list of the n_e > 128 elements, 3 per item (index into
   // `order`, first chunk, end chunk; chunks of 8 padded points), largest first
@@ -164,7 +164,7 @@ struct pufe_ctx {
   int asm64_work = 0;         // doubles of its shared work area
   int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
   int rser_len = 0;           // entries per serendipity function in rser_i, rser_v
-  int n_kitems = 0;           // items of the FP64 tabulation
+  int n_kitems = 0;           // items of the tabulation
   int n_dunits = 0;           // units of the FP64 density (0: direct form)
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
@@ -173,6 +173,7 @@ struct pufe_ctx {
   bool citems_cut = false;    // some element of that list is cut into several ranges
   int n_pitems = 0;           // items of the FP32 per-point list (point ranges of every element)
   int n_tblk = 0;             // CTAs of the FP32 tabulation (TAB_CHUNK table items each)
+  int max_l = 0;              // largest l of the cell's orbitals
   int max_part_p = 0;         // largest points-per-axis of any (sub)cell
   int strip_stage = 0;        // floats of the strip kernel's shared-memory stage
   uint32_t strip_pmask = 0;   // per-axis counts (bit p) of the strip kernel's cells
@@ -206,7 +207,7 @@ namespace pufe {
 __host__ __device__ inline bool adjoint_sf_fits(int A, int pmax) { return A <= 16 && pmax <= 10; }
 // (slot, padded point) items of the FP32 enrichment table per tabulation CTA
 constexpr int TAB_CHUNK = 2048;
-// points of one FP64 tabulation item
+// points of one tabulation item
 constexpr int TAB64_CHUNK = 128;
 // Shared-memory stage of the E-E overlap kernel (floats): elements whose
 // slots' Psi values on one (sub)cell exceed it take the Gram form instead

@@ -1582,6 +1582,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
     tblk[e + 1] = tblk[e] + (int32_t)((items + TAB_CHUNK - 1) / TAB_CHUNK);
   }
   ctx->n_tblk = tblk[nelem];
+  for (const Orbital &o : S.orb) ctx->max_l = std::max(ctx->max_l, o.l);
 
   // work lists of the sum-factorized FP64 assembly, adjoint and density
   ctx->n_e = n_e;
@@ -1598,7 +1599,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
     sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
     pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits);
   }
-  // FP64 tabulation: runs of slots with one atom and cutoff, in chunks of points
+  // tabulation: runs of slots with one atom and cutoff, in chunks of points
   std::vector<int32_t> kitems;
   for (int64_t e = 0; e < nelem; ++e) {
     const std::vector<int> &al = ealpha[e];

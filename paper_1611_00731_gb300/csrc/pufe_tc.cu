@@ -333,6 +333,105 @@ __global__ void __launch_bounds__(TAB_NT, 6) k_tabulate_f32(
 }
 
 // ---------------------------------------------------------------------------
+// The same table for cells whose orbitals all have l <= 1.
+//
+// One CTA per item of the FP64 tabulation's list, a run of slots of one element that
+// share an atom and 128 of its points (the last chunk also fills the padding); one
+// thread per point.  What bounded the form of one (slot, point) per thread was the
+// arithmetic that the orbitals of an atom repeat: the displacement, its length, the
+// images within r_c, the cutoff and its slope are formed once per point, the
+// exponential and the radial function once per (n, l, zeta).  64 registers, eight CTAs
+// per SM; ncu: 12^3 rocksalt 36 -> 17.5 us, 64-atom cell (65,000
+// items) 0.23 ms.  Orbitals of l >= 2 stay with the form above: there the compiler
+// forms the products of the harmonics outside the loop over the slots and rounds them
+// apart from their sums, which moves H by 3e-9 of its norm, for 26 us of the CsCl-like
+// cell's 1.4 ms step.
+constexpr int TABSP_NT = TAB64_CHUNK;
+
+__global__ void __launch_bounds__(TABSP_NT, 8) k_tabulate_sp_f32(
+    const int4 *__restrict__ items, const int64_t *__restrict__ qpoff,
+    const float4 *__restrict__ qdat, const int32_t *__restrict__ aoff,
+    const int32_t *__restrict__ alist, const int64_t *__restrict__ toff32,
+    const OrbitalF *__restrict__ orbf, const float *__restrict__ eorig, float ax, float ay,
+    float az, float hx, float hy, float hz, float *__restrict__ psi) {
+  const int4 it = items[blockIdx.x];   // element, first slot, slots, first point
+  const int e = it.x, q = it.w + threadIdx.x;
+  const int64_t q0 = qpoff[e];
+  if (q >= (int)(qpoff[e + 1] - q0)) return;
+  const int a0 = aoff[e] + it.y, A = aoff[e + 1] - aoff[e];
+  const float av[3] = {ax, ay, az}, hh[3] = {0.5f * hx, 0.5f * hy, 0.5f * hz};
+  const int32_t *al = alist + a0;
+  const float *eo = eorig + 8 * (int64_t)a0;
+  float *out = psi + 4 * toff32[e] + ((int64_t)(q >> 3) * A + it.y) * 32 + (q & 7);
+  const OrbitalF &o0 = orbf[al[0]];   // the atom and the cutoff of the run
+  const float rc = o0.rc, irc = o0.inv_rc;
+  const float4 xq = qdat[q0 + q];
+  const float xi[3] = {xq.x, xq.y, xq.z};
+  float d[3];
+  int lo[3], hi[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    d[k] = (eo[k] + (xi[k] + 1.0f) * hh[k]) + eo[3 + k];
+    const float rcw = rc * 1.0001f, ia = 1.0f / av[k];
+    lo[k] = (int)ceilf((-rcw - d[k]) * ia);
+    hi[k] = (int)floorf((rcw - d[k]) * ia);
+  }
+  bool first = true;
+  for (int i = lo[0]; i <= hi[0]; ++i)
+    for (int j = lo[1]; j <= hi[1]; ++j)
+      for (int k = lo[2]; k <= hi[2]; ++k) {
+        const float v[3] = {d[0] + i * av[0], d[1] + j * av[1], d[2] + k * av[2]};
+        const float r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        if (r2 >= rc * rc) continue;
+        const float r = sqrtf(r2), t = r * irc, t3 = t * t * t, om = 1.0f - t;
+        const float hc = 1.0f + t3 * t * (-35.0f + t * (84.0f + t * (-70.0f + 20.0f * t)));
+        const float dh = -140.0f * t3 * om * om * om * irc;
+        float zeta = -1.0f, ex = 0.0f, f = 0.0f, df = 0.0f;
+        int pn = -1, pl = -1;
+        for (int c = 0; c < it.z; ++c) {
+          const OrbitalF o = orbf[al[c]];
+          if (o.zeta != zeta || o.n != pn || o.l != pl) {   // the radial function of (n, l, zeta)
+            if (o.zeta != zeta) ex = expf(-o.zeta * r);
+            zeta = o.zeta;
+            pn = o.n;
+            pl = o.l;
+            const int kk = pn - 1 - pl;
+            float rk = 1.0f, rkm = 0.0f;
+            for (int u = 0; u < kk; ++u) {
+              rkm = rk;
+              rk *= r;
+            }
+            const float ez = o.norm * ex;
+            f = ez * rk * hc;
+            df = ez * ((float)kk * rkm * hc - zeta * rk * hc + rk * dh);
+          }
+          float gs[3];
+          const float S = solid_harmonic<float>(o.l, o.m, v[0], v[1], v[2], gs);
+          const float sr = (r > 1e-14f) ? df * S / r : 0.0f;
+          float *dst = out + 32 * c;
+          float w0 = 0.0f, w1 = 0.0f, w2 = 0.0f, w3 = 0.0f;
+          if (!first) {   // a second image within r_c adds to the first's
+            w0 = dst[0];
+            w1 = dst[8];
+            w2 = dst[16];
+            w3 = dst[24];
+          }
+          w0 += f * S;
+          w1 += sr * v[0] + f * gs[0];
+          w2 += sr * v[1] + f * gs[1];
+          w3 += sr * v[2] + f * gs[2];
+          dst[0] = w0;
+          dst[8] = w1;
+          dst[16] = w2;
+          dst[24] = w3;
+        }
+        first = false;
+      }
+  if (first)
+    for (int c = 0; c < 4 * it.z; ++c) out[8 * c] = 0.0f;
+}
+
+// ---------------------------------------------------------------------------
 // Tensor-core element contraction for elements with n_e > 128 (up to 256
 // basis functions): persistent, warp-specialized.
 //
@@ -1337,11 +1436,19 @@ __global__ void __launch_bounds__(AS_NT) k_adjoint_strip_f32(
 pufe_status launch_tabulate_f32(pufe_ctx *ctx, cudaStream_t st) {
   if (ctx->psi32_len == 0) return PUFE_OK;
   auto &D = ctx->d;
-  if (ctx->n_tblk <= 0) return PUFE_OK;
-  k_tabulate_f32<<<(unsigned)ctx->n_tblk, TAB_NT, 0, st>>>(
-      D.qpoff, D.qdat, D.aoff, D.alist, D.toff32, D.orbf, D.eorig, (float)ctx->a[0],
-      (float)ctx->a[1], (float)ctx->a[2], (float)ctx->h[0], (float)ctx->h[1], (float)ctx->h[2],
-      D.tblk, (int)ctx->nelem, D.psi32);
+  if (ctx->max_l <= 1) {
+    if (ctx->n_kitems <= 0) return PUFE_OK;
+    k_tabulate_sp_f32<<<(unsigned)ctx->n_kitems, TABSP_NT, 0, st>>>(
+        reinterpret_cast<const int4 *>(D.kitems), D.qpoff, D.qdat, D.aoff, D.alist, D.toff32,
+        D.orbf, D.eorig, (float)ctx->a[0], (float)ctx->a[1], (float)ctx->a[2], (float)ctx->h[0],
+        (float)ctx->h[1], (float)ctx->h[2], D.psi32);
+  } else {
+    if (ctx->n_tblk <= 0) return PUFE_OK;
+    k_tabulate_f32<<<(unsigned)ctx->n_tblk, TAB_NT, 0, st>>>(
+        D.qpoff, D.qdat, D.aoff, D.alist, D.toff32, D.orbf, D.eorig, (float)ctx->a[0],
+        (float)ctx->a[1], (float)ctx->a[2], (float)ctx->h[0], (float)ctx->h[1], (float)ctx->h[2],
+        D.tblk, (int)ctx->nelem, D.psi32);
+  }
   PUFE_CUDA_TRY(cudaGetLastError());
   return PUFE_OK;
 }
