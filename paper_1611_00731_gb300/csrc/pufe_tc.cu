@@ -862,7 +862,7 @@ constexpr int DEN_NT = 128;
 // KC states k0 .. k0 + KC - 1 of one point added into r: sum_k f_k (sum_j b_j C_jk)^2 over
 // the 64 tricubic columns (from the 1D factors L) and the enrichment columns
 // (PU factor times the point's Psi value of the column's slot)
-template <int KC>
+template <int KC, bool SLOTS>
 __device__ __forceinline__ float density_states(const float (&L)[3][4], const float (&pu)[8],
                                                 const float *pq, const int32_t *ec, int nenr,
                                                 const float *Cb, const float *fs, int noccp,
@@ -883,20 +883,46 @@ __device__ __forceinline__ float density_states(const float (&L)[3][4], const fl
         for (int k = 0; k < KC; ++k) acc[k] = fmaf(b, cr[k], acc[k]);
       }
     }
-  for (int j = 0; j < nenr; ++j) {
-    const int code = ec[j];
-    const float b = pu[code & 7] * pq[(code >> 3) * 32];
+  auto column = [&](int j, float b) {
     const float *cr = Cb + (64 + j) * noccp + k0;
 #pragma unroll
     for (int k = 0; k < KC; ++k) acc[k] = fmaf(b, cr[k], acc[k]);
+  };
+  if (!SLOTS) {
+    for (int j = 0; j < nenr; ++j) {
+      const int code = ec[j];
+      column(j, pu[code & 7] * pq[(code >> 3) * 32]);
+    }
+  }
+  for (int j = SLOTS ? 0 : nenr; j < nenr;) {
+    const int code = ec[j];
+    const float ps = pq[(code >> 3) * 32];
+    // a slot with its eight vertices in order (the elements whose vertices do not wrap
+    // around the cell): its Psi is read once and the PU factors need no selection
+    bool full = (code & 7) == 0 && j + 8 <= nenr;
+#pragma unroll
+    for (int v = 1; v < 8; ++v) full = full && ec[j + v] == code + v;
+    if (full) {
+#pragma unroll
+      for (int v = 0; v < 8; ++v) column(j + v, pu[v] * ps);
+      j += 8;
+    } else {
+      column(j, pu[code & 7] * ps);
+      ++j;
+    }
   }
 #pragma unroll
   for (int k = 0; k < KC; ++k) r = fmaf(fs[k0 + k] * acc[k], acc[k], r);
   return r;
 }
 
-template <bool BLOCH>
-__global__ void __launch_bounds__(DEN_NT) k_density_f32(
+// NARROW: at most 8 real states, one pass without the loop over states (whose basis
+// values the compiler would keep in 128 registers), twice the CTAs per SM, the
+// coefficients gathered four at a time and enrichments taken a slot at a time: 12^3
+// rocksalt, 8 states (ncu) 54 -> 47 us.  The same gather and slots with 16 states per
+// pass measured slower (CsCl-like cell, 35 states: 254 -> 333 us) and are not taken there.
+template <bool BLOCH, bool NARROW>
+__global__ void __launch_bounds__(DEN_NT, NARROW ? 8 : 4) k_density_f32(
     const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
     const int64_t *__restrict__ qpoff, const float4 *__restrict__ qdat,
     const int64_t *__restrict__ doff, const int32_t *__restrict__ dofs,
@@ -921,7 +947,20 @@ __global__ void __launch_bounds__(DEN_NT) k_density_f32(
   float *Cs = fsm;              // n x noccp
   float *fs = Cs + n * noccp;   // noccp
   float *Cz = fs + noccp;       // n x noccp: imaginary parts (Bloch states, Ci != nullptr)
-  for (int k = threadIdx.x; k < n * noccp; k += DEN_NT) {
+  if (NARROW) {   // four (column, value) load chains in flight per thread
+    for (int o0 = threadIdx.x; o0 < n * 8; o0 += 4 * DEN_NT) {
+      double c[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int o = min(o0 + u * DEN_NT, n * 8 - 1), kk = o & 7;
+        c[u] = kk < nocc ? C[(int64_t)dl[o >> 3] * ldc + kk] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (o0 + u * DEN_NT < n * 8) Cs[o0 + u * DEN_NT] = f64_to_f32(c[u]);
+    }
+  }
+  for (int k = threadIdx.x; !NARROW && k < n * noccp; k += DEN_NT) {
     const int j = k / noccp, kk = k - j * noccp;
     if (BLOCH) {   // (C + i Ci) exp(i k.R_j) in FP64, then rounded
       double cr = 0.0, ci = 0.0;
@@ -958,12 +997,18 @@ __global__ void __launch_bounds__(DEN_NT) k_density_f32(
     // real parts (the only ones at Gamma), then the imaginary parts; at Gamma
     // states 16 at a time while 16 remain, then 8 (each state's sums in the
     // same order either way; the Bloch form measured faster with 8 only)
-    for (int part = 0; part < (BLOCH ? 2 : 1); ++part) {
-      const float *Cb = part ? Cz : Cs;
-      int k0 = 0;
-      for (; !BLOCH && k0 + 16 <= noccp; k0 += 16)
-        r = density_states<16>(L, pu, pq, ec, nenr, Cb, fs, noccp, k0, r);
-      for (; k0 < noccp; k0 += 8) r = density_states<8>(L, pu, pq, ec, nenr, Cb, fs, noccp, k0, r);
+    if (NARROW) {   // (the coefficients are read per point, not kept across the points)
+      asm volatile("" ::: "memory");
+      r = density_states<8, true>(L, pu, pq, ec, nenr, Cs, fs, 8, 0, r);
+    } else {
+      for (int part = 0; part < (BLOCH ? 2 : 1); ++part) {
+        const float *Cb = part ? Cz : Cs;
+        int k0 = 0;
+        for (; !BLOCH && k0 + 16 <= noccp; k0 += 16)
+          r = density_states<16, false>(L, pu, pq, ec, nenr, Cb, fs, noccp, k0, r);
+        for (; k0 < noccp; k0 += 8)
+          r = density_states<8, false>(L, pu, pq, ec, nenr, Cb, fs, noccp, k0, r);
+      }
     }
     rho[q0 + q] = (double)r;
   }
@@ -1013,36 +1058,40 @@ __global__ void __launch_bounds__(256, 2) k_density_tile_f32(
   float *fs = Ls + 20 * DT_PT;          // [ncol]
   float *Bs = fs + ncol;                // [DT_J][DT_PT]; then [ncol / 2][DT_PT]
   for (int k = tid; k < ncol; k += NT) fs[k] = (k % noccp < nocc) ? (float)f[k % noccp] : 0.0f;
-  {   // coefficients, a warp along the states of four columns at a time; columns of a
-      // zero lattice shift carry no phase
-    const int lane = tid & 31, nw = NT >> 5;
-    for (int j0 = tid >> 5; j0 < n; j0 += 4 * nw) {
-      int64_t g[4];
-      int cd[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = min(j0 + u * nw, n - 1);
-        g[u] = (int64_t)dl[j] * ldc;
-        cd[u] = BLOCH ? es[j] : 0;
-      }
-      for (int k = lane; k < noccp; k += 32) {
-        double ar[4], ai[4];
+  {   // coefficients, a warp along 64 states of four columns at a time; columns
+      // of a zero lattice shift carry no phase
+    const int lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
+    for (int r0 = 0; warp + r0 * nw < n; r0 += 32) {   // this warp's columns, 32 at a time
+      const int jl = warp + (r0 + lane) * nw;
+      const int dj = jl < n ? dl[jl] : 0, cj = BLOCH && jl < n ? es[jl] : 0;
+      for (int r = 0; r < 32 && warp + (r0 + r) * nw < n; r += 4) {
+        int64_t g[4];
+        int cds[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          ar[u] = k < nocc ? C[g[u] + k] : 0.0;
-          ai[u] = BLOCH && k < nocc ? Ci[g[u] + k] : 0.0;
+          g[u] = (int64_t)__shfl_sync(0xffffffffu, dj, r + u) * ldc;
+          cds[u] = __shfl_sync(0xffffffffu, cj, r + u);
         }
+        for (int k0 = lane; k0 < noccp; k0 += 64) {   // 4 columns x 2 runs of states in flight
+          double ar[8], ai[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = j0 + u * nw;
-          if (j >= n) break;
-          double cr = ar[u], ci = ai[u];
-          if (BLOCH && (cd[u] != 0 || !isfinite(cr) || !isfinite(ci))) {
-            cr = ph.re[cd[u]] * ar[u] - ph.im[cd[u]] * ai[u];
-            ci = ph.re[cd[u]] * ai[u] + ph.im[cd[u]] * ar[u];
+          for (int u = 0; u < 8; ++u) {
+            const int k = k0 + 32 * (u & 1);
+            ar[u] = k < nocc ? C[g[u >> 1] + k] : 0.0;
+            ai[u] = BLOCH && k < nocc ? Ci[g[u >> 1] + k] : 0.0;
           }
-          Cs[j * ncol + k] = f64_to_f32(cr);
-          if (BLOCH) Cs[j * ncol + noccp + k] = f64_to_f32(ci);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int j = warp + (r0 + r + (u >> 1)) * nw, k = k0 + 32 * (u & 1), cd = cds[u >> 1];
+            if (j >= n || k >= noccp) continue;
+            double cr = ar[u], ci = ai[u];
+            if (BLOCH && (cd != 0 || !isfinite(cr) || !isfinite(ci))) {
+              cr = ph.re[cd] * ar[u] - ph.im[cd] * ai[u];
+              ci = ph.re[cd] * ai[u] + ph.im[cd] * ar[u];
+            }
+            Cs[j * ncol + k] = f64_to_f32(cr);
+            if (BLOCH) Cs[j * ncol + noccp + k] = f64_to_f32(ci);
+          }
         }
       }
     }
@@ -1595,7 +1644,8 @@ pufe_status launch_density_tc(pufe_ctx *ctx, const double *C, int64_t ldc, const
     PUFE_CUDA_TRY(cudaGetLastError());
     return PUFE_OK;
   }
-  auto kern = Ci ? k_density_f32<true> : k_density_f32<false>;
+  auto kern = Ci ? k_density_f32<true, false>
+                 : (noccp == 8 ? k_density_f32<false, true> : k_density_f32<false, false>);
   PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   if (ctx->n_pitems <= 0) return PUFE_OK;
   kern<<<(unsigned)ctx->n_pitems, DEN_NT, sm, st>>>(
