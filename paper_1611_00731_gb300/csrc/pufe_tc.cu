@@ -1203,12 +1203,15 @@ __global__ void __launch_bounds__(256, 2) k_density_tile_f32(
 // The element block is gathered with eight (map, value) load chains in flight per
 // thread -- one after the other they took most of the kernel on a 184-function
 // element -- and the 1D factors of a chunk's points are formed once per point.
-// QB points per chunk: 64 (46 x 16 register tiles of such an element fill three
-// passes of 256 threads) where the block leaves room in shared memory, else 32.
-constexpr int ADJ_NT = 256;
+// QB points per chunk: 64 (46 x 16 register tiles of such an element fill two
+// passes of 384 threads) where the block leaves room in shared memory, else 32.
+// A thread's four points lie QB / 4 apart, so that the lanes of a 16-byte read take
+// neighbouring rows of Bq, whose pitch puts them on different banks; the basis values
+// are formed with the lanes along the points, which the Psi table stores together.
+constexpr int ADJ_NT = 384;
 
 template <bool BLOCH, int ADJ_QB>
-__global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
+__global__ void __launch_bounds__(ADJ_NT, 1) k_adjoint_f32(
     const int32_t *__restrict__ order, const int64_t *__restrict__ qoff,
     const int64_t *__restrict__ qpoff, const float4 *__restrict__ qdat,
     const double *__restrict__ w, const int64_t *__restrict__ doff,
@@ -1254,9 +1257,9 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
     for (int u = 0; u < 8; ++u) {
       const int k = k0 + u * ADJ_NT, i = k / n, j = k - i * n;
       if (k >= n * n) break;
-      Hs[i * n4 + j] = BLOCH ? (float)cot_entry(h[u], hi[u], bc.eshift[doff[e] + i],
-                                                bc.eshift[doff[e] + j], bc.ph)
-                             : (float)h[u];
+      Hs[i * n4 + j] = f64_to_f32(BLOCH ? cot_entry(h[u], hi[u], bc.eshift[doff[e] + i],
+                                                    bc.eshift[doff[e] + j], bc.ph)
+                                        : h[u]);
     }
   }
   const int nI = n4 / 4;
@@ -1273,8 +1276,9 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
       for (int a = 0; a < 4; ++a) Lq[(4 * d + a) * ADJ_QB + qq] = L[a];
     }
     __syncthreads();
+#pragma unroll 4
     for (int k = threadIdx.x; k < ADJ_QB * n4; k += ADJ_NT) {
-      const int qq = k / n4, c = k - qq * n4;
+      const int c = k / ADJ_QB, qq = k - c * ADJ_QB;
       const int q = qc + qq;
       float b = 0.0f;
       if (q < qend && c < n) {
@@ -1296,7 +1300,8 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
     __syncthreads();
     for (int t = threadIdx.x; t < ntile; t += ADJ_NT) {
       const int tq = t & (ADJ_QB / 4 - 1), ti = t / (ADJ_QB / 4);
-      const float *b0 = Bq + (4 * tq) * ldb;
+      const float *b0 = Bq + tq * ldb;
+      const int xs = (ADJ_QB / 4) * ldb;   // to the thread's next point
       const float *h0 = Hs + (4 * ti) * n4;
       float a[4][4];
 #pragma unroll
@@ -1306,7 +1311,7 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
       for (int j = 0; j < n4; j += 4) {
         float4 bv[4], hv[4];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) bv[x] = *reinterpret_cast<const float4 *>(b0 + x * ldb + j);
+        for (int x = 0; x < 4; ++x) bv[x] = *reinterpret_cast<const float4 *>(b0 + x * xs + j);
 #pragma unroll
         for (int y = 0; y < 4; ++y) hv[y] = *reinterpret_cast<const float4 *>(h0 + y * n4 + j);
 #pragma unroll
@@ -1319,8 +1324,8 @@ __global__ void __launch_bounds__(ADJ_NT) k_adjoint_f32(
       for (int x = 0; x < 4; ++x) {
         float s = 0.0f;
 #pragma unroll
-        for (int y = 0; y < 4; ++y) s = fmaf(b0[x * ldb + 4 * ti + y], a[x][y], s);
-        part[ti * ADJ_QB + 4 * tq + x] = s;
+        for (int y = 0; y < 4; ++y) s = fmaf(b0[x * xs + 4 * ti + y], a[x][y], s);
+        part[ti * ADJ_QB + tq + (ADJ_QB / 4) * x] = s;
       }
     }
     __syncthreads();
