@@ -1541,9 +1541,31 @@ static pufe_status run_assemble_tc(pufe_ctx *ctx, const double *V, int what, dou
   if (pufe_status e = mark(0, st)) return e;
   if (prof) ctx->prof_ran[0] = true;
   const size_t bytes = (size_t)ctx->nnz * sizeof(double);
+  // Without a tensor-core tile the FE-FE kernel, which only needs H = 0, runs first
+  // on the caller's stream, beside the copy of S on the side stream; the strip
+  // follows when S is there (12^3 rocksalt mixed step 477 -> 472 us against memset, copy
+  // and strip first; 20^3 gradient, which wants H alone, unchanged)
+  const bool early = nbig == 0 && (what & PUFE_WANT_H) && (what & PUFE_WANT_S);
+  auto fefe = [&](cudaStream_t sf) -> pufe_status {
+    if (pufe_status e = mark(2, sf)) return e;
+    if (pufe_status e = launch_fefe(ctx, V, H, sf)) return e;
+    if (prof) ctx->prof_ran[1] = true;
+    return mark(3, sf);
+  };
+  if (early) {
+    PUFE_CUDA_TRY(cudaEventRecord(D.ev_fork, st));
+    PUFE_CUDA_TRY(cudaStreamWaitEvent(D.side, D.ev_fork, 0));
+    PUFE_CUDA_TRY(cudaMemcpyAsync(S, D.S0, bytes, cudaMemcpyDeviceToDevice, D.side));
+    PUFE_CUDA_TRY(cudaEventRecord(D.ev_fork, D.side));
+  }
   if (what & PUFE_WANT_H) PUFE_CUDA_TRY(cudaMemsetAsync(H, 0, bytes, st));
-  if (what & PUFE_WANT_S) PUFE_CUDA_TRY(cudaMemcpyAsync(S, D.S0, bytes, cudaMemcpyDeviceToDevice, st));
-  PUFE_CUDA_TRY(cudaEventRecord(D.ev_fork, st));
+  if (early) {
+    if (pufe_status e = fefe(st)) return e;
+    PUFE_CUDA_TRY(cudaStreamWaitEvent(st, D.ev_fork, 0));
+  } else if (what & PUFE_WANT_S) {
+    PUFE_CUDA_TRY(cudaMemcpyAsync(S, D.S0, bytes, cudaMemcpyDeviceToDevice, st));
+  }
+  if (!early) PUFE_CUDA_TRY(cudaEventRecord(D.ev_fork, st));
   // the strip kernels go first, so that their CTAs take their share of every
   // SM; the side stream's kernels are small enough to run beside them
   if (nbig > 0) {
@@ -1575,15 +1597,9 @@ static pufe_status run_assemble_tc(pufe_ctx *ctx, const double *V, int what, dou
   // side stream before the E-E kernels (measured: 12^3 rocksalt step 0.559 ->
   // 0.543 ms with it on the caller's stream; the CsCl-like cell, whose
   // caller's stream also carries the tensor-core tile, 1.71 -> 1.76 ms)
-  PUFE_CUDA_TRY(cudaStreamWaitEvent(D.side, D.ev_fork, 0));
-  if (what & PUFE_WANT_H) {
-    const cudaStream_t sf = nbig > 0 ? D.side : st;
-    if (pufe_status e = mark(2, sf)) return e;
-    pufe_status e0 = launch_fefe(ctx, V, H, sf);
-    if (e0 != PUFE_OK) return e0;
-    if (pufe_status e = mark(3, sf)) return e;
-    if (prof) ctx->prof_ran[1] = true;
-  }
+  if (!early) PUFE_CUDA_TRY(cudaStreamWaitEvent(D.side, D.ev_fork, 0));
+  if ((what & PUFE_WANT_H) && !early)
+    if (pufe_status e = fefe(nbig > 0 ? D.side : st)) return e;
   if (what & PUFE_WANT_S) {
     if (pufe_status e = mark(4, D.side)) return e;
     pufe_status e0 = launch_see(ctx, nullptr, S, nullptr, D.side);
