@@ -679,9 +679,8 @@ def run_pufe(args):
         "c5": c5,
         "fp64_path": (None if fp64_ms is None else {
             "ms_per_step": fp64_ms, "speedup_of_this_path": fp64_ms / ms_per_step,
-            "note": "same step on the plain FP64 kernels (direct element contraction, the "
-                    "1e-12 reference path); the ratio includes the mixed path's sum "
-                    "factorization as well as its precision. At equal eigenvalue "
+            "note": "same step on the FP64 kernels (sum-factorized too, the 1e-12 "
+                    "reference path). At equal eigenvalue "
                     "accuracy: on this cell the mixed path's 8 lowest eigenvalues are "
                     "within 6.5e-8 Ha of the FP64 oracle (tests/test_gpu_c2_full.py), "
                     "inside the 1e-5 Ha target"}),
