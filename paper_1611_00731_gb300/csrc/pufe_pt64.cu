@@ -41,6 +41,12 @@ namespace {
 
 constexpr int P64_NT = 128;
 constexpr int P64_WORK = 7000;   // shared doubles of an adjoint CTA: 56 KB, four CTAs per SM
+// Direct enrichment blocks of the adjoint.  A triangle goes through shared memory whole,
+// beside 64 points, up to P64_WHOLE doubles (163 columns); larger ones in ranges of
+// rows of P64_ROWS doubles (112 KB, two CTAs per SM), with room for P64_QC_MIN points.
+// Eight elements of one-vertex slots and 4^3 points: 150 columns 217 us whole, 225 us in
+// ranges; 185 columns 331 and 262 us.
+constexpr int P64_WHOLE = 24000, P64_ROWS = 14000, P64_QC_MIN = 16, P64_MAX = 227 * 1024 / 8;
 
 struct Adj64 {
   const int32_t *items;   // six per item: element, kind, range, (sub)cell range
@@ -400,30 +406,31 @@ __device__ void adj_pairs(const Adj64 &P, int e, int k0, int k1, int cb, int ce,
   }
 }
 
-// direct E x E products over the points [qa, qb): the symmetrised block and the
-// columns' values of a chunk of points in shared memory, threads over points and
-// row groups
+// direct E x E products of the block's rows [ra, rb) over the points [qa, qb): those
+// rows of the symmetrised block and the columns' values of a chunk of points in shared
+// memory, threads over points and row groups
 template <bool BLOCH>
-__device__ void adj_direct(const Adj64 &P, int e, int qa, int qb, double *sm) {
+__device__ void adj_direct(const Adj64 &P, int e, int qa, int qb, int ra, int rb, double *sm) {
   const int tid = threadIdx.x;
   const CotElem<BLOCH> H = cot_elem<BLOCH>(P, e);
-  const int nE = H.n - P.nfe, nent = nE * (nE + 1) / 2;
+  const int h0 = ra * (ra + 1) / 2, nent = rb * (rb + 1) / 2 - h0;   // packed rows ra .. rb - 1
   const int64_t q0 = P.qoff[e];
   const int Q = (int)(P.qoff[e + 1] - q0);
   const double *pe = P.psi + 4 * P.toff[e];
   const int32_t *ec = P.ecol + (P.doff[e] - (int64_t)P.nfe * e);
   double *Hs = sm, *B = sm + nent;
-  for (int o = tid; o < nE * nE; o += P64_NT) {
-    const int r = o / nE, c = o - r * nE;
+  for (int o = tid; o < (rb - ra) * rb; o += P64_NT) {
+    const int r = ra + o / rb, c = o % rb;
     if (c > r) continue;
-    Hs[r * (r + 1) / 2 + c] = r == c ? H(P.nfe + r, P.nfe + r) : H(P.nfe + r, P.nfe + c) + H(P.nfe + c, P.nfe + r);
+    Hs[r * (r + 1) / 2 - h0 + c] =
+        r == c ? H(P.nfe + r, P.nfe + r) : H(P.nfe + r, P.nfe + c) + H(P.nfe + c, P.nfe + r);
   }
-  const int QC = max(1, min(min((P.work - nent) / nE, P64_NT), qb - qa)), PG = P64_NT / QC;
+  const int QC = max(1, min(min((P.work - nent) / rb, P64_NT), qb - qa)), PG = P64_NT / QC;
   const int qq = tid % QC, grp = tid / QC;
   for (int qc = qa; qc < qb; qc += QC) {
     const int nq = min(QC, qb - qc);
     __syncthreads();
-    for (int o = tid; o < nE * nq; o += P64_NT) {
+    for (int o = tid; o < rb * nq; o += P64_NT) {
       const int j = o / nq, t = o - j * nq, q = qc + t, code = ec[j];
       const double *x = P.xi + 3 * (q0 + q);
       const double lx = code & 1 ? 1.0 + x[0] : 1.0 - x[0], ly = code & 2 ? 1.0 + x[1] : 1.0 - x[1],
@@ -431,16 +438,15 @@ __device__ void adj_direct(const Adj64 &P, int e, int qa, int qb, double *sm) {
       B[j * QC + t] = 0.125 * lx * (ly * lz) * pe[(int64_t)(code >> 3) * 4 * Q + q];
     }
     __syncthreads();
-    // (one thread steps over all points where QC exceeds the block, host emulation)
-    for (int t = qq; t < nq && grp < PG; t += P64_NT) {
+    if (qq < nq && grp < PG) {
       double s = 0.0;
-      for (int r = grp; r < nE; r += PG) {
-        const double *h = Hs + r * (r + 1) / 2;
+      for (int r = ra + grp; r < rb; r += PG) {
+        const double *h = Hs + r * (r + 1) / 2 - h0;
         double g = 0.0;
-        for (int c = 0; c <= r; ++c) g = fma(h[c], B[c * QC + t], g);
-        s = fma(B[r * QC + t], g, s);
+        for (int c = 0; c <= r; ++c) g = fma(h[c], B[c * QC + qq], g);
+        s = fma(B[r * QC + qq], g, s);
       }
-      atomicAdd(P.out + q0 + qc + t, P.w[q0 + qc + t] * s);
+      atomicAdd(P.out + q0 + qc + qq, P.w[q0 + qc + qq] * s);
     }
   }
 }
@@ -457,7 +463,7 @@ __global__ void __launch_bounds__(P64_NT) k_adjoint_sf64(Adj64 P) {
   else if (kind == 2)
     adj_pairs<BLOCH>(P, e, a, b, cb, ce, sma64);
   else
-    adj_direct<BLOCH>(P, e, a, b, sma64);
+    adj_direct<BLOCH>(P, e, a, b, cb, ce, sma64);
 }
 
 // ---- density ------------------------------------------------------------------
@@ -595,10 +601,14 @@ __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
 
 // Work lists (host).  Adjoint: items (element, kind 0 FE x FE / 1 slot range /
 // 2 pair range / 3 point range of the direct E x E products, begin, end, (sub)cell
-// range) cut to the mean cost of a CTA slot (four per SM), by (sub)cells where
-// their work outweighs the coefficients that every range forms, and to the
-// shared work area, largest first.  Density: int4 units (element, (sub)cell, first z plane, end z plane),
-// cut to the mean cost of a CTA slot.
+// range, or for kind 3 the range of the block's rows) cut to the mean cost of a CTA
+// slot (four per SM), by (sub)cells where their work outweighs the coefficients that
+// every range forms, and to the shared work area, largest first.  The E x E block takes
+// the form of fewer operations, but the pair form, which any work area holds, where
+// one row of the triangle and its columns' points are beyond half an SM's shared
+// memory (over 907 columns; eight such elements of 912 columns 5.5 ms, of 800 in the
+// direct form 1.0 ms).  Density: int4 units (element, (sub)cell, first z plane, end z plane),
+// cut to the mean cost of a CTA slot, and the doubles that one column takes at most.
 void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
                      std::vector<int32_t> &den) {
   adj.clear();
@@ -653,13 +663,24 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
       adj_work = std::max(adj_work, G * (adj_slot_doubles(p) + 4) + 15 * p);
       for (int a = 0; a < A; a += G)
         cells(e, 1, a, std::min(A, a + G), cs[e] * std::min(G, A - a), 8000.0 * G);
-      if (cd[e] < np * cp[e]) {
+      if (cd[e] < np * cp[e] && (nE + 1) * P64_QC_MIN <= P64_MAX / 2) {
         const int Q = ctx->q_e[e];
         const int cuts = std::max(1, std::min(Q / 32, (int)std::min(1e6, std::ceil(cd[e] / target))));
-        adj_work = std::max(adj_work, nE * (nE + 1) / 2 + nE * std::min(64, Q));
-        for (int j = 0; j < cuts; ++j) {
-          const int a = (int)((int64_t)j * Q / cuts), b = (int)((int64_t)(j + 1) * Q / cuts);
-          L.push_back(Item{{(int32_t)e, 3, a, b, 0, 0}, cd[e] * (b - a) / Q});
+        // the whole triangle where it fits beside up to 64 points, else ranges of rows
+        // beside P64_QC_MIN of them
+        const int whole = nE * (nE + 1) / 2 + nE * std::min(64, Q);
+        const int qc = std::min(P64_QC_MIN, Q);
+        const int area = std::max(P64_ROWS, 2 * nE * qc);
+        for (int ra = 0, rb; ra < nE; ra = rb) {
+          rb = whole <= P64_WHOLE ? nE : ra + 1;
+          int ent = rb * (rb + 1) / 2 - ra * (ra + 1) / 2;
+          while (rb < nE && ent + rb + 1 + nE * qc <= area) ent += ++rb;
+          adj_work = std::max(adj_work, whole <= P64_WHOLE ? whole : ent + nE * qc);
+          const double c = cd[e] * ent / (0.5 * nE * (nE + 1));
+          for (int j = 0; j < cuts; ++j) {
+            const int a = (int)((int64_t)j * Q / cuts), b = (int)((int64_t)(j + 1) * Q / cuts);
+            L.push_back(Item{{(int32_t)e, 3, a, b, ra, rb}, c * (b - a) / Q});
+          }
         }
         continue;
       }
