@@ -165,7 +165,8 @@ struct pufe_ctx {
   int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
   int rser_len = 0;           // entries per serendipity function in rser_i, rser_v
   int n_kitems = 0;           // items of the tabulation
-  int n_dunits = 0;           // units of the FP64 density (0: direct form)
+  int n_dunits = 0;           // units of the FP64 density
+  int den64_column = 0;       // shared doubles that one of its columns takes at most
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
   int n_gitems32 = 0, n_gitems64 = 0;   // items of the Gram-form lists
@@ -497,7 +498,7 @@ pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double 
                                 const double *Ci, int64_t ldc, const double *f, int nocc,
                                 double *rho, cudaStream_t s);
 void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
-                     std::vector<int32_t> &den);
+                     std::vector<int32_t> &den, int &den_col);
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,
                                       const double *Ci, int64_t ldc, const double *f, int nocc,
                                       double *rho, cudaStream_t s);

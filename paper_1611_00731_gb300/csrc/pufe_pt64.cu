@@ -486,11 +486,11 @@ struct Den64 {
   double *rho;
 };
 
-__host__ __device__ inline int den_doubles(int n, int p, int kc) {
-  // coefficients of the columns (64 FE functions whatever the space) and, for the
-  // serendipity space, its own; 1D factors; x and y stages; phi_v of each thread
-  return kc * (n + 32 + 16 * p + 4 * p * p) + 12 * p + 8 * P64_NT + kc;
-}
+// doubles of one column: its coefficients (64 FE functions whatever the space) and, for
+// the serendipity space, its own; x and y stages
+int den_column(int n, int p) { return n + 32 + 16 * p + 4 * p * p; }
+// kc columns and their occupations; 1D factors; phi_v of each thread
+int den_doubles(int column, int p, int kc) { return kc * (column + 1) + 12 * p + 8 * P64_NT; }
 
 template <bool BLOCH, int KC>
 __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
@@ -610,10 +610,10 @@ __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
 // direct form 1.0 ms).  Density: int4 units (element, (sub)cell, first z plane, end z plane),
 // cut to the mean cost of a CTA slot, and the doubles that one column takes at most.
 void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
-                     std::vector<int32_t> &den) {
+                     std::vector<int32_t> &den, int &den_col) {
   adj.clear();
   den.clear();
-  adj_work = 0;
+  adj_work = den_col = 0;
   const int64_t ne = (int64_t)ctx->n_e.size();
   struct Item {
     int32_t v[6];
@@ -711,6 +711,7 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
   int32_t cell = 0;
   for (int64_t e = 0; e < ne; ++e)
     for (int p : ctx->part_p_host[e]) {
+      den_col = std::max(den_col, den_column(ctx->n_e[e], p));
       const double fix = 64.0 * p + 16.0 * p * p, pl = plane(e, p);
       const int cuts = std::max(1, std::min(p, (int)std::min(64.0, std::ceil(p * pl / target))));
       for (int j = 0; j < cuts; ++j)
@@ -784,9 +785,16 @@ pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double 
   if (ph) P.ph = *ph;
   P.rho = rho;
   PUFE_CUDA_TRY(cudaMemsetAsync(rho, 0, (size_t)ctx->nq * sizeof(double), st));
-  // columns per CTA: the width (a multiple of 4, up to 16) that pads the fewest
-  const int groups = (P.ncol + 15) / 16, kc = ((P.ncol + groups - 1) / groups + 3) & ~3;
-  const size_t sm = (size_t)den_doubles(ctx->max_basis, ctx->max_part_p, kc) * sizeof(double);
+  // columns per CTA: the width (a multiple of 4, up to 16) that pads the fewest; less
+  // where the work area of the largest (sub)cell does not fit an SM
+  const int most = (P.ncol + 15) / 16;
+  int kc = ((P.ncol + most - 1) / most + 3) & ~3;
+  auto bytes = [&] {
+    return (size_t)den_doubles(ctx->den64_column, ctx->max_part_p, kc) * sizeof(double);
+  };
+  while (kc > 4 && bytes() > 227 * 1024) kc -= 4;
+  const int groups = (P.ncol + kc - 1) / kc;
+  const size_t sm = bytes();
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e too large for the density kernel");
   auto run = [&](auto kern) -> pufe_status {
     PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));

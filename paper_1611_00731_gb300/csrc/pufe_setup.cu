@@ -1597,7 +1597,7 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
         nsm = v;
     }
     sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
-    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits);
+    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits, ctx->den64_column);
   }
   // tabulation: runs of slots with one atom and cutoff, in chunks of points
   std::vector<int32_t> kitems;
