@@ -160,6 +160,7 @@ struct pufe_ctx {
   int n_big = 0;              // elements with n_e > 128 (listed first in `order`)
   int64_t big_pad_end = 0;    // end of the last n_e > 128 element's padded points (0: none)
   int64_t n_wsplit = 0;       // items of the FP64 point-range work list (0: none)
+  int nsm = 152;              // SMs of the device (of a GB300 without one)
   int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
   int asm64_work = 0;         // doubles of its shared work area
   int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
@@ -167,6 +168,7 @@ struct pufe_ctx {
   int n_kitems = 0;           // items of the tabulation
   int n_dunits = 0;           // units of the FP64 density
   int den64_column = 0;       // shared doubles that one of its columns takes at most
+  int den64_points = 0;       // points that one of its units has at most
   int n_titems = 0;           // items of the mixed path's list for the n_e > 128 elements
   int n_sitems = 0;           // items of the E-E overlap kernel's list (slot-pair ranges)
   int n_gitems32 = 0, n_gitems64 = 0;   // items of the Gram-form lists
@@ -498,7 +500,7 @@ pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double 
                                 const double *Ci, int64_t ldc, const double *f, int nocc,
                                 double *rho, cudaStream_t s);
 void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
-                     std::vector<int32_t> &den, int &den_col);
+                     std::vector<int32_t> &den, int &den_col, int &den_pts);
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,
                                       const double *Ci, int64_t ldc, const double *f, int nocc,
                                       double *rho, cudaStream_t s);

@@ -32,6 +32,8 @@
 // Measured, direct kernels before: adjoint 12^3 rocksalt 9.34 -> 0.35 ms, CsCl-like
 // 16^3 19.4 -> 0.60 ms, two-atom 4^3 1.06 -> 0.031 ms; density 0.80 -> 0.23 ms (8
 // states), 17.5 -> 0.99 ms (35 states), 0.21 -> 0.025 ms (2 states).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "pufe_internal.h"
@@ -470,6 +472,21 @@ __global__ void __launch_bounds__(P64_NT) k_adjoint_sf64(Adj64 P) {
 // One CTA per (unit, group of KC real columns): a unit is a (sub)cell of an element
 // and a range of its z planes, a column a state (Gamma) or the real or imaginary
 // part of one (Bloch).
+//
+// The groups of a unit meet in an order that the launch fixes, so that the density
+// repeats bit for bit (one atomic per group does not, from three groups on):
+//  * two halves of the groups on two CTAs, which keep their sum in shared memory and add
+//    it into the zeroed density with one atomic per point (two terms commute);
+//  * from three groups on, on a mesh too small to fill the chip with that (all units and
+//    groups fit four CTAs per SM), a CTA per group: up to five as one cluster, more as two
+//    of them, whose CTAs read one another's sums through distributed shared memory, in
+//    rank order.
+// 64 complex states, against one CTA and atomic per group: eight elements of 6^3 points
+// 38 -> 40 us (halves alone 85 us), 6^3 rocksalt 1,073 -> 1,140 us (clusters 1,169 us),
+// 12^3 rocksalt 3,495 -> 3,447 us; 35 real states on the CsCl-like 16^3 cell 975 -> 967
+// us (clusters 1,045 us); one group, which needs neither, two-atom 4^3 40 -> 35 us.
+constexpr int DEN_CLUSTER = 8;   // largest portable cluster
+
 struct Den64 {
   const int4 *units;   // element, (sub)cell, first plane, end plane
   const int64_t *qoff;
@@ -480,7 +497,8 @@ struct Den64 {
   const int64_t *toff;
   const double *psi, *C, *Ci, *f, *Rser;
   int64_t ldc;
-  int ncol, nfe;
+  int ncol, groups, nfe;
+  int halves, cs;   // halves of the groups (or 1: all together), CTAs in the cluster of one
   const uint8_t *eshift;
   PhaseTab ph;
   double *rho;
@@ -496,7 +514,7 @@ template <bool BLOCH, int KC>
 __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
   extern __shared__ __align__(16) double smd64[];
   const int4 u = P.units[blockIdx.x];
-  const int tid = threadIdx.x, e = u.x, k0 = blockIdx.y * KC;
+  const int tid = threadIdx.x, e = u.x;
   const int n = (int)(P.doff[e + 1] - P.doff[e]), nE = n - P.nfe;
   const int p = P.part_p[u.y], p2 = p * p, pq = P.part_q[u.y];
   const int64_t q0 = P.qoff[e], qs = q0 + pq;
@@ -508,93 +526,128 @@ __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
   double *L = Cs + (64 + nE) * KC;              // [axis][4][p]
   double *T1 = L + 12 * p, *T2 = T1 + 16 * p * KC;   // [bc][k][qx], [c][k][qx qy]
   double *ph8 = T2 + 4 * p2 * KC;               // [vertex][thread]
+  double *acc = ph8 + 8 * P64_NT;               // [point]: sum over this CTA's groups
   double *raw = P.nfe == 64 ? Cs : T1;          // serendipity coefficients before the lift
-  for (int o = tid; o < KC; o += P64_NT) {
-    const int k = k0 + o;
-    fs[o] = k < P.ncol ? P.f[BLOCH ? k >> 1 : k] : 0.0;
-  }
-  for (int o = tid; o < n * KC; o += P64_NT) {
-    const int j = o / KC, kk = o - j * KC, k = k0 + kk;
-    double c = 0.0;
-    if (k < P.ncol) {
-      const int64_t g = (int64_t)dl[j] * P.ldc;
-      if (!BLOCH) {
-        c = P.C[g + k];
-      } else {   // real (even k) or imaginary part of the phased coefficient
-        const double ar = P.C[g + (k >> 1)], ai = P.Ci[g + (k >> 1)];
-        const int s = es[j];
-        c = k & 1 ? P.ph.re[s] * ai + P.ph.im[s] * ar : P.ph.re[s] * ar - P.ph.im[s] * ai;
-      }
-    }
-    if (j < P.nfe)
-      raw[o] = c;
-    else
-      Cs[(64 + j - P.nfe) * KC + kk] = c;
-  }
   for (int o = tid; o < 3 * p; o += P64_NT) {
     const int d = o / p, t = o - d * p;
     double l[4], dl4[4];
     lagrange3(pt_axis_xi(P.xi, qs, p, d, t), l, dl4);
     for (int a = 0; a < 4; ++a) L[(d * 4 + a) * p + t] = l[a];
   }
-  __syncthreads();
-  if (P.nfe != 64) {   // the serendipity functions in the tricubic ones: their nodal values
-    for (int o = tid; o < 64 * KC; o += P64_NT) {
-      const int j = o / KC, kk = o - j * KC;
-      double s = 0.0;
-      for (int c = 0; c < 32; ++c) {
-        const double r = P.Rser[j * 32 + c];
-        if (r != 0.0) s = fma(r, raw[c * KC + kk], s);
+  const int first = u.z * p2, np = (u.w - u.z) * p2;   // the unit's points
+  // this CTA's groups: its share of all of them or of one half
+  const int half = blockIdx.y / P.cs, rank = blockIdx.y - half * P.cs;
+  const int cut = P.halves == 1 ? P.groups : (P.groups + 1) / 2;
+  const int h0 = half ? cut : 0, hn = half ? P.groups - cut : cut;
+  const int g0 = h0 + rank * hn / P.cs, g1 = h0 + (rank + 1) * hn / P.cs;
+  const bool direct = P.groups <= 2;   // one group to a CTA, which needs no sum
+  if (g0 == g1)
+    for (int q = tid; q < np; q += P64_NT) acc[q] = 0.0;
+  for (int grp = g0; grp < g1; ++grp) {
+    const int k0 = grp * KC;
+    __syncthreads();
+    for (int o = tid; o < KC; o += P64_NT) {
+      const int k = k0 + o;
+      fs[o] = k < P.ncol ? P.f[BLOCH ? k >> 1 : k] : 0.0;
+    }
+    for (int o = tid; o < n * KC; o += P64_NT) {
+      const int j = o / KC, kk = o - j * KC, k = k0 + kk;
+      double c = 0.0;
+      if (k < P.ncol) {
+        const int64_t g = (int64_t)dl[j] * P.ldc;
+        if (!BLOCH) {
+          c = P.C[g + k];
+        } else {   // real (even k) or imaginary part of the phased coefficient
+          const double ar = P.C[g + (k >> 1)], ai = P.Ci[g + (k >> 1)];
+          const int s = es[j];
+          c = k & 1 ? P.ph.re[s] * ai + P.ph.im[s] * ar : P.ph.re[s] * ar - P.ph.im[s] * ai;
+        }
       }
-      Cs[o] = s;
+      if (j < P.nfe)
+        raw[o] = c;
+      else
+        Cs[(64 + j - P.nfe) * KC + kk] = c;
     }
     __syncthreads();
-  }
-  for (int o = tid; o < 16 * p * KC; o += P64_NT) {   // x: (b c, k, qx)
-    const int r = o / p, qx = o - r * p, bc = r / KC, kk = r - bc * KC;
-    const double *c = Cs + 4 * bc * KC + kk;
-    T1[o] = fma(c[0], L[qx], fma(c[KC], L[p + qx], fma(c[2 * KC], L[2 * p + qx], c[3 * KC] * L[3 * p + qx])));
-  }
-  __syncthreads();
-  for (int o = tid; o < 4 * p2 * KC; o += P64_NT) {   // y: (c, k, qx qy)
-    const int r = o / p2, xy = o - r * p2, qy = xy / p, qx = xy - qy * p, c = r / KC, kk = r - c * KC;
-    const double *t = T1 + (4 * c * KC + kk) * p + qx, *l = L + 4 * p + qy;
-    const int st = KC * p;
-    T2[o] = fma(t[0], l[0], fma(t[st], l[p], fma(t[2 * st], l[2 * p], t[3 * st] * l[3 * p])));
-  }
-  __syncthreads();
-  double *ph = ph8 + tid;
-  for (int q = u.z * p2 + tid; q < u.w * p2; q += P64_NT) {
-    const int qz = q / p2, xy = q - qz * p2;
-    double a[KC];
-    {
-      const double l0 = L[8 * p + qz], l1 = L[9 * p + qz], l2 = L[10 * p + qz], l3 = L[11 * p + qz];
-#pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        const double *t = T2 + k * p2 + xy;
-        a[k] = fma(t[0], l0, fma(t[KC * p2], l1, fma(t[2 * KC * p2], l2, t[3 * KC * p2] * l3)));
+    if (P.nfe != 64) {   // the serendipity functions in the tricubic ones: their nodal values
+      for (int o = tid; o < 64 * KC; o += P64_NT) {
+        const int j = o / KC, kk = o - j * KC;
+        double s = 0.0;
+        for (int c = 0; c < 32; ++c) {
+          const double r = P.Rser[j * 32 + c];
+          if (r != 0.0) s = fma(r, raw[c * KC + kk], s);
+        }
+        Cs[o] = s;
       }
+      __syncthreads();
     }
-    if (nE > 0) {
-      const double *x = P.xi + 3 * (qs + q);
-      const double lx[2] = {0.125 * (1.0 - x[0]), 0.125 * (1.0 + x[0])},
-                   ly[2] = {1.0 - x[1], 1.0 + x[1]}, lz[2] = {1.0 - x[2], 1.0 + x[2]};
+    for (int o = tid; o < 16 * p * KC; o += P64_NT) {   // x: (b c, k, qx)
+      const int r = o / p, qx = o - r * p, bc = r / KC, kk = r - bc * KC;
+      const double *c = Cs + 4 * bc * KC + kk;
+      T1[o] = fma(c[0], L[qx], fma(c[KC], L[p + qx], fma(c[2 * KC], L[2 * p + qx], c[3 * KC] * L[3 * p + qx])));
+    }
+    __syncthreads();
+    for (int o = tid; o < 4 * p2 * KC; o += P64_NT) {   // y: (c, k, qx qy)
+      const int r = o / p2, xy = o - r * p2, qy = xy / p, qx = xy - qy * p, c = r / KC, kk = r - c * KC;
+      const double *t = T1 + (4 * c * KC + kk) * p + qx, *l = L + 4 * p + qy;
+      const int st = KC * p;
+      T2[o] = fma(t[0], l[0], fma(t[st], l[p], fma(t[2 * st], l[2 * p], t[3 * st] * l[3 * p])));
+    }
+    __syncthreads();
+    double *ph = ph8 + tid;
+    auto point = [&](int q) -> double {   // this group's part of the density at point q
+      const int qz = q / p2, xy = q - qz * p2;
+      double a[KC];
+      {
+        const double l0 = L[8 * p + qz], l1 = L[9 * p + qz], l2 = L[10 * p + qz], l3 = L[11 * p + qz];
 #pragma unroll
-      for (int v = 0; v < 8; ++v)
-        ph[v * P64_NT] = lx[v & 1] * ly[(v >> 1) & 1] * lz[v >> 2];
-      for (int j = 0; j < nE; ++j) {
-        const int code = ec[j];
-        const double b = ph[(code & 7) * P64_NT] * pe[(int64_t)(code >> 3) * 4 * Q + pq + q];
-        const double *c = Cs + (64 + j) * KC;
-#pragma unroll
-        for (int k = 0; k < KC; ++k) a[k] = fma(b, c[k], a[k]);
+        for (int k = 0; k < KC; ++k) {
+          const double *t = T2 + k * p2 + xy;
+          a[k] = fma(t[0], l0, fma(t[KC * p2], l1, fma(t[2 * KC * p2], l2, t[3 * KC * p2] * l3)));
+        }
       }
+      if (nE > 0) {
+        const double *x = P.xi + 3 * (qs + q);
+        const double lx[2] = {0.125 * (1.0 - x[0]), 0.125 * (1.0 + x[0])},
+                     ly[2] = {1.0 - x[1], 1.0 + x[1]}, lz[2] = {1.0 - x[2], 1.0 + x[2]};
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+          ph[v * P64_NT] = lx[v & 1] * ly[(v >> 1) & 1] * lz[v >> 2];
+        for (int j = 0; j < nE; ++j) {
+          const int code = ec[j];
+          const double b = ph[(code & 7) * P64_NT] * pe[(int64_t)(code >> 3) * 4 * Q + pq + q];
+          const double *c = Cs + (64 + j) * KC;
+#pragma unroll
+          for (int k = 0; k < KC; ++k) a[k] = fma(b, c[k], a[k]);
+        }
+      }
+      double r = 0.0;
+#pragma unroll
+      for (int k = 0; k < KC; ++k) r = fma(fs[k] * a[k], a[k], r);
+      return r;
+    };
+    // (a thread meets its own points again in the next group)
+    double *o = direct ? P.rho + qs + first : acc;
+    for (int q = tid; q < np; q += P64_NT) {
+      const double r = point(first + q);
+      if (direct && P.halves == 2)
+        atomicAdd(o + q, r);
+      else
+        o[q] = grp > g0 ? o[q] + r : r;
     }
+  }
+  if (direct) return;
+  const auto cluster = cooperative_groups::this_cluster();
+  if (P.cs > 1) cluster.sync();
+  for (int q = rank * P64_NT + tid; q < np; q += P.cs * P64_NT) {
     double r = 0.0;
-#pragma unroll
-    for (int k = 0; k < KC; ++k) r = fma(fs[k] * a[k], a[k], r);
-    atomicAdd(P.rho + qs + q, r);
+    for (int y = 0; y < P.cs; ++y) r += *cluster.map_shared_rank(acc + q, y);
+    if (P.halves == 2)
+      atomicAdd(P.rho + qs + first + q, r);
+    else
+      P.rho[qs + first + q] = r;
   }
+  if (P.cs > 1) cluster.sync();   // no CTA leaves while its part is read
 }
 
 }  // namespace
@@ -610,10 +663,10 @@ __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
 // direct form 1.0 ms).  Density: int4 units (element, (sub)cell, first z plane, end z plane),
 // cut to the mean cost of a CTA slot, and the doubles that one column takes at most.
 void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
-                     std::vector<int32_t> &den, int &den_col) {
+                     std::vector<int32_t> &den, int &den_col, int &den_pts) {
   adj.clear();
   den.clear();
-  adj_work = den_col = 0;
+  adj_work = den_col = den_pts = 0;
   const int64_t ne = (int64_t)ctx->n_e.size();
   struct Item {
     int32_t v[6];
@@ -714,6 +767,7 @@ void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, in
       den_col = std::max(den_col, den_column(ctx->n_e[e], p));
       const double fix = 64.0 * p + 16.0 * p * p, pl = plane(e, p);
       const int cuts = std::max(1, std::min(p, (int)std::min(64.0, std::ceil(p * pl / target))));
+      den_pts = std::max(den_pts, (p + cuts - 1) / cuts * p * p);
       for (int j = 0; j < cuts; ++j)
         L.push_back(Item{{(int32_t)e, cell, j * p / cuts, (j + 1) * p / cuts},
                          fix + pl * ((j + 1) * p / cuts - j * p / cuts)});
@@ -784,23 +838,40 @@ pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double 
   P.eshift = D.eshift;
   if (ph) P.ph = *ph;
   P.rho = rho;
-  PUFE_CUDA_TRY(cudaMemsetAsync(rho, 0, (size_t)ctx->nq * sizeof(double), st));
   // columns per CTA: the width (a multiple of 4, up to 16) that pads the fewest; less
   // where the work area of the largest (sub)cell does not fit an SM
   const int most = (P.ncol + 15) / 16;
   int kc = ((P.ncol + most - 1) / most + 3) & ~3;
-  auto bytes = [&] {
-    return (size_t)den_doubles(ctx->den64_column, ctx->max_part_p, kc) * sizeof(double);
+  auto bytes = [&] {   // (the sums of a unit's points from three groups on)
+    const int sums = P.ncol > 2 * kc ? ctx->den64_points : 0;
+    return (size_t)(den_doubles(ctx->den64_column, ctx->max_part_p, kc) + sums) * sizeof(double);
   };
   while (kc > 4 && bytes() > 227 * 1024) kc -= 4;
-  const int groups = (P.ncol + kc - 1) / kc;
+  const int groups = P.groups = (P.ncol + kc - 1) / kc;
+  P.cs = 1;
+  P.halves = std::min(groups, 2);
+  if (groups > 2 && (int64_t)ctx->n_dunits * groups <= 4 * ctx->nsm) {
+    P.halves = groups > 5 ? 2 : 1;
+    P.cs = std::min(DEN_CLUSTER, (groups + P.halves - 1) / P.halves);
+  }
+  const int ny = P.halves * P.cs;
   const size_t sm = bytes();
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e too large for the density kernel");
+  if (P.halves == 2) PUFE_CUDA_TRY(cudaMemsetAsync(rho, 0, (size_t)ctx->nq * sizeof(double), st));
   auto run = [&](auto kern) -> pufe_status {
     PUFE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const dim3 grid((unsigned)ctx->n_dunits, (unsigned)groups);
-    kern<<<grid, P64_NT, sm, st>>>(P);
-    PUFE_CUDA_TRY(cudaGetLastError());
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = at[0].val.clusterDim.z = 1;
+    at[0].val.clusterDim.y = (unsigned)P.cs;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctx->n_dunits, (unsigned)ny);
+    cfg.blockDim = dim3(P64_NT);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = P.cs > 1 ? 1 : 0;
+    PUFE_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, P));
     return PUFE_OK;
   };
   if (ph) {

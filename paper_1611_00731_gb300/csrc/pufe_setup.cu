@@ -1596,8 +1596,10 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
           v > 0)
         nsm = v;
     }
+    ctx->nsm = nsm;
     sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
-    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits, ctx->den64_column);
+    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits, ctx->den64_column,
+                    ctx->den64_points);
   }
   // tabulation: runs of slots with one atom and cutoff, in chunks of points
   std::vector<int32_t> kitems;
