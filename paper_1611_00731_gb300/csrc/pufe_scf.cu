@@ -32,6 +32,7 @@ struct ScfState {
   int n1[3] = {0, 0, 0};
   double *X[3] = {nullptr, nullptr, nullptr};     // n1 x n1, row-major X[node][mode]
   double *lam[3] = {nullptr, nullptr, nullptr};   // n1, ascending
+  bool b_dirty = false;     // a solve that failed left the load vector b as it was
   double *b = nullptr, *t0 = nullptr, *t1 = nullptr;   // n_fe each
   double *n_out = nullptr;  // n_q: output density of a step
   double *sums = nullptr;   // SCF_SUMS x SCF_SLOTS partial sums of the energies
@@ -638,13 +639,16 @@ pufe_status scf_prepare(pufe_ctx *ctx) {
   }
   const size_t nfe = (size_t)ctx->n_fe * sizeof(double), nq = (size_t)ctx->nq * sizeof(double);
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->b, nfe));
-  PUFE_CUDA_TRY(cudaMemset(S->b, 0, nfe));   // every solve leaves it zero again
+  PUFE_CUDA_TRY(cudaMemset(S->b, 0, nfe));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->t0, nfe));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->t1, nfe));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->n_out, nq));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->sums, SCF_SUMS * SCF_SLOTS * sizeof(double)));
   PUFE_CUDA_TRY(cudaMallocHost((void **)&S->h_sums, SCF_SUMS * SCF_SLOTS * sizeof(double)));
   PUFE_CUDA_TRY(cudaMalloc((void **)&S->f, 64 * 64 * sizeof(double)));
+  // the copies and the clearing above are done before a solve on a caller's stream,
+  // which need not wait for the default one
+  PUFE_CUDA_TRY(cudaStreamSynchronize(0));
   return PUFE_OK;
 }
 
@@ -708,6 +712,10 @@ static pufe_status coulomb(pufe_ctx *ctx, const double *rho_I, const InterpOut &
   auto lines = [&](int n) { return (unsigned)((nfe / n + nb - 1) / nb); };
   PUFE_CUDA_TRY(cudaFuncSetAttribute(k_axis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ax));
   PUFE_CUDA_TRY(cudaFuncSetAttribute(k_axis_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ax));
+  // the load vector is zero here unless a launch of an earlier solve failed between
+  // the kernel that adds into it and the one that clears it
+  if (S->b_dirty) PUFE_CUDA_TRY(cudaMemsetAsync(S->b, 0, nfe * sizeof(double), st));
+  S->b_dirty = true;
   // -K v = 4 pi int phi (rho_I - n)  <=>  K v = 4 pi int phi (n - rho_I)
   k_fe_load<<<(unsigned)ctx->nelem, SCF_NT, sm_load, st>>>(
       D.qoff, D.w, D.xi, D.partoff, D.part_p, D.part_q, D.doff, D.dofs, O.n, rho_I, 4.0 * PI, pm,
@@ -716,6 +724,8 @@ static pufe_status coulomb(pufe_ctx *ctx, const double *rho_I, const InterpOut &
                                                     nullptr);
   k_axis<<<lines(n1), AX_NT, sm_ax, st>>>(n0, n1, n2, 1, nb, staged, S->X[1], true, S->t0, S->t1,
                                                     S->b);
+  PUFE_CUDA_TRY(cudaGetLastError());
+  S->b_dirty = false;
   k_axis_z<<<lines(n2), AX_NT, sm_ax, st>>>(n0, n1, n2, nb, staged, S->X[2], S->lam[0], S->lam[1],
                                                       S->lam[2], S->t1, S->t0);
   k_axis<<<lines(n1), AX_NT, sm_ax, st>>>(n0, n1, n2, 1, nb, staged, S->X[1], false, S->t0, S->t1,
