@@ -5,6 +5,9 @@
 // The element basis (the FE columns -- 64 tricubic or 32 cubic serendipity
 // functions -- then phi_v^PU Psi_alpha columns) is rebuilt on chip from the reference coordinates of each quadrature point
 // and the tabulated Psi / grad Psi; it is never stored in HBM.
+//
+// The contraction here is the direct one, for rules of fewer than 4 points per axis; the
+// others, the density and the adjoint are sum factorized (pufe_sf64.cu, pufe_pt64.cu).
 #include <math.h>
 
 #include "pufe_internal.h"

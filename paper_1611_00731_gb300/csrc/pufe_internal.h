@@ -99,13 +99,14 @@ struct DeviceArrays {
   int32_t *smap = nullptr;    // CSR slot of each local pair (i, j), row-major
   // work list: elements sorted by (n_e, Q_e) class, largest first
   int32_t *order = nullptr;   // nelem
-  // FP64 assembly/adjoint work list, 3 per item (element, first point, end
-  // point), largest first; null when every item is a whole element
+  // work list of the direct FP64 assembly (rules of fewer than 4 points per axis), 3
+  // per item (element, first point, end point), largest first; null when every item
+  // is a whole element
   int32_t *wsplit = nullptr;
   // sum-factorized FP64 assembly: (element, kind, begin, end, (sub)cell range) items
   int32_t *aitems = nullptr;
-  // FP64 adjoint: (element, kind, begin, end, (sub)cell range) items; FP64 density: (element,
-  // (sub)cell, first plane, end plane) units; nodal values of the serendipity
+  // FP64 adjoint: (element, kind, begin, end, (sub)cell or row range) items; FP64 density:
+  // (element, (sub)cell, first plane, end plane) units; nodal values of the serendipity
   // functions at the tricubic nodes (64 x 32, serendipity space only)
   int32_t *jitems = nullptr, *dunits = nullptr;
   double *Rser = nullptr;
@@ -126,8 +127,9 @@ struct DeviceArrays {
   int32_t *tblk = nullptr;     // nelem + 1: FP32 tabulation CTAs per element, prefix summed
   int8_t *eeform = nullptr;   // per element: E x E form of the strip (0 model, 1 pair, 2 direct)
   unsigned *err = nullptr;    // device error flag
-  // side stream and events: the FE-FE kernel of the mixed assembly runs on
-  // `side`, forked from and joined back into the caller's stream
+  // side stream and events: the E-E kernels of S of the mixed assembly run on `side`
+  // (the copy of S0 or the FE-FE kernel before them), forked from and joined back into
+  // the caller's stream
   cudaStream_t side = nullptr;
   ProjDev *proj = nullptr;     // 64 projector descriptions (allocated on first use)
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -159,11 +161,11 @@ struct pufe_ctx {
   bool fe_exact = false;      // every rule has >= 4 points per axis per (sub)cell
   int n_big = 0;              // elements with n_e > 128 (listed first in `order`)
   int64_t big_pad_end = 0;    // end of the last n_e > 128 element's padded points (0: none)
-  int64_t n_wsplit = 0;       // items of the FP64 point-range work list (0: none)
+  int64_t n_wsplit = 0;       // items of the direct FP64 assembly's point-range list (0: none)
   int nsm = 152;              // SMs of the device (of a GB300 without one)
   int n_aitems = 0;           // items of the sum-factorized FP64 assembly (0: direct form)
   int asm64_work = 0;         // doubles of its shared work area
-  int n_jitems = 0, adj64_work = 0;   // the same of the FP64 adjoint (0: direct form)
+  int n_jitems = 0, adj64_work = 0;   // items and shared doubles of the FP64 adjoint
   int rser_len = 0;           // entries per serendipity function in rser_i, rser_v
   int n_kitems = 0;           // items of the tabulation
   int n_dunits = 0;           // units of the FP64 density
@@ -492,14 +494,14 @@ pufe_status launch_assemble_fp64(pufe_ctx *ctx, const PhaseTab *ph, const double
 // its sum-factorized form, and the work list of that form
 pufe_status launch_assemble_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *V, int what,
                                  double *H, double *Hi, double *S, double *Si, cudaStream_t s);
-void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, int &work);
+void sf64_work_list(const pufe_ctx *ctx, std::vector<int32_t> &items, int &work);
 // FP64 adjoint and density by sum factorization, and their work lists
 pufe_status launch_adjoint_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *Hr,
                                 const double *Hi, double *Vbar, cudaStream_t s);
 pufe_status launch_density_sf64(pufe_ctx *ctx, const PhaseTab *ph, const double *C,
                                 const double *Ci, int64_t ldc, const double *f, int nocc,
                                 double *rho, cudaStream_t s);
-void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
+void pt64_work_lists(const pufe_ctx *ctx, std::vector<int32_t> &adj, int &adj_work,
                      std::vector<int32_t> &den, int &den_col, int &den_pts);
 pufe_status launch_density_fp64_bloch(pufe_ctx *ctx, const PhaseTab &ph, const double *Cr,
                                       const double *Ci, int64_t ldc, const double *f, int nocc,

@@ -281,7 +281,7 @@ pufe_status launch_projections(pufe_ctx *ctx, const ProjDev *pj, int P, const do
   const int amax = std::max(1, ctx->max_alpha), pm = ctx->max_part_p;
   A.pc = std::min(8, P);
   while (A.pc > 1 && (proj_doubles(nc * A.pc, A.pc, 1, amax, pm, nc) > PJ_WORK ||
-                      ctx->nelem * ((P + A.pc - 1) / A.pc) < 304))
+                      ctx->nelem * ((P + A.pc - 1) / A.pc) < 2 * ctx->nsm))
     A.pc = (A.pc + 1) / 2;
   A.sc = 1;
   while (A.sc < amax && proj_doubles(nc * A.pc, A.pc, A.sc + 1, amax, pm, nc) <= PJ_WORK) ++A.sc;

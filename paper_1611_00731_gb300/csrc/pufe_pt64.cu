@@ -20,14 +20,14 @@
 //    27 p + 9 p^2 + 3 p^3, times Psi_a Psi_b; or the direct products of the
 //    columns where the slots hold few vertices.
 // 97,000 operations for an element of 104 functions and 6^3 points against the
-// 2,360,000 of the direct form (k_adjoint_fp64).  The parts add into Vbar (zeroed
+// 2,360,000 of contracting the element's whole block at every point.  The parts add into Vbar (zeroed
 // first) with one atomic per point, so that an element's parts can run on
 // different SMs.
 //
 // Density, n_q = sum_k f_k (sum_j B_qj C_jk)^2: the 64 tricubic functions by
 // sum factorization per state (64 p + 16 p^2 + 4 p^3 against 64 p^3), the
-// enrichment columns directly, each point's b_r formed once for the states that
-// its thread carries.
+// enrichment columns directly, each point's b_r formed once for the group of up to 16
+// columns that its thread carries.
 //
 // Measured, direct kernels before: adjoint 12^3 rocksalt 9.34 -> 0.35 ms, CsCl-like
 // 16^3 19.4 -> 0.60 ms, two-atom 4^3 1.06 -> 0.031 ms; density 0.80 -> 0.23 ms (8
@@ -661,9 +661,11 @@ __global__ void __launch_bounds__(P64_NT) k_density_sf64(Den64 P) {
 // one row of the triangle and its columns' points are beyond half an SM's shared
 // memory (over 907 columns; eight such elements of 912 columns 5.5 ms, of 800 in the
 // direct form 1.0 ms).  Density: int4 units (element, (sub)cell, first z plane, end z plane),
-// cut to the mean cost of a CTA slot, and the doubles that one column takes at most.
-void pt64_work_lists(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &adj, int &adj_work,
+// cut to the mean cost of a CTA slot; the doubles that one column takes and the points
+// that one unit has at most.
+void pt64_work_lists(const pufe_ctx *ctx, std::vector<int32_t> &adj, int &adj_work,
                      std::vector<int32_t> &den, int &den_col, int &den_pts) {
+  const int nsm = ctx->nsm;
   adj.clear();
   den.clear();
   adj_work = den_col = den_pts = 0;

@@ -1257,24 +1257,21 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   } else {
     PUFE_CUDA_TRY(cudaGetDevice(&ctx->device));
     ctx->on_device = true;
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
+        v > 0)
+      ctx->nsm = v;
   }
-  // ---- FP64 work list ---------------------------------------------------------
-  // The FP64 assembly and adjoint take one CTA per work item.  An element
+  const int nsm = ctx->nsm;
+  // ---- work list of the direct FP64 assembly -----------------------------------
+  // (rules of fewer than 4 points per axis only.)  One CTA per work item.  An element
   // whose cost Q_e * npad_e^2 exceeds the mean cost of a CTA slot (two per
-  // SM) is cut into point ranges: multiples of 8 points (the kernels' chunk),
+  // SM) is cut into point ranges: multiples of 8 points (the kernel's chunk),
   // at least 64 points each.  The ranges' partial element matrices meet in
-  // the atomic scatter; the adjoint's ranges write disjoint points.  Items
-  // run largest first.  No list (one CTA per element, in `order`) when no
-  // element is cut.
+  // the atomic scatter.  Items run largest first.  No list (one CTA per element, in
+  // `order`) when no element is cut.
   std::vector<int32_t> wsplit;
-  {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
+  if (!fe_exact) {
     auto cost = [&](int64_t e, int64_t npts) {
       const int64_t np = (n_e[e] + 3) & ~3;
       return (double)npts * (double)(np * np);
@@ -1328,13 +1325,6 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   // adjoint of these elements takes the same ranges (disjoint points).
   std::vector<int32_t> titems;
   {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
     struct TItem {
       int32_t k, c0, c1;
       int64_t c;
@@ -1383,13 +1373,6 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   // share an SM); the ranges' entries are disjoint, so no order is implied.
   std::vector<int32_t> sitems;
   {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
     struct SItem {
       int32_t k, pb, pe;
       int64_t c;
@@ -1467,13 +1450,6 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   // ranges of its (sub)cells; the ranges' partial blocks meet in the atomics.
   std::vector<int32_t> citems;
   {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
     struct CItem {
       int32_t k, c0, c1;
       int64_t c;
@@ -1528,13 +1504,6 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   // quarter of the mean per SM.  Each point is written by one range only.
   std::vector<int32_t> pitems;
   {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
     struct PItem {
       int32_t k, qa, qb;
       int64_t c;
@@ -1589,16 +1558,8 @@ static pufe_status build(const pufe_cell *cell, const pufe_species *species, int
   ctx->q_e = q_e;
   std::vector<int32_t> aitems, jitems, dunits;
   {
-    int nsm = 152;
-    if (ctx->on_device) {
-      int v = 0;
-      if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, ctx->device) == cudaSuccess &&
-          v > 0)
-        nsm = v;
-    }
-    ctx->nsm = nsm;
-    sf64_work_list(ctx, nsm, aitems, ctx->asm64_work);
-    pt64_work_lists(ctx, nsm, jitems, ctx->adj64_work, dunits, ctx->den64_column,
+    sf64_work_list(ctx, aitems, ctx->asm64_work);
+    pt64_work_lists(ctx, jitems, ctx->adj64_work, dunits, ctx->den64_column,
                     ctx->den64_points);
   }
   // tabulation: runs of slots with one atom and cutoff, in chunks of points

@@ -965,7 +965,8 @@ static double ee_pair_ops(const std::vector<int32_t> &cells) {
 // fewer operations: slots of one vertex column each (64 + 30 functions, 30 slots,
 // 4,096 points: 12 M direct against 88 M) fall on the direct side, slots of eight
 // (64 + 40, 5 slots, 216 points: 1.06 M against 0.18 M) on the other.
-void sf64_work_list(const pufe_ctx *ctx, int nsm, std::vector<int32_t> &items, int &work) {
+void sf64_work_list(const pufe_ctx *ctx, std::vector<int32_t> &items, int &work) {
+  const int nsm = ctx->nsm;
   items.clear();
   work = 0;
   if (!ctx->fe_exact || ctx->max_part_p > 16) return;

@@ -1526,10 +1526,9 @@ static pufe_status run_assemble_tc(pufe_ctx *ctx, const double *V, int what, dou
   const int nsmall = (int)ctx->nelem - nbig;
   if (nbig > 0 && sm256 > 227 * 1024)
     return fail(PUFE_EINVAL, "too many enrichments per element for TF32X3");
-  // H = 0 and S = the constant FE-FE overlap; then the strip kernels on the
-  // caller's stream and, on the context's side stream, the FE-FE kernel (V
-  // term and kinetic constants of H) and the E-E kernel of S, concurrently
-  // (all of them only add into H and S)
+  // H = 0 and S = the constant FE-FE overlap; then the FE-FE kernel (V term and kinetic
+  // constants of H), the tile and the strip, and the E-E kernels of S, on the caller's and
+  // the context's side stream in the orders below (all of them only add into H and S)
   if (ctx->max_part_p > 16) return fail(PUFE_EINVAL, "rule with more than 16 points per axis");
   const bool prof = ctx->prof;
   auto mark = [&](int i, cudaStream_t s) -> pufe_status {
@@ -1592,11 +1591,11 @@ static pufe_status run_assemble_tc(pufe_ctx *ctx, const double *V, int what, dou
   if (e1 != PUFE_OK) return e1;
   if (pufe_status e = mark(9, st)) return e;
   if (prof) ctx->prof_ran[4] = nsmall > 0;
-  // the E-E kernels of S on the side stream; the FE-FE kernel after the strip
-  // on the caller's stream when no tensor-core tile runs there, else on the
-  // side stream before the E-E kernels (measured: 12^3 rocksalt step 0.559 ->
-  // 0.543 ms with it on the caller's stream; the CsCl-like cell, whose
-  // caller's stream also carries the tensor-core tile, 1.71 -> 1.76 ms)
+  // the E-E kernels of S on the side stream; the FE-FE kernel (unless it ran early: a
+  // call for H alone, or a mesh with tensor-core tiles) after the strip on the caller's
+  // stream when no tile runs there, else on the side stream before the E-E kernels (measured:
+  // 12^3 rocksalt step 0.559 -> 0.543 ms with it on the caller's stream; the CsCl-like
+  // cell, whose caller's stream also carries the tile, 1.71 -> 1.76 ms)
   if (!early) PUFE_CUDA_TRY(cudaStreamWaitEvent(D.side, D.ev_fork, 0));
   if ((what & PUFE_WANT_H) && !early)
     if (pufe_status e = fefe(nbig > 0 ? D.side : st)) return e;
