@@ -46,9 +46,9 @@ __device__ __forceinline__ void lag3(float t, float L[4]) {
 // 128-thread CTAs per SM), one output per loop turn (three instructions per
 // multiply-add) and the widening of each entry on the FP64 pipe (two per clock and SM).
 // Now a thread owns a line of each stage with five or ten outputs, shared memory
-// follows the largest rule (12 KB at 8 points: 40 registers bind, 12 CTAs per SM) and
+// follows the largest rule (15 KB at 10 points: 48 registers bind, 10 CTAs per SM) and
 // entries are widened on the integer pipe; what is left is the 7 M atomics.
-// 12^3 rocksalt (ncu) 59 -> 34 us; at a wavevector, where elements away from the upper
+// 12^3 rocksalt (ncu) 59 -> 33 us; at a wavevector, where elements away from the upper
 // faces skip phases that are 1, 64-atom cell 2.41 -> 1.26 ms.
 template <bool BLOCH>
 __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
@@ -149,9 +149,25 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
   const int n = (int)(doff[e + 1] - doff[e]);
   const int32_t *m = smap + soff[e];
   const int j = tid & 63, ih = tid >> 6;
-  // most elements touch no upper face of the cell: every phase is 1
+  // most elements touch no upper face of the cell: every phase is 1.  The others read
+  // the phase of a pair of shift codes, and what it adds to S, from a table (P and G2
+  // are done with): formed per entry its FP64 operations bound meshes of a few hundred
+  // elements, many of them at a face (7^3 rocksalt 48 us when every entry of every element
+  // had them, 57 us for the faces alone with the tests on top, 44 us from the table).
   const uint8_t *es = BLOCH ? eshift + doff[e] : nullptr;
   const bool phased = BLOCH && __syncthreads_or(tid < 64 ? es[tid] : 0) != 0;
+  double *tab = reinterpret_cast<double *>(sm_ff);   // [re, im, re - 1][ci][cj]
+  if (phased) {
+    if (tid < 64) {
+      const int ci = tid >> 3, cj = tid & 7;
+      const double pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
+      tab[tid] = pr;
+      tab[64 + tid] = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
+      tab[128 + tid] = pr - 1.0;
+    }
+    __syncthreads();
+  }
+  const int cj = phased ? es[j] : 0;
   int pa[2], pb[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -172,12 +188,8 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
         // S starts as the summed constants, so only pairs whose phase is not 1 (the
         // elements on the cell's upper faces) correct it; a zero imaginary part is
         // not added (unless the value is not finite)
-        const int ci = phased ? es[i] : 0, cj = phased ? es[j] : 0;
-        double pr = 1.0, pi = 0.0;
-        if (ci != cj) {
-          pr = ph.re[ci] * ph.re[cj] + ph.im[ci] * ph.im[cj];
-          pi = ph.re[ci] * ph.im[cj] - ph.im[ci] * ph.re[cj];
-        }
+        const int ci = phased ? es[i] : 0, cc = 8 * ci + cj;
+        const double pr = ci != cj ? tab[cc] : 1.0, pi = ci != cj ? tab[64 + cc] : 0.0;
         if (what & PUFE_WANT_H) {
           const double hv = __ldg(Tfe + o) + v;
           atomicAdd(H + slot, ci != cj ? hv * pr : hv);
@@ -185,7 +197,7 @@ __global__ void __launch_bounds__(SF_NT) k_fefe_sumfac(
         }
         if ((what & PUFE_WANT_S) && ci != cj) {
           const double sv = __ldg(Sfe + o);
-          atomicAdd(S + slot, sv * (pr - 1.0));
+          atomicAdd(S + slot, sv * tab[128 + cc]);
           atomicAdd(Si + slot, sv * pi);
         }
       }
