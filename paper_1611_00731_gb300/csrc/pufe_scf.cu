@@ -293,9 +293,12 @@ __global__ void __launch_bounds__(SCF_NT) k_fe_load(
 // multiply-adds per node bind it (2.7 us for 36^3 nodes) as long as nothing waits:
 // M is staged in shared memory by one round of independent loads (reading it from
 // L2 inside the sums, a few values ahead, took 13-25 us), and a sum runs in four
-// chains.  M too large for the stage (over 112 nodes per axis) is read in place.
+// chains.  M of more than AX_STAGE nodes per axis is read in place: its stage leaves two
+// CTAs per SM, then one (whole potential at 96 nodes per axis 1,556 us staged, 1,582 us in
+// place; at 102 2,085 and 1,838 us, at 111 2,724 and 2,483 us).
 // `clear` (may be null): an array of the same size set to zero.
 constexpr int AX_NT = 256;
+constexpr int AX_STAGE = 96;
 
 __device__ __forceinline__ int64_t line_base(int n0, int n1, int axis, int64_t line) {
   if (axis == 0) return line * n0;
@@ -705,7 +708,7 @@ static pufe_status coulomb(pufe_ctx *ctx, const double *rho_I, const InterpOut &
   int nb = 8;   // lines per CTA: what two copies of the longest axis' lines leave
   const int nmax = std::max(n0, std::max(n1, n2));
   while (nb > 1 && (size_t)2 * nmax * nb * sizeof(double) > 96 * 1024) nb /= 2;
-  const bool staged = nmax <= 112;   // the matrix beside the lines
+  const bool staged = nmax <= AX_STAGE;   // the matrix beside the lines
   const size_t sm_ax = ((size_t)2 * nmax * nb + (staged ? (size_t)nmax * nmax : 0)) * sizeof(double);
   if (sm_ax > 227 * 1024)
     return fail(PUFE_EINVAL, "more nodes per axis than the Poisson solve takes");
