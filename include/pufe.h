@@ -231,7 +231,9 @@ pufe_status pufe_assemble_HS_static(pufe_ctx *ctx, const double *V, int what, do
  * quadrature point.  C: device float64, N x nocc, row-major with leading
  * dimension ldc >= nocc (C[j * ldc + k]); f: device float64 (nocc);
  * rho: device float64 (n_q), overwritten.  1 <= nocc <= 64.  PUFE_TF32X3
- * evaluates in FP32 on the CUDA cores.  Asynchronous. */
+ * evaluates in FP32 on the CUDA cores.  The values repeat bit for bit from call
+ * to call (those of the assembly and the adjoint up to the order in which FP64
+ * atomics land).  Asynchronous. */
 pufe_status pufe_density(pufe_ctx *ctx, const double *C, int64_t ldc,
                          const double *f, int nocc, int prec, double *rho,
                          void *stream);

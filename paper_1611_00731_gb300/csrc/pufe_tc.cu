@@ -1019,8 +1019,11 @@ __global__ void __launch_bounds__(DEN_NT, NARROW ? 8 : 4) k_density_f32(
 // points with the element's coefficients, both in shared memory: a thread owns 8
 // points x 8 columns, so four 16-byte reads feed 64 multiply-adds, where
 // k_density_f32 (one point and 8 columns per thread) reads two for 8 and is bound
-// by that (shared-memory wavefronts 88 % of their peak, FMA pipe 20 %); a basis
-// value is formed once per point instead of once per 8 columns.  The columns'
+// by that (64-atom cell on 16^3 elements, ncu: shared-memory wavefronts 75 % of their
+// peak, FMA pipe 21 %, 1.71 ms; here 42 %, 40 %, 0.95 ms); a basis
+// value is formed once per point instead of once per 8 columns.  Barriers between
+// gather, basis, product and reduction are what holds it (32^3 elements: 6.36 ms, 31 %
+// of the FP32 rate).  The columns'
 // sums run over the basis in the same order as there, and one thread per point
 // then adds the columns' f psi^2 in that kernel's order, so the values are the
 // same bit for bit.  16 x CG threads (CG = columns / 8); two CTAs share an SM.
