@@ -494,6 +494,7 @@ pufe_status launch_density_fp64(pufe_ctx *ctx, const double *C, int64_t ldc, con
                                 int nocc, double *rho, cudaStream_t st) {
   auto &D = ctx->d;
   const int noccp = (nocc + 7) & ~7;
+  // (the call's limit of basis x states; the kernel's own need is less)
   const size_t sm = ((size_t)ctx->max_basis * noccp + noccp) * sizeof(double);
   if (sm > 227 * 1024) return fail(PUFE_EINVAL, "n_e * nocc too large for the density kernel");
   return launch_density_sf64(ctx, nullptr, C, nullptr, ldc, f, nocc, rho, st);
